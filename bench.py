@@ -291,7 +291,7 @@ def knn_kernel_name(t):
         return "knn32_kernel"
     if buf:
         return "knn_kernel (single scan)"
-    return "knn_wq_kernel (one warp per query)" if qpw == 4 else "knn_cg_kernel (grouped queries)"
+    return "knn_gq_kernel (four queries per warp)"
 
 
 def stage(st):

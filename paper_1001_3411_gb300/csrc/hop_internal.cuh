@@ -61,6 +61,7 @@ enum Slot {
     S_HALO,                             // halo statistics scratch
     S_SUB,                              // subhalos: dense chain ids, per-particle chain ids
     S_SUB_C,                            // subhalos: arrays over chains and boundaries
+    S_KNN_HAND,                         // queries that the grouped kNN hands over
     S_COUNT
 };
 
@@ -406,8 +407,13 @@ struct KnnArgs {
 };
 int knn_launch(hop_ctx *c, const KnnArgs &a, bool f64, int qpw, int cpr);
 int knn32_launch(hop_ctx *c, const KnnArgs &a, int cpr);   // knn32.cu: one query per lane, float32
-// knn_cg.cu: count-then-gather, float32, 4, 8 or 16 queries per warp
-int knn_cg_launch(hop_ctx *c, const KnnArgs &a, int qpw, int cpr);
+// knn_gq.cu: float32, radius chunks of 4, 8 or 16 queries; four queries per
+// warp, the ones it does not take handed over to knn_wq_launch
+int knn_gq_launch(hop_ctx *c, const KnnArgs &a, int qpw, int cpr);
+// knn_cg.cu: one warp per query, over a list of *hand_n sorted indices;
+// `counter` is a device word that is zero on entry
+int knn_wq_launch(hop_ctx *c, const KnnArgs &a, int qpw, int cpr, const uint32_t *hand,
+                  const unsigned long long *hand_n, unsigned long long *counter);
 
 // link.cu
 int make_dkey(hop_ctx *c, const float *dens, const uint32_t *orig, int64_t n, uint64_t *dkey);
