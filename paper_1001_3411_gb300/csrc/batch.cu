@@ -146,7 +146,7 @@ constexpr int kBoruvkaBodyKernels = 6;   // fill, best edge, target, hook, compr
 // Host-side description of one batched pass.
 struct BatchPlan {
     int B = 0;
-    int64_t n = 0, n_chunks = 0, n_cells = 0;
+    int64_t n = 0, n_chunks = 0, n_units = 0, n_cells = 0;
     std::vector<SegDesc> seg;
 };
 
@@ -158,7 +158,7 @@ int make_plan(hop_ctx *c, const int64_t *offsets, const double *boxes, int B, co
     if (offsets[0] != 0) return ctx_fail(c, HOP_EINVAL, "offsets[0] must be 0");
     pl->B = B;
     pl->seg.resize(B);
-    int64_t chunks = 0, cells = 0;
+    int64_t chunks = 0, units = 0, cells = 0;
     for (int b = 0; b < B; ++b) {
         const int64_t nb = offsets[b + 1] - offsets[b];
         if (nb < p->n_dens) return ctx_fail(c, HOP_EINVAL, "every subvolume needs at least n_dens particles");
@@ -168,17 +168,20 @@ int make_plan(hop_ctx *c, const int64_t *offsets, const double *boxes, int B, co
         d.base = offsets[b];
         d.n = nb;
         d.chunk0 = chunks;
+        d.unit0 = units;
         d.cell0 = cells;
         d.box = box;
         d.norm = box * box * box / ((double)nb * 3.14159265358979323846);
         d.plain_r = plain_radius_for(nb, box, p->n_dens);
         d.level_dense = dense_level_for(nb);
         chunks += (nb + qpw - 1) / qpw;
+        units += (nb + 15) / 16;
         cells += (int64_t(1) << (3 * d.level_dense)) + 1;
     }
     pl->n = offsets[B];
     if (pl->n >= (int64_t(1) << 31) - 1) return ctx_fail(c, HOP_EINVAL, "total particles must be < 2^31 - 1");
     pl->n_chunks = chunks;
+    pl->n_units = units;
     pl->n_cells = cells;
     return HOP_OK;
 }
@@ -258,6 +261,7 @@ int enqueue_pass(hop_ctx *c, const BatchPlan &pl, const SegDesc *seg, const Pass
     a.seg = seg;
     a.B = pl.B;
     a.n_chunks = pl.n_chunks;
+    a.n_units = pl.n_units;
     if (pl.B == 1) {
         // one subvolume: the kernel without per-chunk descriptors, with the
         // same box, table, radius and normalisation as kernel arguments

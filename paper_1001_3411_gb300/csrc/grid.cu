@@ -70,12 +70,16 @@ __global__ void keys_seg_kernel(const T *__restrict__ pos, int64_t n, const SegD
 }
 
 // Sorted float4 records; with kout set, also the sorted keys without the
-// subvolume field (the Morton key within the particle's own box).
+// subvolume field (the Morton key within the particle's own box).  The
+// kSposPad records from n on are NaN (no distance test accepts them), so that
+// particles can be read in runs of eight without a bound.
 template <typename T>
 __global__ void gather_kernel(const T *__restrict__ pos, const uint32_t *__restrict__ perm,
                               int64_t n, typename V4<T>::type *__restrict__ spos,
                               const uint64_t *__restrict__ kin, uint64_t *__restrict__ kout)
 {
+    if (blockIdx.x == 0 && threadIdx.x < kSposPad)
+        spos[n + threadIdx.x] = make_rec((T)NAN, (T)NAN, (T)NAN, 0u);
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
          s += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t p = perm[s];
@@ -202,7 +206,7 @@ int grid_build_t(hop_ctx *c, const T *pos, int64_t n, double box, void **spos_ou
     uint32_t *v0 = (uint32_t *)ctx_buf(c, S_VAL0, n * sizeof(uint32_t));
     uint32_t *v1 = (uint32_t *)ctx_buf(c, S_VAL1, n * sizeof(uint32_t));
     void *tmp = ctx_buf(c, S_SORT_TMP, radix_sort_scratch_bytes(n));
-    auto *spos = (typename V4<T>::type *)ctx_buf(c, S_SPOS, n * sizeof(typename V4<T>::type));
+    auto *spos = (typename V4<T>::type *)ctx_buf(c, S_SPOS, (n + kSposPad) * sizeof(typename V4<T>::type));
     const int Ld = dense_level_for(n);
     const int64_t ncell = int64_t(1) << (3 * Ld);
     uint32_t *cellT = (uint32_t *)ctx_buf(c, S_CELLT, (ncell + 1) * sizeof(uint32_t));
@@ -288,7 +292,7 @@ int grid_build_seg(hop_ctx *c, const float *pos, int64_t n, const SegDesc *seg, 
     uint32_t *v0 = (uint32_t *)ctx_buf(c, S_VAL0, n * sizeof(uint32_t));
     uint32_t *v1 = (uint32_t *)ctx_buf(c, S_VAL1, n * sizeof(uint32_t));
     void *tmp = ctx_buf(c, S_SORT_TMP, radix_sort_scratch_bytes(n));
-    float4 *spos = (float4 *)ctx_buf(c, S_SPOS, n * sizeof(float4));
+    float4 *spos = (float4 *)ctx_buf(c, S_SPOS, (n + kSposPad) * sizeof(float4));
     uint32_t *cellT = (uint32_t *)ctx_buf(c, S_CELLT, n_cells * sizeof(uint32_t));
     if (!k0 || !k1 || !v0 || !v1 || !tmp || !spos || !cellT) return HOP_ENOMEM;
     int blocks = (int)std::min<int64_t>((n + 255) / 256, (int64_t)c->num_sms * 32);

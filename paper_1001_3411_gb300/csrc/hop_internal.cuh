@@ -19,6 +19,8 @@ constexpr int kMaxLevel = 16;
 constexpr int kMaxDens = 128;    // Ndens limit (search buffer is 4 * Ndens + slack)
 constexpr int kHistBins = 32;    // 1/8-octave bins of d^2 used for selection
 
+constexpr int kSposPad = 16;     // NaN records after the sorted positions (the last run and one past it)
+
 // Device error word bits (atomicOr'ed by kernels, read by the host).
 enum : uint32_t {
     kErrBadPos = 1u << 0,       // a coordinate outside [0, box) or NaN
@@ -62,6 +64,7 @@ enum Slot {
     S_SUB,                              // subhalos: dense chain ids, per-particle chain ids
     S_SUB_C,                            // subhalos: arrays over chains and boundaries
     S_KNN_HAND,                         // queries that the grouped kNN hands over
+    S_BOX,                              // bounding boxes over the sorted particles
     S_COUNT
 };
 
@@ -197,6 +200,7 @@ inline float plain_radius_for(int64_t n, double box, int k)
 // entries holding global sorted positions) starts at cell0.
 struct SegDesc {
     int64_t base, n, chunk0, cell0;
+    int64_t unit0;        // first unit of 16 queries (the grouped kNN)
     double box;
     double norm;          // box^3 / (n pi): density normalisation
     float plain_r;
@@ -210,6 +214,17 @@ __device__ __forceinline__ int seg_of_chunk(const SegDesc *__restrict__ seg, int
     while (lo < hi) {
         const int m = (lo + hi + 1) >> 1;
         if (seg[m].chunk0 <= ch) lo = m; else hi = m - 1;
+    }
+    return lo;
+}
+
+// The subvolume holding unit `u` of 16 queries.
+__device__ __forceinline__ int seg_of_unit(const SegDesc *__restrict__ seg, int B, int64_t u)
+{
+    int lo = 0, hi = B - 1;
+    while (lo < hi) {
+        const int m = (lo + hi + 1) >> 1;
+        if (seg[m].unit0 <= u) lo = m; else hi = m - 1;
     }
     return lo;
 }
@@ -384,6 +399,17 @@ int radius_closed(hop_ctx *c, const void *spos, const uint64_t *keys, const uint
                   int64_t n_chunks, int qpw, double box, const SegDesc *seg, int B, int k, float log_margin,
                   float *chunk_r);
 
+// boxtree.cu: node i of level j is the box of sorted particles
+// [i << (3 j + 3), (i + 1) << (3 j + 3)), at lo / hi [off[j] + i]
+constexpr int kBoxTop = 32;        // nodes of the top level, at most
+constexpr int kBoxLevels = 12;
+struct BoxTree {
+    const float4 *lo, *hi;
+    uint32_t off[kBoxLevels];
+    int levels;
+};
+int box_tree_build(hop_ctx *c, const float4 *spos, int64_t n, BoxTree *t);
+
 // knn.cu
 struct KnnArgs {
     const void *spos;          // sorted positions (float4 / double4)
@@ -404,6 +430,7 @@ struct KnnArgs {
     const SegDesc *seg = nullptr;   // batched pass: subvolume descriptors (device)
     int B = 0;                      // number of subvolumes
     int64_t n_chunks = 0;           // batched pass: total query chunks
+    int64_t n_units = 0;            // batched pass: total units of 16 queries
 };
 int knn_launch(hop_ctx *c, const KnnArgs &a, bool f64, int qpw, int cpr);
 int knn32_launch(hop_ctx *c, const KnnArgs &a, int cpr);   // knn32.cu: one query per lane, float32

@@ -2,41 +2,51 @@
 // step 1, Parallel HOP Sec. 2) for float32 positions: four queries per warp,
 // eight lanes per query.
 //
-// A warp takes four consecutive Morton-sorted particles.  Consecutive ones
-// farther apart than the first radius (a jump of the Morton curve) are
-// searched one after another, the others together:
-//   1. Cells.  The cells (side about R / cpr) that meet the members' bounding
-//      box grown by R are listed once for all of them; the Morton code and
-//      the gap of each axis cell are computed by one lane each and combined
-//      by shuffles.
-//   2. Staging.  The lanes read the cells' particles, 128 per step (four
-//      independent 16-byte loads per lane), and the ones within R of the box
-//      go to a tile in shared memory.
-//   3. Evaluation.  Lane p of a query takes every eighth staged particle; d^2
-//      and sorted index of those within R go to the lane's own list, one
-//      column of a [slot][lane] array, so that no two lanes meet in a bank
-//      and no ballot is needed.  When a list is nearly full, the query's
-//      limit drops to the upper edge of the bin holding its Ndens-th entry.
+// A warp takes a unit of 16 consecutive Morton-sorted particles and serves
+// them in four groups of four.  Consecutive ones farther apart than the
+// first radius (a jump of the Morton curve) are searched one after another,
+// the others of a group together:
+//   1. Boxes, down to 512 particles.  The tree of bounding boxes over the
+//      sorted particles (boxtree.cu) is walked once per unit, level by level,
+//      32 boxes per step, to the 512-particle nodes that meet the unit's box
+//      grown by its largest first radius.
+//   2. Boxes, down to eight particles.  Of those, the nodes that meet the
+//      group's box grown by R are opened, then the 64-particle nodes below
+//      them; what is left is a list of runs of eight particles.
+//   3. Evaluation.  Lane p of a query reads particle p of each run, so the
+//      four queries share one 128-byte line; d^2 and sorted index of those
+//      within R go to the lane's own list, one column of a [slot][lane]
+//      array: no two lanes meet in a bank and no ballot is needed.  When a
+//      list is nearly full, the query's limit drops to the upper edge of the
+//      bin holding its Ndens-th entry.
 //   4. Selection.  A histogram of the query's lists (32 bins linear in d^2,
-//      two 16-bit counts per word) places the entries up to the Ndens-th
+//      16-bit counts) places the entries up to the Ndens-th
 //      bin, bin by bin, in one array (a counting sort).  The exact Ndens-th
 //      d^2 is ranked within its bin, the density is a fixed-point sum over
 //      the array, and an entry's place in the neighbour list is the start of
 //      its bin plus its rank in it by (d^2, original index).
 // A query is certified when at least Ndens particles lie within R; the
 // others search again with a larger R.  What this kernel does not take -- a
-// ball that wraps around the box, more cells than it lists, a crowd at the
+// ball that wraps around the box, more nodes than it lists, a crowd at the
 // Ndens-th distance -- it hands over to the warp-per-query kernel
 // (knn_cg.cu), which runs after it over the list of such queries.
 //
-// What bounds it: instruction issue and latency (2.0k warp instructions per
-// particle, issue 43 % busy at 16 warps per SM; DRAM and tensor cores play no
-// part).  Four queries share the cell listing and the reads that a warp per
-// query repeats for each, and eight lanes per query keep private lists, which
-// need no ballots.  Kernel time against a warp per query (3.7k instructions),
-// learned first radius unless stated: 16.8M particles 82.1 -> 68.4 ms, 64
-// subvolumes of 22M together 111.8 -> 86.2 ms, 3M with Ndens = Nhop = 65
-// (closed form) 22.2 -> 15.3 ms, 4,913 particles 0.99 -> 0.40 ms.
+// What bounds it: shared-memory wavefronts (72 % of peak; every run is read
+// by the four queries' lanes, 16 bytes each) and instruction issue (60 % busy
+// at 16 warps per SM, 1.6k warp instructions per particle); DRAM and tensor
+// cores play no part.  Four queries share the walk and the reads that a warp
+// per query repeats for each.  The code is kept small on purpose (loops not
+// unrolled, one call site of what is long, rare parts out of line): at 55 KB
+// instead of 42 KB instruction-cache misses were the largest stall and the
+// 16.8M-particle kNN took 48.3 ms instead of 37.7.  Runs come through
+// cp.async, three steps ahead: with loads into registers the loop held 60
+// register moves per step and took 77 ms.
+// Kernel time, with learned first radius unless stated, against a cell
+// listing per four queries (and a warp per query): 16.8M particles 68.4 ->
+// 37.7 ms (82.1), 64 subvolumes of 22M together 86.2 -> 53.1 ms (111.8), 3M
+// with Ndens = Nhop = 65 (closed form) 15.3 -> 10.2 ms (22.2), 2.1M with the
+// plain radius, whose start is cut to what the boxes show to be enough, 53.8
+// -> 20.5 ms (59.2).
 //
 // Results equal those of the other kNN kernels bit for bit: the same
 // per-component minimum-image differences, the same fused d^2, the same
@@ -53,20 +63,21 @@ constexpr uint32_t kAll = 0xffffffffu;
 constexpr int kGqWarps = 4;            // warps per block
 constexpr int kGqQ = 4;                // queries per warp (eight lanes each)
 constexpr int kGqSlots = 32;           // list entries per lane
-constexpr int kGqTile = 160;           // staged particles
-constexpr int kGqCells = 128;          // cells held at once
-constexpr int kGqAxis = 10;            // axis cells of a region, at most
+constexpr int kGqUnit = 16;            // queries of a unit
+constexpr int kGqN2 = 96;              // 512-particle nodes held
+constexpr int kGqN1 = 192;             // 64-particle nodes held at once
+constexpr int kGqN0 = 256;             // runs of eight particles held at once
 constexpr int kGqBins = 32;            // histogram bins, linear in d^2
 constexpr int kGqTries = 96;
 
 struct GqDev {
     const float4 *spos;
-    const uint64_t *keys;
-    const uint32_t *cellT;
-    int level_dense;
-    int64_t n, n_groups;
-    int gpc;                           // groups per radius chunk
-    float box, norm, cells_per_box;
+    BoxTree tree;
+    uint32_t n, pad_run;               // pad_run: a run past the last particle
+    int64_t n_tasks;                   // units of 16 queries, in `split` parts each
+    int split;
+    int qpw;                           // queries per radius chunk
+    float box, norm;
     int k, n_out, ld_out, capq;
     const float *chunk_r;
     float plain_r;
@@ -77,38 +88,136 @@ struct GqDev {
     float *rk_s;
     uint32_t *hand;                    // queries handed over ...
     unsigned long long *hand_n;        // ... and their number
-    unsigned long long *group_counter, *counters;
+    unsigned long long *task_counter, *counters;
     uint32_t *err;
 };
 
-// Shared memory of one warp, byte offsets.  The cells and the tile (search)
-// share their space with the sorted arrays (selection).
+// Shared memory of one warp, byte offsets.  The node lists (search) share
+// their space with the sorted arrays (selection).
 struct GqSmem {
-    static constexpr int ld = 0;                                    // [kGqSlots][32] d^2
-    static constexpr int ls = ld + kGqSlots * 128;                  // [kGqSlots][32] sorted index
-    static constexpr int hist = ls + kGqSlots * 128;                // [kGqBins / 2][32] two 16-bit counts
-    static constexpr int bst = hist + kGqBins / 2 * 128;            // [kGqQ][kGqBins + 2] u16 bin starts
-    static constexpr int cra = (bst + kGqQ * (kGqBins + 2) * 2 + 15) & ~15;   // kGqCells range starts
-    static constexpr int cpre = cra + kGqCells * 4;                 // kGqCells + 4 prefix offsets
-    static constexpr int tile = cpre + (kGqCells + 4) * 4;          // kGqTile float4
-    static_assert(tile % 16 == 0, "the tile is read 16 bytes at a time");
+    static constexpr int list = 0;                                  // [kGqSlots][32] d^2 and run
+    static constexpr int hist = list + kGqSlots * 256;              // [kGqBins][32] u16 counts
+    static constexpr int bst = hist + kGqBins * 64;                 // [kGqQ][kGqBins + 2] u16 bin starts
+    static constexpr int u2 = (bst + kGqQ * (kGqBins + 2) * 2 + 15) & ~15;   // the unit's 512-particle nodes
+    static constexpr int t0 = u2 + kGqN2 * 4;                       // a search's runs (read 16 bytes at a time) ...
+    static constexpr int t1 = t0 + (kGqN0 + 8) * 4;                 // ... 64-particle nodes ...
+    static constexpr int t2 = t1 + kGqN1 * 4;                       // ... and 512-particle nodes
+    static constexpr int search_end = t2 + kGqN2 * 4;
+    static_assert(t0 % 16 == 0, "runs are read 16 bytes at a time");
+    // Row stride of the sorted arrays: 8 mod 32, so that the four queries'
+    // lanes (eight consecutive words each) read distinct banks.
+    __host__ __device__ static int stride(int capq) { return (capq + 23) / 32 * 32 + 8; }
     __host__ __device__ static int total(int capq)
     {
-        const int search = tile + kGqTile * 16, sel = cra + kGqQ * capq * 8;
-        return ((search > sel ? search : sel) + 15) & ~15;
+        const int sel = t0 + kGqQ * stride(capq) * 8;
+        return ((search_end > sel ? search_end : sel) + 15) & ~15;
     }
 };
 
-__device__ __forceinline__ float quad_min(float v)
+static_assert(kGqBins * 64 == 4 * 512, "the histogram's space holds four steps of four runs");
+
+extern __shared__ __align__(16) unsigned char gq_smem[];
+
+// Shared-memory byte address of an offset into gq_smem.
+__device__ __forceinline__ uint32_t gq_addr(uint32_t o) { return (uint32_t)__cvta_generic_to_shared(gq_smem + o); }
+
+__device__ __forceinline__ void copy16_async(uint32_t dst, const void *src)
 {
-    v = fminf(v, __shfl_xor_sync(kAll, v, 8));
-    return fminf(v, __shfl_xor_sync(kAll, v, 16));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
-__device__ __forceinline__ float quad_max(float v)
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// Appends (d2, run) to the lane's list when d2 <= tau: one predicated store
+// and one predicated add.
+__device__ __forceinline__ void gq_keep(uint32_t &lp, float d2, float tau, uint32_t run)
 {
-    v = fmaxf(v, __shfl_xor_sync(kAll, v, 8));
-    return fmaxf(v, __shfl_xor_sync(kAll, v, 16));
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.le.f32 p, %1, %2;\n\t@p st.shared.v2.b32 [%0], {%3, %4};\n\t"
+                 "@p add.u32 %0, %0, 256;\n\t}"
+                 : "+r"(lp)
+                 : "f"(d2), "f"(tau), "r"(__float_as_uint(d2)), "r"(run)
+                 : "memory");
 }
+
+__device__ __forceinline__ float warp_min(float v)
+{
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float warp_max(float v)
+{
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+// A box grown by a radius: a node meets it when its distance from the box
+// (made a little smaller, so that rounding never drops one) is within r.
+// Where the grown box crosses a face, coordinates >= L/2 move by -L (exact),
+// and a node is taken at both places.
+struct Region {
+    float lx, hx, ly, hy, lz, hz, r2c, box;
+    bool wx, wy, wz, shifted;
+    __device__ __forceinline__ static float gap(float lo, float hi, float l, float h)
+    {
+        return fmaxf(fmaxf(lo - h, l - hi), 0.f);
+    }
+    __device__ __forceinline__ bool meets(const float4 &lo, const float4 &hi) const
+    {
+        float gx = gap(lo.x, hi.x, lx, hx), gy = gap(lo.y, hi.y, ly, hy), gz = gap(lo.z, hi.z, lz, hz);
+        if (shifted) {
+            // (an axis that is not shifted takes the same place twice)
+            const float bx = wx ? box : 0.f, by = wy ? box : 0.f, bz = wz ? box : 0.f;
+            gx = fminf(gx, gap(lo.x - bx, hi.x - bx, lx, hx));
+            gy = fminf(gy, gap(lo.y - by, hi.y - by, ly, hy));
+            gz = fminf(gz, gap(lo.z - bz, hi.z - bz, lz, hz));
+        }
+        return gx * gx + gy * gy + gz * gz <= r2c;
+    }
+    // The region of the lanes' points (those with `in`) for radius r; false
+    // when it wraps around the box or crosses both a face and L/2 on an
+    // axis.  x, y, z become the points' coordinates in the region's frame.
+    __device__ __forceinline__ bool build(bool in, float &x, float &y, float &z, float r, float box_)
+    {
+        box = box_;
+        const float half = 0.5f * box, eps = box * 9.5367431640625e-7f;   // 2^-20 of the box: far above rounding
+        lx = warp_min(in ? x : INFINITY);
+        hx = warp_max(in ? x : -INFINITY);
+        ly = warp_min(in ? y : INFINITY);
+        hy = warp_max(in ? y : -INFINITY);
+        lz = warp_min(in ? z : INFINITY);
+        hz = warp_max(in ? z : -INFINITY);
+        wx = lx - r < 0.f || hx + r >= box;
+        wy = ly - r < 0.f || hy + r >= box;
+        wz = lz - r < 0.f || hz + r >= box;
+        shifted = wx || wy || wz;
+        if (2.f * r >= half) return false;
+        if (shifted) {
+            if ((wx && lx - r < half && half <= hx + r) || (wy && ly - r < half && half <= hy + r) ||
+                (wz && lz - r < half && half <= hz + r))
+                return false;
+            if (wx && x >= half) x -= box;
+            if (wy && y >= half) y -= box;
+            if (wz && z >= half) z -= box;
+            lx = warp_min(in ? x : INFINITY);
+            hx = warp_max(in ? x : -INFINITY);
+            ly = warp_min(in ? y : INFINITY);
+            hy = warp_max(in ? y : -INFINITY);
+            lz = warp_min(in ? z : INFINITY);
+            hz = warp_max(in ? z : -INFINITY);
+        }
+        lx -= eps;
+        hx += eps;
+        ly -= eps;
+        hy += eps;
+        lz -= eps;
+        hz += eps;
+        r2c = r * r * 1.00001f + box * box * 1e-12f;
+        return true;
+    }
+};
+
 // Sum over the eight lanes of a query.
 __device__ __forceinline__ int oct_sum(int v)
 {
@@ -117,63 +226,78 @@ __device__ __forceinline__ int oct_sum(int v)
     return v + __shfl_xor_sync(kAll, v, 4);
 }
 
-__device__ __forceinline__ int gq_bin(float d2, float scale) { return min((int)(d2 * scale), kGqBins - 1); }
+// Bin of a d^2 <= tau: the integer part of d^2 * scale, left in the low bits
+// of a float (one instruction, exact product, rounded towards zero); scale
+// keeps it below kGqBins.
+__device__ __forceinline__ float gq_scale(float tau) { return fminf(__fdividef(kGqBins - 0.01f, tau), 5e37f); }
+__device__ __forceinline__ int gq_bin(float d2, float scale)
+{
+    return (int)(__float_as_uint(__fmaf_rz(d2, scale, 8388608.f)) - 0x4b000000u);
+}
+// A value that only later bins exceed.
+__device__ __forceinline__ float gq_edge(int bin, float scale) { return __fdividef((float)(bin + 1), scale) * 1.000002f; }
 
-// Counts the lanes' lists into the histogram and finds, for each query, the
-// bin of the rank-th entry: packed as bin << 20 | below << 10 | upto (0 when
-// the lists hold fewer).  With `place` the histogram words become the
-// positions at which each lane's entries of a bin go, and bst the bins'
-// starts.
+// Counts the lanes' lists (cnt entries) into the histogram and
+// finds, for each query, the bin of its k-th and of its n_out-th entry:
+// packed as bin << 20 | below << 10 | upto (0 when the lists hold fewer).
+// With PLACE the histogram becomes the positions at which each lane's
+// entries of a bin go, and bst the bins' starts.
 struct GqFound {
     uint32_t k, o;
 };
 template <bool PLACE>
-__device__ __forceinline__ GqFound gq_count(const float *Ld, uint32_t *hist, uint16_t *bst, int cnt, int cmax,
-                                            float scale, int k, int n_out, int lane)
+__device__ __forceinline__ GqFound gq_count(const float2 *list, int cnt, int cmax, uint16_t *hist,
+                                            uint16_t *bst, float scale, int k, int n_out, int lane)
 {
     const int q = lane >> 3, p = lane & 7;
 #pragma unroll
-    for (int i = 0; i < kGqBins / 2 * 32 / 128; ++i)
-        reinterpret_cast<uint4 *>(hist)[i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 0; i < kGqBins * 64 / 512; ++i) reinterpret_cast<uint4 *>(hist)[i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
-    for (int i = 0; i < cmax; ++i) {
-        if (i < cnt) {
-            const int b = gq_bin(Ld[i * 32], scale);
-            hist[(b >> 1) * 32 + lane] += 1u << ((b & 1) * 16);
+    uint16_t *col = hist + lane;
+#pragma unroll 1
+    for (int i = 0; i < cmax; i += 2) {
+        // (a column has an even number of slots)
+        const float v0 = list[i * 32].x, v1 = list[(i + 1) * 32].x;
+        if (i < cnt) ++col[gq_bin(v0, scale) * 32];
+        if (i + 1 < cnt) ++col[gq_bin(v1, scale) * 32];
+    }
+    __syncwarp();
+    // lane p holds bins p, p + 8, p + 16, p + 24 of its query, each one read
+    // of 16 bytes (the query's eight lanes)
+    uint4 w[4];
+    int t[4], st[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        w[j] = *reinterpret_cast<const uint4 *>(hist + (p + 8 * j) * 32 + q * 8);
+        const uint32_t s = w[j].x + w[j].y + w[j].z + w[j].w;
+        t[j] = (int)((s & 0xffffu) + (s >> 16));
+    }
+    {
+        uint32_t a = (uint32_t)t[0] | ((uint32_t)t[1] << 16), b = (uint32_t)t[2] | ((uint32_t)t[3] << 16);
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+            const uint32_t ya = __shfl_up_sync(kAll, a, o, 8), yb = __shfl_up_sync(kAll, b, o, 8);
+            if (p >= o) {
+                a += ya;
+                b += yb;
+            }
         }
+        const uint32_t sa = __shfl_sync(kAll, a, 7, 8), sb = __shfl_sync(kAll, b, 7, 8);
+        const int n0 = sa & 0xffffu, n1 = n0 + (int)(sa >> 16), n2 = n1 + (int)(sb & 0xffffu);
+        st[0] = (int)(a & 0xffffu) - t[0];
+        st[1] = n0 + (int)(a >> 16) - t[1];
+        st[2] = n1 + (int)(b & 0xffffu) - t[2];
+        st[3] = n2 + (int)(b >> 16) - t[3];
+        if constexpr (PLACE)
+            if (p == 7) bst[q * (kGqBins + 2) + kGqBins] = (uint16_t)(n2 + (int)(sb >> 16));
     }
-    __syncwarp();
-    // lane p holds bins 4p .. 4p + 3 (words 2p, 2p + 1) of its query; column
-    // r of the query's eight is read in an order of each lane's own, so that
-    // the lanes read distinct banks
-    uint32_t *w0 = hist + 2 * p * 32 + q * 8, *w1 = w0 + 32;
-    uint32_t s0 = 0, s1 = 0;
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-        const int c = (r + p) & 7;
-        s0 += w0[c];
-        s1 += w1[c];
-    }
-    const int n0 = s0 & 0xffffu, n1 = s0 >> 16, n2 = s1 & 0xffffu, n3 = s1 >> 16;
-    int incl = n0 + n1 + n2 + n3;
-    const int tot = incl;
-#pragma unroll
-    for (int o = 1; o < 8; o <<= 1) {
-        const int y = __shfl_up_sync(kAll, incl, o, 8);
-        if (p >= o) incl += y;
-    }
-    const int b0 = incl - tot, b1 = b0 + n0, b2 = b1 + n1, b3 = b2 + n2, b4 = incl;
     auto find = [&](int rank) {
         uint32_t v = 0;
-        const bool has = b0 < rank && rank <= b4;
-        if (has) {
-            int bin = 4 * p, lo = b0, hi = b1;
-            if (rank > b1) { bin = 4 * p + 1; lo = b1; hi = b2; }
-            if (rank > b2) { bin = 4 * p + 2; lo = b2; hi = b3; }
-            if (rank > b3) { bin = 4 * p + 3; lo = b3; hi = b4; }
-            v = ((uint32_t)bin << 20) | ((uint32_t)lo << 10) | (uint32_t)hi;
-        }
-        const uint32_t m = (__ballot_sync(kAll, has) >> (q * 8)) & 0xffu;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (st[j] < rank && rank <= st[j] + t[j])
+                v = ((uint32_t)(p + 8 * j) << 20) | ((uint32_t)st[j] << 10) | (uint32_t)(st[j] + t[j]);
+        const uint32_t m = (__ballot_sync(kAll, v != 0u) >> (q * 8)) & 0xffu;
         v = __shfl_sync(kAll, v, q * 8 + (m ? __ffs(m) - 1 : 0));
         return m ? v : 0u;
     };
@@ -181,198 +305,246 @@ __device__ __forceinline__ GqFound gq_count(const float *Ld, uint32_t *hist, uin
     f.k = find(k);
     f.o = n_out > 0 ? find(n_out) : 0u;
     if constexpr (PLACE) {
-        uint32_t r0 = (uint32_t)b0 | ((uint32_t)b1 << 16), r1 = (uint32_t)b2 | ((uint32_t)b3 << 16);
-        uint16_t *t = bst + q * (kGqBins + 2) + 4 * p;
-        t[0] = (uint16_t)b0;
-        t[1] = (uint16_t)b1;
-        t[2] = (uint16_t)b2;
-        t[3] = (uint16_t)b3;
-        if (p == 7) t[4] = (uint16_t)b4;
 #pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            const int c = (r + p) & 7;
-            const uint32_t x0 = w0[c], x1 = w1[c];
-            w0[c] = r0;
-            w1[c] = r1;
-            r0 += x0;
-            r1 += x1;
+        for (int j = 0; j < 4; ++j) {
+            uint32_t r = (uint32_t)st[j];
+            auto next = [&](uint32_t x) {
+                const uint32_t out = r * 0x10001u + (x << 16);
+                r += (x & 0xffffu) + (x >> 16);
+                return out;
+            };
+            uint4 o;
+            o.x = next(w[j].x);
+            o.y = next(w[j].y);
+            o.z = next(w[j].z);
+            o.w = next(w[j].w);
+            *reinterpret_cast<uint4 *>(hist + (p + 8 * j) * 32 + q * 8) = o;
+            bst[q * (kGqBins + 2) + p + 8 * j] = (uint16_t)st[j];
         }
         __syncwarp();
     }
     return f;
 }
 
-// The largest d^2 of bin `bin`, rounded up: every value above it falls in a
-// later bin.
-__device__ __forceinline__ float gq_edge(int bin, float scale) { return (float)(bin + 1) / scale * 1.000001f; }
-
 // Drops the limit of every query that holds at least k entries (and is in
 // `which`) to the upper edge of the bin of its k-th, and its lists to the
 // entries up to it.  Out of line: only lists that are nearly full, or a
 // crowded k-th bin, need it.
-__device__ __noinline__ void gq_tighten(float *Ld, uint32_t *Ls, uint32_t *hist, bool which, int &cnt, float &tau, int k,
-                                        int lane)
+struct Tight {
+    int cnt;
+    float tau;
+};
+__device__ __noinline__ Tight gq_tighten(uint32_t wo, int cnt, bool which, float tau, int k, int lane)
 {
-    const int cmax = (int)__reduce_max_sync(kAll, (unsigned)cnt);
-    const float scale = (float)kGqBins / tau;
-    const GqFound f = gq_count<false>(Ld, hist, nullptr, which ? cnt : 0, cmax, scale, k, 0, lane);
+    float2 *list = (float2 *)(gq_smem + wo + GqSmem::list) + lane;
+    uint16_t *hist = (uint16_t *)(gq_smem + wo + GqSmem::hist);
+    const int cmax = (int)__reduce_max_sync(kAll, which ? (unsigned)cnt : 0u);
+    const float scale = gq_scale(tau);
+    const GqFound f = gq_count<false>(list, which ? cnt : 0, cmax, hist, nullptr, scale, k, 0, lane);
     if (which && f.k) {
-        const float e = fminf(tau, gq_edge((int)(f.k >> 20), scale));
+        tau = fminf(tau, gq_edge((int)(f.k >> 20), scale));
         int m = 0;
+#pragma unroll 1
         for (int i = 0; i < cnt; ++i) {
-            const float v = Ld[i * 32];
-            const uint32_t s = Ls[i * 32];
-            if (v <= e) {
-                Ld[m * 32] = v;
-                Ls[m * 32] = s;
+            const float2 v = list[i * 32];
+            if (v.x <= tau) {
+                list[m * 32] = v;
                 ++m;
             }
         }
         cnt = m;
-        tau = e;
     }
     __syncwarp();
+    return {cnt, tau};
 }
 
-// Lists the non-empty cells of level l that meet the box [fl, fh] grown by
-// r; returns their count, or -1 if an axis or the list is too long.
-__device__ __forceinline__ int gq_cells(float flx, float fhx, float fly, float fhy, float flz, float fhz, float r,
-                                        float box, int l, const uint32_t *__restrict__ cellT,
-                                        const uint64_t *__restrict__ keys, int level_dense, uint32_t *cra, uint32_t *cln,
-                                        int lane, uint32_t lt)
+// The 512-particle nodes over sorted particles [base, end) that meet the
+// region, at offset oa (ob: scratch of the same size); returns their count, or -1 if
+// a level has more than kGqN2.  Out of line: once per unit, and for searches
+// beyond the unit's radius.
+__device__ __noinline__ int gq_descend(const BoxTree &t, const Region rg, uint32_t base, uint32_t end, uint32_t oa,
+                                       uint32_t ob, int lane)
 {
-    const int G = 1 << l;
-    const float csz = box / (float)G, sc = (float)G / box;
-    const float eps = box * 9.5367431640625e-7f;   // 2^-20 of the box: far above coordinate rounding
-    const float r2c = r * r * 1.00001f + box * box * 1e-12f;
-    // lane 10 a + i: cell i of axis a
-    const int ax = lane < kGqAxis ? 0 : lane < 2 * kGqAxis ? 1 : 2;
-    const float fl = ax == 0 ? flx : ax == 1 ? fly : flz, fh = ax == 0 ? fhx : ax == 1 ? fhy : fhz;
-    const int c0 = (int)floorf((fl - r - eps) * sc), na = (int)floorf((fh + r + eps) * sc) - c0 + 1;
-    const int nx = __shfl_sync(kAll, na, 0), ny = __shfl_sync(kAll, na, kGqAxis), nz = __shfl_sync(kAll, na, 2 * kGqAxis);
-    if (max(nx, max(ny, nz)) > min(kGqAxis, G)) return -1;
-    const int ca = c0 + (lane - kGqAxis * ax);
-    const float gap = fmaxf(0.f, fmaxf(fl - (float)(ca + 1) * csz, (float)ca * csz - fh) - eps);
-    const float gap2 = gap * gap;
-    const uint32_t cw = (uint32_t)ca & (uint32_t)(G - 1);
-    const uint32_t m0 = spread3_8(cw) << ax, m1 = spread3_8(cw >> 8) << ax;
-    const int nxy = nx * ny, ncube = nxy * nz;
-    // cell ci of the cube is (ci mod nx, (ci / nx) mod ny, ci / (nx ny)); the
-    // quotients come from float reciprocals, exact for these small integers
-    const float inx = 1.f / (float)nx, inxy = 1.f / (float)nxy;
-    int nkeep = 0;
-    for (int cb = 0; cb < ncube; cb += 32) {
-        const int ci = cb + lane, cc = min(ci, ncube - 1);
-        const int iz = (int)(((float)cc + 0.5f) * inxy);
-        const int rxy = cc - iz * nxy;
-        const int iy = (int)(((float)rxy + 0.5f) * inx);
-        const int ix = rxy - iy * nx;
-        const int jy = iy + kGqAxis, jz = iz + 2 * kGqAxis;
-        const float g2 = __shfl_sync(kAll, gap2, ix) + __shfl_sync(kAll, gap2, jy) + __shfl_sync(kAll, gap2, jz);
-        const uint32_t lo = __shfl_sync(kAll, m0, ix) | __shfl_sync(kAll, m0, jy) | __shfl_sync(kAll, m0, jz);
-        const uint32_t hi = __shfl_sync(kAll, m1, ix) | __shfl_sync(kAll, m1, jy) | __shfl_sync(kAll, m1, jz);
-        uint32_t ra = 0, rb = 0;
-        if (ci < ncube && g2 <= r2c) cell_range(cellT, keys, level_dense, l, ((uint64_t)hi << 24) | lo, ra, rb);
-        const uint32_t bal = __ballot_sync(kAll, rb > ra);
-        const int pos = nkeep + __popc(bal & lt);
-        if (rb > ra && pos < kGqCells) {
-            cra[pos] = ra;
-            cln[pos] = rb - ra;
+    uint32_t *A = (uint32_t *)(gq_smem + oa), *B = (uint32_t *)(gq_smem + ob);
+    const uint32_t lt = (1u << lane) - 1u;
+    int lv = 2;
+    while (((end - 1) >> (3 * lv + 3)) - (base >> (3 * lv + 3)) >= (uint32_t)kBoxTop) ++lv;
+    uint32_t *cur = (lv & 1) ? B : A, *nxt = (lv & 1) ? A : B;
+    const uint32_t first = base >> (3 * lv + 3), cnt = ((end - 1) >> (3 * lv + 3)) - first + 1;
+    int n;
+    {
+        const uint32_t node = first + (uint32_t)lane;
+        bool in = (uint32_t)lane < cnt;
+        if (in) in = rg.meets(t.lo[t.off[lv] + node], t.hi[t.off[lv] + node]);
+        const uint32_t bal = __ballot_sync(kAll, in);
+        if (in) cur[__popc(bal & lt)] = node;
+        n = __popc(bal);
+    }
+    for (--lv; lv >= 2; --lv) {
+        __syncwarp();
+        int m = 0;
+        for (int i = 0; i < n; i += 4) {
+            const int j = i + (lane >> 3);
+            bool in = j < n;
+            uint32_t node = 0;
+            if (in) {
+                node = cur[j] * 8 + (lane & 7);
+                in = rg.meets(t.lo[t.off[lv] + node], t.hi[t.off[lv] + node]);
+            }
+            const uint32_t bal = __ballot_sync(kAll, in);
+            const int pos = m + __popc(bal & lt);
+            if (in && pos < kGqN2) nxt[pos] = node;
+            m += __popc(bal);
         }
-        nkeep += __popc(bal);
-        if (nkeep > kGqCells) break;
+        if (m > kGqN2) return -1;
+        n = m;
+        uint32_t *x = cur;
+        cur = nxt;
+        nxt = x;
     }
     __syncwarp();
-    return nkeep <= kGqCells ? nkeep : -1;
+    return n;
 }
 
-// Turns the nc cell lengths in cpre into their exclusive prefix, cpre[nc] the
-// total (returned); four cells per lane.
-__device__ __forceinline__ uint32_t gq_prefix(uint32_t *cpre, int nc, int lane)
+// Appends the children of up to 16 nodes of level lv + 1 (list[i ..  n)) that
+// meet the region to out (m entries so far; room for 128 more); the four
+// steps' loads are independent.
+__device__ __forceinline__ int gq_open(const BoxTree &t, int lv, const Region &rg, const uint32_t *list, int i, int n,
+                                       uint32_t *out, int m, int lane, uint32_t lt)
 {
-    static_assert(kGqCells == 128, "four cells per lane");
-    const uint4 v = reinterpret_cast<const uint4 *>(cpre)[lane];
-    const int j = 4 * lane;
-    const uint32_t a = j < nc ? v.x : 0u, b = j + 1 < nc ? v.y : 0u, c = j + 2 < nc ? v.z : 0u, d = j + 3 < nc ? v.w : 0u;
-    const uint32_t mine = a + b + c + d;
-    uint32_t incl = mine;
+    const float4 *lo = t.lo + t.off[lv], *hi = t.hi + t.off[lv];
+    uint32_t node[4];
+    float4 l[4], h[4];
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(kAll, incl, o);
-        if (lane >= o) incl += y;
+    for (int u = 0; u < 4; ++u) {
+        const int j = i + 4 * u + (lane >> 3);
+        node[u] = list[min(j, n - 1)] * 8 + (lane & 7);
+        if (i + 4 * u < n) {
+            l[u] = lo[node[u]];
+            h[u] = hi[node[u]];
+        }
     }
-    const uint32_t e = incl - mine, total = __shfl_sync(kAll, incl, 31);
-    __syncwarp();
-    reinterpret_cast<uint4 *>(cpre)[lane] = make_uint4(e, e + a, e + a + b, e + a + b + c);
-    if (lane == 0) cpre[kGqCells] = total;   // read as cpre[nc] when every cell is in use
-    __syncwarp();
-    return total;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        if (i + 4 * u >= n) break;
+        const bool in = i + 4 * u + (lane >> 3) < n && rg.meets(l[u], h[u]);
+        const uint32_t bal = __ballot_sync(kAll, in);
+        if (in) out[m + __popc(bal & lt)] = node[u];
+        m += __popc(bal);
+    }
+    return m;
+}
+
+// The first radius of the plain policy at particle s: the mean-density
+// distance, or where that is larger the distance to the farthest corner of
+// the boxes that hold the particle's own 64 (more than 64 wanted: 128)
+// neighbours in sort order, which is enough for k of them.
+__device__ __noinline__ float gq_plain_radius(const BoxTree &t, float4 v, uint32_t s, uint32_t base, uint32_t end, int k,
+                                              float plain_r)
+{
+    const int nodes = k <= 64 ? 1 : 2;
+    const uint32_t node = (s >> 6) & ~(uint32_t)(nodes - 1);
+    if (node * 64 < base || (uint64_t)(node + nodes) * 64 > end) return plain_r;
+    float dx = 0.f, dy = 0.f, dz = 0.f;
+    for (int i = 0; i < nodes; ++i) {
+        const float4 lo = t.lo[t.off[1] + node + i], hi = t.hi[t.off[1] + node + i];
+        dx = fmaxf(dx, fmaxf(v.x - lo.x, hi.x - v.x));
+        dy = fmaxf(dy, fmaxf(v.y - lo.y, hi.y - v.y));
+        dz = fmaxf(dz, fmaxf(v.z - lo.z, hi.z - v.z));
+    }
+    return fminf(plain_r, sqrtf(dx * dx + dy * dy + dz * dz) * 1.0001f);
+}
+
+// The factor by which a radius grows that held tot < k particles.
+__device__ __noinline__ float gq_grow(int k, int tot)
+{
+    return fmaxf(1.25f, 1.1f * cbrtf((float)k / (float)max(tot, 1)));
 }
 
 template <bool SEG>
-__global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(GqDev a)
+__global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
 {
     using L = GqSmem;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int lane = threadIdx.x & 31;
+    int lane;
+    asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));   // (kept in a register)
     const int q = lane >> 3, p = lane & 7;
     const uint32_t lt = (1u << lane) - 1u;
-    unsigned char *wb = smem_raw + L::total(a.capq) * (threadIdx.x >> 5);
-    float *Ld = (float *)(wb + L::ld) + lane;
-    uint32_t *Ls = (uint32_t *)(wb + L::ls) + lane;
-    uint32_t *hist = (uint32_t *)(wb + L::hist);
+    const uint32_t wo = (uint32_t)L::total(a.capq) * (threadIdx.x >> 5);   // the warp's shared memory
+    unsigned char *wb = gq_smem + wo;
+    float2 *list = (float2 *)(wb + L::list) + lane;
+    const uint32_t list0 = gq_addr(wo + L::list) + lane * 8;
+    const uint32_t full = list0 + (kGqSlots - 4) * 256;   // a list beyond it has no room for four more
+    const uint32_t stage_st = gq_addr(wo + L::hist) + lane * 16;
+    uint16_t *hist = (uint16_t *)(wb + L::hist);
     uint16_t *bst = (uint16_t *)(wb + L::bst);
-    uint32_t *cra = (uint32_t *)(wb + L::cra), *cpre = (uint32_t *)(wb + L::cpre);
-    float4 *tile = (float4 *)(wb + L::tile);
-    float *Dd = (float *)(wb + L::cra) + q * a.capq;
-    uint32_t *Ds = (uint32_t *)(wb + L::cra) + (kGqQ + q) * a.capq;
+    uint32_t *U2 = (uint32_t *)(wb + L::u2), *T0 = (uint32_t *)(wb + L::t0), *T1 = (uint32_t *)(wb + L::t1),
+             *T2 = (uint32_t *)(wb + L::t2);
+    float *Dd = (float *)(wb + L::t0) + q * L::stride(a.capq);                     // the query's entries, bin by bin
+    uint32_t *Ds = (uint32_t *)(wb + L::t0) + (kGqQ + q) * L::stride(a.capq);
     const int k = a.k, n_out = a.nbr_s ? a.n_out : 0;
     unsigned long long cand_acc = 0;
     uint32_t search_acc = 0, retry_acc = 0, warp_acc = 0;
 
     for (;;) {
-        unsigned long long gr = 0;
-        if (lane == 0) gr = atomicAdd(a.group_counter, 1ull);
-        gr = __shfl_sync(kAll, gr, 0);
-        if ((int64_t)gr >= a.n_groups) break;
-        const int64_t ch = (int64_t)gr / a.gpc;
-        int64_t s_first, n_end;
-        float box, norm, R0;
-        const uint32_t *cellT;
-        int level_dense;
+        unsigned long long task = 0;
+        if (lane == 0) task = atomicAdd(a.task_counter, 1ull);
+        task = __shfl_sync(kAll, task, 0);
+        if ((int64_t)task >= a.n_tasks) break;
+        const int per_task = kGqUnit / a.split;
+        uint32_t base, end, s_unit, ch0;
+        float box, norm, plain_r;
         if constexpr (SEG) {
-            const SegDesc &sd = a.seg[seg_of_chunk(a.seg, a.B, ch)];
-            n_end = sd.base + sd.n;
-            s_first = sd.base + ((int64_t)gr - sd.chunk0 * a.gpc) * kGqQ;
+            const SegDesc &sd = a.seg[seg_of_unit(a.seg, a.B, (int64_t)task / a.split)];
+            base = (uint32_t)sd.base;
+            end = (uint32_t)(sd.base + sd.n);
+            s_unit = base + (uint32_t)((int64_t)task - sd.unit0 * a.split) * per_task;
+            ch0 = (uint32_t)sd.chunk0;
             box = (float)sd.box;
             norm = (float)sd.norm;
-            cellT = a.cellT + sd.cell0;
-            level_dense = sd.level_dense;
-            R0 = sd.plain_r;
+            plain_r = sd.plain_r;
         } else {
-            n_end = a.n;
-            s_first = (int64_t)gr * kGqQ;
+            base = 0;
+            end = a.n;
+            s_unit = (uint32_t)task * per_task;
+            ch0 = 0;
             box = a.box;
             norm = a.norm;
-            cellT = a.cellT;
-            level_dense = a.level_dense;
-            R0 = a.plain_r;
+            plain_r = a.plain_r;
         }
-        const int nq = (int)min((int64_t)kGqQ, n_end - s_first);
-        if (nq <= 0) continue;   // the last chunk of a subvolume may hold fewer groups
-        ++warp_acc;
-        if (a.chunk_r) R0 = a.chunk_r[ch];
-        if (!(R0 > 0.f)) R0 = box * 1e-6f;
-        const float half = 0.5f * box;
-        const float eps = box * 9.5367431640625e-7f;
-        const int64_t sq = s_first + min(q, nq - 1);
-        float qx, qy, qz;
+        const int nu = (int)min((int64_t)per_task, (int64_t)end - (int64_t)s_unit);
+        if (nu <= 0) continue;   // the last unit of a subvolume may hold fewer parts
+        // lane i (and i + 16) holds query i of the unit; r4: its group's radius
+        float ux, uy, uz, r4, ru;
         {
-            const float4 v = a.spos[sq];
-            qx = v.x;
-            qy = v.y;
-            qz = v.z;
+            const uint32_t su = s_unit + min(lane & (kGqUnit - 1), nu - 1);
+            const float4 v = a.spos[su];
+            ux = v.x;
+            uy = v.y;
+            uz = v.z;
+            float r;
+            if (a.chunk_r) {
+                r = a.chunk_r[ch0 + (su - base) / (uint32_t)a.qpw];
+            } else {
+                r = gq_plain_radius(a.tree, v, su, base, end, k, plain_r);
+            }
+            if (!(r > 0.f)) r = box * 1e-6f;
+            r = fmaxf(r, __shfl_xor_sync(kAll, r, 1));
+            r4 = fmaxf(r, __shfl_xor_sync(kAll, r, 2));
+            ru = warp_max(r4);
         }
+        int n2u = -1;
+        {
+            Region rg;
+            float x = ux, y = uy, z = uz;
+            if (rg.build(true, x, y, z, ru, box)) n2u = gq_descend(a.tree, rg, base, end, wo + L::u2, wo + L::t2, lane);
+        }
+        for (int g = 0; g < nu; g += kGqQ) {
+        const int nq = min(kGqQ, nu - g);
+        ++warp_acc;
+        const uint32_t sq = s_unit + g + min(q, nq - 1);
+        const float R0 = __shfl_sync(kAll, r4, g);
+        const float qx = __shfl_sync(kAll, ux, g + min(q, nq - 1)), qy = __shfl_sync(kAll, uy, g + min(q, nq - 1)),
+                    qz = __shfl_sync(kAll, uz, g + min(q, nq - 1));
         // a query farther than R0 from the one before it starts a new search
         const float ex = qx - __shfl_up_sync(kAll, qx, 8), ey = qy - __shfl_up_sync(kAll, qy, 8),
                     ez = qz - __shfl_up_sync(kAll, qz, 8);
@@ -386,143 +558,128 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(GqDev a)
             float R = R0;
             int tries = 0;
             for (;;) {
-                // ------------- the region: the members' box, grown by R
-                float flx = quad_min(member ? qx : INFINITY), fhx = quad_max(member ? qx : -INFINITY);
-                float fly = quad_min(member ? qy : INFINITY), fhy = quad_max(member ? qy : -INFINITY);
-                float flz = quad_min(member ? qz : INFINITY), fhz = quad_max(member ? qz : -INFINITY);
-                // where it crosses a face, coordinates >= L/2 move by -L (exact)
-                const bool wx = flx - R < 0.f || fhx + R >= box, wy = fly - R < 0.f || fhy + R >= box,
-                           wz = flz - R < 0.f || fhz + R >= box;
-                const bool mixed = (wx && flx - R < half && half <= fhx + R) || (wy && fly - R < half && half <= fhy + R) ||
-                                   (wz && flz - R < half && half <= fhz + R);
+                // ------------- the 512-particle nodes that meet the region
+                Region rg;
                 float fx = qx, fy = qy, fz = qz;
-                const bool shifted = wx || wy || wz;
-                if (shifted) {
-                    if (wx && qx >= half) fx = qx - box;
-                    if (wy && qy >= half) fy = qy - box;
-                    if (wz && qz >= half) fz = qz - box;
-                    flx = quad_min(member ? fx : INFINITY);
-                    fhx = quad_max(member ? fx : -INFINITY);
-                    fly = quad_min(member ? fy : INFINITY);
-                    fhy = quad_max(member ? fy : -INFINITY);
-                    flz = quad_min(member ? fz : INFINITY);
-                    fhz = quad_max(member ? fz : -INFINITY);
-                }
-                bool give_up = 2.f * R >= half || mixed || tries >= kGqTries;
-                uint32_t total = 0;
-                int nc = 0;
-                if (!give_up) {
-                    // the finest level whose cells have a side of at least R / cells_per_box ...
-                    const float cells = box * a.cells_per_box / R;
-                    int l = min(max((int)((__float_as_uint(cells) >> 23) & 0xFFu) - 127, 1), kMaxLevel);
-                    for (;;) {
-                        nc = gq_cells(flx, fhx, fly, fhy, flz, fhz, R, box, l, cellT, a.keys, level_dense, cra, cpre,
-                                      lane, lt);
-                        if (nc >= 0 || l <= 1) break;
-                        --l;   // too many cells meet the region: take coarser ones
+                int n2 = -1;
+                if (rg.build(member, fx, fy, fz, R, box) && tries < kGqTries) {
+                    if (n2u >= 0 && R <= ru) {
+                        n2 = 0;
+                        for (int i = 0; i < n2u; i += 32) {
+                            bool in = i + lane < n2u;
+                            uint32_t node = 0;
+                            if (in) {
+                                node = U2[i + lane];
+                                in = rg.meets(a.tree.lo[a.tree.off[2] + node], a.tree.hi[a.tree.off[2] + node]);
+                            }
+                            const uint32_t bal = __ballot_sync(kAll, in);
+                            if (in) T2[n2 + __popc(bal & lt)] = node;
+                            n2 += __popc(bal);
+                        }
+                        __syncwarp();
+                    } else {
+                        n2 = gq_descend(a.tree, rg, base, end, wo + L::t2, wo + L::t1, lane);
                     }
-                    give_up = nc < 0;
                 }
-                if (give_up) {
-                    if (member && p == 0) a.hand[atomicAdd(a.hand_n, 1ull)] = (uint32_t)sq;
+                if (n2 < 0) {
+                    if (member && p == 0) a.hand[atomicAdd(a.hand_n, 1ull)] = sq;
                     break;
                 }
-                total = gq_prefix(cpre, nc, lane);
                 ++search_acc;
-                // ------------- stage and evaluate
-                int cnt = 0, m = 0;
+                // ------------- open them and evaluate the runs
+                uint32_t lp = list0;   // the end of the lane's list
                 float tau = member ? R * R : -1.f;
                 bool crowd = false;
-                {
-                    const float lx = flx - eps, hx = fhx + eps, ly = fly - eps, hy = fhy + eps, lz = flz - eps, hz = fhz + eps;
-                    const float r2c = R * R * 1.00001f + box * box * 1e-12f;
-                    const uint32_t upto_lane = lane == 31 ? kAll : ((2u << lane) - 1u);
-                    const int nmem = __popc(__ballot_sync(kAll, member)) >> 3;
-                    int cbase = -1;   // the cell holding particle g - 1
-                    for (uint32_t g = 0; g < total; g += 128) {
-                        uint32_t s[4];
-                        float4 v[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            // the cell of each lane's particle, from the cell
-                            // starts inside the window (one bit each)
-                            const uint32_t w0 = g + 32 * u;
-                            const int j = cbase + 1 + lane;
-                            const uint32_t st = j < nc ? cpre[j] : total;
-                            const uint32_t bit = (st >= w0 && st < w0 + 32) ? 1u << (st - w0) : 0u;
-                            const uint32_t starts = __reduce_or_sync(kAll, bit);
-                            const int c = cbase + __popc(starts & upto_lane);
-                            const uint32_t gi = w0 + (uint32_t)lane;
-                            s[u] = gi < total ? cra[c] + (gi - cpre[c]) : 0xffffffffu;
-                            cbase += __popc(starts);
+                int i2 = 0, i1 = 0, n1 = 0;
+                for (;;) {
+                    int n0 = 0;
+                    // 16 nodes at a time: 512-particle ones while the list
+                    // below has room, then 64-particle ones
+                    bool fill = n1 == 0;
+                    while (n0 <= kGqN0 - 128) {
+                        if (fill && (i2 >= n2 || n1 > kGqN1 - 128)) {
+                            fill = false;
+                            __syncwarp();
                         }
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            v[u] = s[u] != 0xffffffffu ? a.spos[s[u]] : make_float4(INFINITY, 0.f, 0.f, 0.f);
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            float4 c = v[u];
-                            if (shifted) {
-                                if (wx && c.x >= half) c.x -= box;   // the padding's INFINITY stays one
-                                if (wy && c.y >= half) c.y -= box;
-                                if (wz && c.z >= half) c.z -= box;
-                            }
-                            const float gx = fmaxf(fmaxf(lx - c.x, c.x - hx), 0.f);
-                            const float gy = fmaxf(fmaxf(ly - c.y, c.y - hy), 0.f);
-                            const float gz = fmaxf(fmaxf(lz - c.z, c.z - hz), 0.f);
-                            const bool keep = gx * gx + gy * gy + gz * gz <= r2c;
-                            const uint32_t bal = __ballot_sync(kAll, keep);
-                            c.w = __uint_as_float(s[u]);
-                            if (keep) tile[m + __popc(bal & lt)] = c;
-                            m += __popc(bal);
+                        if (!fill && i1 >= n1) {
+                            if (i2 >= n2) break;
+                            fill = true;
+                            i1 = n1 = 0;
+                            __syncwarp();
                         }
-                        const bool last = g + 128 >= total;
-                        if (m <= kGqTile - 128 && !last) continue;
-                        if (last) {
-                            // pad to a multiple of 32 with entries no test accepts
-                            const float nan = __int_as_float(0x7fc00000);
-                            if (lane < ((32 - (m & 31)) & 31)) tile[m + lane] = make_float4(nan, nan, nan, 0.f);
-                            cand_acc += (unsigned long long)m * (unsigned long long)nmem;
-                            m = (m + 31) & ~31;
+                        const int m = gq_open(a.tree, fill ? 1 : 0, rg, fill ? T2 : T1, fill ? i2 : i1, fill ? n2 : n1,
+                                              fill ? T1 : T0, fill ? n1 : n0, lane, lt);
+                        if (fill) {
+                            n1 = m;
+                            i2 += 16;
                         } else {
-                            cand_acc += (unsigned long long)(m & ~31) * (unsigned long long)nmem;
+                            n0 = m;
+                            i1 += 16;
                         }
-                        __syncwarp();
-                        int j0 = 0;
-                        for (; j0 + 32 <= m; j0 += 32) {
+                    }
+                    if (n0 == 0) break;
+                    cand_acc += (unsigned long long)(8 * n0) * (unsigned long long)(__popc(__ballot_sync(kAll, member)) >> 3);
+                    // up to a multiple of four with runs past the last particle
+                    if (lane < 4) T0[n0 + lane] = a.pad_run;
+                    __syncwarp();
+                    const int steps = (n0 + 3) >> 2;
+                    const float4 *sp = a.spos + p;
+                    // step j stages four runs in slot j mod 4 (the histogram's
+                    // space), one particle per lane, three steps ahead
+                    auto fetch = [&](int j) {
+                        if (j < steps) copy16_async(stage_st + (j & 3) * 512, sp + (size_t)(T0[4 * j + q] * 8));
+                        copy_commit();
+                    };
+                    int j = 0;
+                    while (j < steps) {
+                        fetch(j);
+                        fetch(j + 1);
+                        fetch(j + 2);
+                        bool over = false;
+                        for (; j < steps && !over; ++j) {
+                            copy_wait<2>();
+                            __syncwarp();
+                            fetch(j + 3);
+                            const uint4 id = reinterpret_cast<const uint4 *>(T0)[j];
+                            const float4 *st = (const float4 *)(wb + L::hist) + (j & 3) * 32 + p;
+                            float4 c[4] = {st[0], st[8], st[16], st[24]};
+                            if (rg.shifted) {
+                                const float half = 0.5f * box;
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) {
+                                    if (rg.wx && c[u].x >= half) c[u].x -= box;
+                                    if (rg.wy && c[u].y >= half) c[u].y -= box;
+                                    if (rg.wz && c[u].z >= half) c[u].z -= box;
+                                }
+                            }
+                            const uint32_t run[4] = {id.x, id.y, id.z, id.w};
 #pragma unroll
                             for (int u = 0; u < 4; ++u) {
-                                const float4 c = tile[j0 + u * 8 + p];
-                                const float dx = c.x - fx, dy = c.y - fy, dz = c.z - fz;
-                                const float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                                if (d2 <= tau) {
-                                    Ld[cnt * 32] = d2;
-                                    Ls[cnt * 32] = __float_as_uint(c.w);
-                                    ++cnt;
-                                }
+                                const float dx = c[u].x - fx, dy = c[u].y - fy, dz = c[u].z - fz;
+                                float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                                // a run at the end of a subvolume also holds particles of the next
+                                if constexpr (SEG)
+                                    if (run[u] * 8 + p - base >= end - base) d2 = INFINITY;
+                                gq_keep(lp, d2, tau, run[u]);
                             }
-                            if (__any_sync(kAll, cnt > kGqSlots - 4)) {
-                                gq_tighten(Ld, Ls, hist, member && !crowd, cnt, tau, k, lane);
-                                // a list that stays full: a crowd at the limit
-                                const uint32_t f = __ballot_sync(kAll, cnt > kGqSlots - 4);
-                                if ((f >> (q * 8)) & 0xffu) {
-                                    crowd = true;
-                                    cnt = 0;
-                                    tau = -1.f;
-                                }
-                            }
+                            over = __any_sync(kAll, lp > full);
                         }
-                        m -= j0;
-                        if (!last) {
-                            // the remainder moves to the front
-                            float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
-                            if (lane < m) c = tile[j0 + lane];
-                            __syncwarp();
-                            if (lane < m) tile[lane] = c;
-                        }
+                        copy_wait<0>();
                         __syncwarp();
+                        if (over) {
+                            const Tight t = gq_tighten(wo, (int)(lp - list0) >> 8, member && !crowd, tau, k, lane);
+                            lp = list0 + t.cnt * 256;
+                            tau = t.tau;
+                            // a list that stays full: a crowd at the limit
+                            if ((__ballot_sync(kAll, lp > full) >> (q * 8)) & 0xffu) {
+                                crowd = true;
+                                lp = list0;
+                                tau = -1.f;
+                            }
+                        }
                     }
                 }
+                int cnt = (int)(lp - list0) >> 8;
                 // ------------- selection
                 const int tot = oct_sum(cnt);
                 bool ok = member && !crowd && tot >= k;
@@ -532,62 +689,66 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(GqDev a)
                     GqFound f;
                     for (int it = 0;; ++it) {
                         cmax = (int)__reduce_max_sync(kAll, ok ? (unsigned)cnt : 0u);
-                        scale = (float)kGqBins / tau;
-                        f = gq_count<true>(Ld, hist, bst, ok ? cnt : 0, cmax, scale, k, n_out, lane);
-                        const bool full = ok && (int)(f.k & 1023u) > a.capq;
-                        if (!__any_sync(kAll, full)) break;
+                        scale = gq_scale(tau);
+                        f = gq_count<true>(list, ok ? cnt : 0, cmax, hist, bst, scale, k, n_out, lane);
+                        const bool over = ok && (int)(f.k & 1023u) > a.capq;
+                        if (!__any_sync(kAll, over)) break;
                         if (it == 3) {
                             // the bin stays crowded
-                            if (full) {
+                            if (over) {
                                 ok = false;
                                 crowd = true;
                             }
                             break;
                         }
-                        gq_tighten(Ld, Ls, hist, full, cnt, tau, k, lane);
+                        const Tight t = gq_tighten(wo, cnt, over, tau, k, lane);
+                        cnt = t.cnt;
+                        tau = t.tau;
                     }
-                    const int bk = (int)(f.k >> 20), below = (int)((f.k >> 10) & 1023u), upto = ok ? (int)(f.k & 1023u) : 0;
+                    const int bk = ok ? (int)(f.k >> 20) : -1, below = (int)((f.k >> 10) & 1023u),
+                              upto = ok ? (int)(f.k & 1023u) : 0;
+                    uint16_t *col = hist + lane;
+#pragma unroll 2
                     for (int i = 0; i < cmax; ++i) {
-                        if (ok && i < cnt) {
-                            const float v = Ld[i * 32];
-                            const int b = gq_bin(v, scale);
-                            if (b <= bk) {
-                                uint32_t *w = hist + (b >> 1) * 32 + lane;
-                                const uint32_t x = *w;
-                                const int pos = (int)((x >> ((b & 1) * 16)) & 0xffffu);
-                                *w = x + (1u << ((b & 1) * 16));
-                                Dd[pos] = v;
-                                Ds[pos] = Ls[i * 32];
-                            }
+                        const float2 v = list[i * 32];
+                        const int b = gq_bin(v.x, scale);
+                        if (i < cnt && b <= bk) {
+                            const uint32_t pos = col[b * 32];
+                            col[b * 32] = (uint16_t)(pos + 1);
+                            Dd[pos] = v.x;
+                            Ds[pos] = __float_as_uint(v.y) * 8 + p;
                         }
                     }
                     __syncwarp();
-                    // the exact k-th d^2, within its bin
+                    // the exact k-th d^2: the largest of its bin with fewer
+                    // than k smaller entries
                     float vk = -1.f;
+#pragma unroll 1
                     for (int e = below + p; e < upto; e += 8) {
                         const float v = Dd[e];
-                        int l0 = below, le = below;
-                        for (int h = below; h < upto; ++h) {
-                            const float u = Dd[h];
-                            l0 += u < v;
-                            le += u <= v;
-                        }
-                        if (l0 < k && k <= le) vk = v;
+                        int l = below;
+#pragma unroll 2
+                        for (int h = below; h < upto; ++h) l += Dd[h] < v;
+                        if (l < k) vk = fmaxf(vk, v);
                     }
                     __syncwarp();
                     vk = fmaxf(vk, __shfl_xor_sync(kAll, vk, 1));
                     vk = fmaxf(vk, __shfl_xor_sync(kAll, vk, 2));
                     vk = fmaxf(vk, __shfl_xor_sync(kAll, vk, 4));
-                    // density: fixed-point sum of w(2 r / r_k) over entries with d^2 < r_k^2
+                    // density: fixed-point (2^-32) sum of w(2 r / r_k) over
+                    // entries with d^2 < r_k^2; a weight of 1 is one more
+                    // than the conversion's largest value
                     const float rk = sqrtf(vk);
                     const float inv_h = vk > 0.f ? 2.f / rk : 0.f;
                     unsigned long long wsum = 0;
+#pragma unroll 1
                     for (int e = p; e < upto; e += 8) {
                         const float v = Dd[e];
-                        if (v < vk) {
-                            const float w = m4<float>(sqrtf(v) * inv_h);
-                            wsum += (unsigned long long)(w * 4294967296.0f + 0.5f);
-                        }
+                        const float w = m4<float>(sqrtf(v) * inv_h) * 4294967296.0f + 0.5f;
+                        uint32_t u = __float2uint_rz(w);
+                        if (!(v < vk)) u = 0u;
+                        wsum += u;
+                        if (v < vk && w >= 4294967296.0f) wsum += 1u;
                     }
                     __syncwarp();
 #pragma unroll
@@ -609,17 +770,24 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(GqDev a)
                         const int upto_o = ok ? (int)(f.o & 1023u) : 0;
                         const uint16_t *t = bst + q * (kGqBins + 2);
                         uint32_t *row = a.nbr_s + (size_t)sq * a.ld_out;
+#pragma unroll 1
                         for (int e = p; e < upto_o; e += 8) {
                             const float v = Dd[e];
                             const uint32_t se = Ds[e];
                             const int b = gq_bin(v, scale);
                             const int h0 = t[b], h1 = t[b + 1];
-                            int rank = h0;
+                            int rank = h0, same = 0;
+#pragma unroll 2
                             for (int h = h0; h < h1; ++h) {
                                 const float u = Dd[h];
                                 rank += u < v;
-                                if (u == v && h != e)
-                                    rank += __float_as_uint(a.spos[Ds[h]].w) < __float_as_uint(a.spos[se].w);
+                                same += u == v;
+                            }
+                            if (same > 1) {
+                                const uint32_t oe = __float_as_uint(a.spos[se].w);
+#pragma unroll 1
+                                for (int h = h0; h < h1; ++h)
+                                    rank += Dd[h] == v && __float_as_uint(a.spos[Ds[h]].w) < oe;
                             }
                             if (rank < n_out) row[rank] = se;
                         }
@@ -632,10 +800,11 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(GqDev a)
                 // the others: too few within R
                 ++retry_acc;
                 ++tries;
-                const float grow = member ? fmaxf(1.25f, 1.1f * cbrtf((float)k / (float)max(tot, 1))) : 1.25f;
-                R *= fminf(quad_max(grow), 8.f);
+                const float grow = member ? gq_grow(k, tot) : 1.25f;
+                R *= fminf(warp_max(grow), 8.f);
                 __syncwarp();
             }
+        }
         }
     }
     if (lane == 0) {
@@ -649,16 +818,21 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(GqDev a)
 template <bool SEG> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int qpw, int cpr)
 {
     GqDev d;
+    const int rc = box_tree_build(c, (const float4 *)ka.spos, ka.n, &d.tree);
+    if (rc) return rc;
     d.spos = (const float4 *)ka.spos;
-    d.keys = ka.keys;
-    d.cellT = ka.cellT;
-    d.level_dense = ka.level_dense;
-    d.n = ka.n;
-    d.gpc = qpw / kGqQ;
-    d.n_groups = SEG ? ka.n_chunks * d.gpc : (ka.n + kGqQ - 1) / kGqQ;
+    d.n = (uint32_t)ka.n;
+    d.pad_run = (uint32_t)((ka.n + 7) / 8);
+    // a warp takes a whole unit, except where that would leave warps idle:
+    // then a half or a quarter of one (4,913 particles: 461 us whole, 371 us in
+    // quarters)
+    const int64_t units = SEG ? ka.n_units : (ka.n + kGqUnit - 1) / kGqUnit;
+    const int64_t warps = (int64_t)c->num_sms * 16;
+    d.split = units >= 2 * warps ? 1 : units >= warps ? 2 : 4;
+    d.n_tasks = units * d.split;
+    d.qpw = qpw;
     d.box = (float)ka.box;
     d.norm = (float)(ka.box * ka.box * ka.box / ((double)(ka.n_norm > 0 ? ka.n_norm : ka.n) * 3.14159265358979323846));
-    d.cells_per_box = (float)std::min(std::max(cpr, 1), 3);
     d.k = ka.k;
     d.n_out = ka.n_out;
     d.ld_out = ka.ld_out;
@@ -671,19 +845,19 @@ template <bool SEG> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int qpw, int c
     d.dens_s = ka.dens_s;
     d.rk_s = ka.rk_s;
     d.counters = c->d_counters;
-    d.group_counter = c->d_counters + kCntNum;
+    d.task_counter = c->d_counters + kCntNum;
     d.hand_n = c->d_counters + kCntNum + 1;
     d.err = c->d_err;
     d.hand = (uint32_t *)ctx_buf(c, S_KNN_HAND, (size_t)ka.n * sizeof(uint32_t));
     if (!d.hand) return HOP_ENOMEM;
-    HOP_CUDA(c, cudaMemsetAsync(d.group_counter, 0, 3 * sizeof(unsigned long long), c->stream));
+    HOP_CUDA(c, cudaMemsetAsync(d.task_counter, 0, 3 * sizeof(unsigned long long), c->stream));
     const size_t smem = (size_t)GqSmem::total(d.capq) * kGqWarps;
     auto kern = knn_gq_kernel<SEG>;
     HOP_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     HOP_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGqWarps * 32, smem));
     if (per_sm < 1) return ctx_fail(c, HOP_EINVAL, "kNN lists do not fit in shared memory");
-    const int64_t need = (d.n_groups + kGqWarps - 1) / kGqWarps;
+    const int64_t need = (d.n_tasks + kGqWarps - 1) / kGqWarps;
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * c->num_sms, need));
     kern<<<(unsigned)blocks, kGqWarps * 32, smem, c->stream>>>(d);
     HOP_LAUNCH(c);

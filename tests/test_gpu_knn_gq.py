@@ -39,7 +39,7 @@ def _both(hop, pos, qpw=4, cpr=2, ld=16, **kw):
         assert torch.equal(x, y), name
 
 
-@pytest.mark.parametrize("n", [64, 65, 127, 129, 511, 513, 1021, 4095, 4097, 32771])
+@pytest.mark.parametrize("n", [64, 65, 127, 129, 511, 513, 1021, 4095, 4097, 32771, 50021, 100003])
 @pytest.mark.parametrize("qpw", [4, 16])
 def test_counts_around_groups_and_nodes(hop, n, qpw):
     _both(hop, synth.uniform_box(n, 300 + n), qpw=qpw)
@@ -72,3 +72,23 @@ def test_sparse_and_dense_neighbours(hop, cpr):
     pos = synth._wrap_f32(np.concatenate([pos, rng.random((100, 3))]) % 1.0, 1.0)
     for mode in (0, 1):
         _both(hop, pos, cpr=cpr, radius_mode=mode)
+
+
+@pytest.mark.parametrize("qpw", [4, 8, 16])
+@pytest.mark.parametrize("sizes", [(65, 999, 64, 5001), (30011, 513, 70001, 8191)])
+def test_subvolumes_at_odd_offsets(hop, sizes, qpw):
+    """Runs of eight particles that straddle two subvolumes."""
+    boxes = [1.0, 0.25, 3.0, 1.0]
+    pos = np.concatenate([synth._wrap_f32(synth.nfw_box(n, 70 + i)[0].astype(np.float64) * b, b)
+                          for i, (n, b) in enumerate(zip(sizes, boxes))])
+    off = np.concatenate([[0], np.cumsum(sizes)])
+    pos = torch.from_numpy(pos).cuda()
+    out = []
+    for tuning in ((qpw, 2, 0), (8, 1, 4)):
+        hop.apply_tuning(*tuning)
+        try:
+            out.append(hop.hop_run_batch(pos, off, boxes, hopgpu.default_params(), ld_nbr=16))
+        finally:
+            hop.apply_tuning(8, 1, 0)
+    for key in ("dens", "nbr", "group"):
+        assert torch.equal(out[0][key], out[1][key]), key
