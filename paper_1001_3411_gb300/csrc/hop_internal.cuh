@@ -65,6 +65,7 @@ enum Slot {
     S_SUB_C,                            // subhalos: arrays over chains and boundaries
     S_KNN_HAND,                         // queries that the grouped kNN hands over
     S_BOX,                              // bounding boxes over the sorted particles
+    S_MLP_PART,                         // the blocks' shares of a network gradient
     S_COUNT
 };
 

@@ -10,6 +10,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <vector>
 
 namespace {
@@ -17,53 +18,7 @@ namespace {
 constexpr int IN = HOP_MLP_IN, H = HOP_MLP_HID, NP = HOP_MLP_NPARAM;
 constexpr int oW1 = 0, oB1 = H * IN, oW2 = oB1 + H, oB2 = oW2 + H * H, oW3 = oB2 + H, oB3 = oW3 + H;
 static_assert(oB3 + 1 == NP, "parameter layout");
-constexpr int kGradThreads = 64;
-
 __device__ __forceinline__ float bf(const __nv_bfloat16 *w, int i) { return __bfloat162float(w[i]); }
-
-// Forward pass of one sample with weights W (fp32 values of the bf16 copy).
-__device__ __forceinline__ float mlp_forward_one(const float *W, const float *x, float *h1)
-{
-#pragma unroll 4
-    for (int j = 0; j < H; ++j) {
-        float a = W[oB1 + j];
-#pragma unroll
-        for (int f = 0; f < IN; ++f) a = fmaf(W[oW1 + j * IN + f], x[f], a);
-        h1[j] = fmaxf(a, 0.f);
-    }
-    float y = W[oB3];
-    for (int o = 0; o < H; ++o) {
-        float a = W[oB2 + o];
-#pragma unroll
-        for (int i = 0; i < H; ++i) a = fmaf(W[oW2 + o * H + i], h1[i], a);
-        y = fmaf(W[oW3 + o], fmaxf(a, 0.f), y);
-    }
-    return y;
-}
-
-// out[s] = MLP(feat[s]); with lvl != null the output is the search radius
-// side(lvl) * exp(y + margin) instead.
-__global__ void mlp_fwd_kernel(const __nv_bfloat16 *__restrict__ w16, const float *__restrict__ feat,
-                               int64_t m, float *__restrict__ out, const uint8_t *__restrict__ lvl,
-                               double box, float margin)
-{
-    __shared__ float W[NP];
-    for (int i = threadIdx.x; i < NP; i += blockDim.x) W[i] = bf(w16, i);
-    __syncthreads();
-    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < m;
-         s += (int64_t)gridDim.x * blockDim.x) {
-        float x[IN], h1[H];
-#pragma unroll
-        for (int f = 0; f < IN; ++f) x[f] = feat[s * IN + f];
-        const float y = mlp_forward_one(W, x, h1);
-        if (lvl) {
-            const float sd = (float)(box / (double)(1u << lvl[s]));
-            out[s] = sd * expf(y + margin);
-        } else {
-            out[s] = y;
-        }
-    }
-}
 
 // The first radius of every chunk in one pass, 32 chunks per warp: each
 // lane finds its chunk's stencil level and centre cell (the same arithmetic
@@ -225,92 +180,293 @@ radius_kernel(const __nv_bfloat16 *__restrict__ w16, const float4 *__restrict__ 
     }
 }
 
-// Mean-squared-error gradient over a set of samples (idx[] or 0..m-1),
-// scaled by `scale` (1 / batch size).  Each block keeps its samples'
-// activations and back-propagated errors in shared memory and forms its share
-// of every parameter gradient as a sum over those samples, then adds it to
-// the global gradient.
-__global__ void mlp_grad_kernel(const __nv_bfloat16 *__restrict__ w16, const float *__restrict__ feat,
-                                const float *__restrict__ target, const uint32_t *__restrict__ idx,
-                                int64_t m, float scale, float *__restrict__ grad,
-                                double *__restrict__ loss)
+// The network over a set of samples (idx[] or 0..m-1): the outputs (GRAD
+// false), or the mean-squared-error gradient scaled by `scale` (1 / batch
+// size), of which every block writes its share to part[block][NP].
+//
+// A block of 128 threads takes tiles of 128 samples.  Each product is a small
+// GEMM over the tile with an 8 x 8 register tile per thread (og, sg): 16
+// reads of 16 bytes feed 256 FMAs, which is where shared-memory wavefronts
+// (four per read) and the FMA pipe balance; one sample per thread needs a
+// read per FMA.  Rows are padded so that the eight rows (or row parts) that a
+// quarter of a warp reads lie in distinct banks.  The weight gradients stay
+// in registers over all tiles of a block.  Weights are fp32 values of the
+// bf16 copy; everything else is fp32, the blocks' shares are summed in fp64.
+// FP32- and shared-memory-bound: 15.9k multiply-adds per sample forward and
+// backward, 5.9k forward only.  Gradient and predictions of 262,147 samples:
+// 3237 us with one sample per thread (rows 64 apart, every lane in one bank;
+// shares added by atomics), 374 us now, of an FP32 floor of 140 us.
+constexpr int kNetThreads = 128, kNetTile = 128;
+constexpr int kLdX = 28, kLdH = 68;          // row strides: features (padded with a zero), hidden units
+struct NetSmem {
+    float w1[H][kLdX];
+    float w2[H][kLdH];
+    float b1[H], b2[H], w3[H];
+    float x[kNetTile][kLdX];
+    float h1[kNetTile][kLdH];                // h1, then d loss / d pre-activation 1
+    float d2[kNetTile][kLdH];                // d loss / d pre-activation 2 (GRAD only, the last member)
+};
+template <bool GRAD> constexpr size_t net_smem() { return GRAD ? sizeof(NetSmem) : offsetof(NetSmem, d2); }
+
+__device__ __forceinline__ void fma4(float &a, const float4 &u, const float4 &v)
 {
-    extern __shared__ float sm[];
-    float *W = sm;                    // NP
-    float *G = W + NP;                // NP
-    float *X = G + NP;                // T x IN
-    float *H1 = X + kGradThreads * IN;   // T x H
-    float *H2 = H1 + kGradThreads * H;   // T x H
-    float *D2 = H2 + kGradThreads * H;   // T x H  (d loss / d pre-activation 2)
-    float *D1 = D2 + kGradThreads * H;   // T x H  (d loss / d pre-activation 1)
-    float *DY = D1 + kGradThreads * H;   // T
-    const int t = threadIdx.x;
-    for (int i = t; i < NP; i += blockDim.x) { W[i] = bf(w16, i); G[i] = 0.f; }
-    __syncthreads();
-    double lsum = 0.0;
-    for (int64_t base = (int64_t)blockIdx.x * kGradThreads; base < m;
-         base += (int64_t)gridDim.x * kGradThreads) {
-        const int64_t sidx = base + t;
-        const bool valid = sidx < m;
-        const int64_t s = valid ? (idx ? (int64_t)idx[sidx] : sidx) : 0;
-        float *x = X + t * IN, *h1 = H1 + t * H, *h2 = H2 + t * H, *d2 = D2 + t * H, *d1 = D1 + t * H;
-        for (int f = 0; f < IN; ++f) x[f] = valid ? feat[s * IN + f] : 0.f;
-        for (int j = 0; j < H; ++j) {
-            float a = W[oB1 + j];
-            for (int f = 0; f < IN; ++f) a = fmaf(W[oW1 + j * IN + f], x[f], a);
-            h1[j] = fmaxf(a, 0.f);
-        }
-        float y = W[oB3];
-        for (int o = 0; o < H; ++o) {
-            float a = W[oB2 + o];
-            for (int i = 0; i < H; ++i) a = fmaf(W[oW2 + o * H + i], h1[i], a);
-            h2[o] = fmaxf(a, 0.f);
-            y = fmaf(W[oW3 + o], h2[o], y);
-        }
-        const float r = valid ? y - target[s] : 0.f;
-        lsum += (double)r * (double)r * (double)scale;
-        const float dy = 2.f * r * scale;
-        DY[t] = dy;
-        for (int o = 0; o < H; ++o) d2[o] = h2[o] > 0.f ? dy * W[oW3 + o] : 0.f;
-        for (int i = 0; i < H; ++i) {
-            float a = 0.f;
-            for (int o = 0; o < H; ++o) a = fmaf(W[oW2 + o * H + i], d2[o], a);
-            d1[i] = h1[i] > 0.f ? a : 0.f;
-        }
-        __syncthreads();
-        for (int pidx = t; pidx < NP; pidx += blockDim.x) {
-            float acc = 0.f;
-            if (pidx < oB1) {
-                const int j = pidx / IN, f = pidx % IN;
-                for (int u = 0; u < kGradThreads; ++u) acc = fmaf(D1[u * H + j], X[u * IN + f], acc);
-            } else if (pidx < oW2) {
-                const int j = pidx - oB1;
-                for (int u = 0; u < kGradThreads; ++u) acc += D1[u * H + j];
-            } else if (pidx < oB2) {
-                const int o = (pidx - oW2) / H, i = (pidx - oW2) % H;
-                for (int u = 0; u < kGradThreads; ++u) acc = fmaf(D2[u * H + o], H1[u * H + i], acc);
-            } else if (pidx < oW3) {
-                const int o = pidx - oB2;
-                for (int u = 0; u < kGradThreads; ++u) acc += D2[u * H + o];
-            } else if (pidx < oB3) {
-                const int o = pidx - oW3;
-                for (int u = 0; u < kGradThreads; ++u) acc = fmaf(DY[u], H2[u * H + o], acc);
-            } else {
-                for (int u = 0; u < kGradThreads; ++u) acc += DY[u];
-            }
-            G[pidx] += acc;
-        }
-        __syncthreads();
+    a = fmaf(u.x, v.x, a);
+    a = fmaf(u.y, v.y, a);
+    a = fmaf(u.z, v.z, a);
+    a = fmaf(u.w, v.w, a);
+}
+
+template <bool GRAD>
+__global__ void __launch_bounds__(kNetThreads, 2)
+mlp_net_kernel(const __nv_bfloat16 *__restrict__ w16, const float *__restrict__ feat, const float *__restrict__ target,
+               const uint32_t *__restrict__ idx, int64_t m, float scale, float *__restrict__ part,
+               double *__restrict__ loss, float *__restrict__ out, const uint8_t *__restrict__ lvl, double box,
+               float margin)
+{
+    extern __shared__ __align__(16) unsigned char net_raw[];
+    NetSmem &S = *(NetSmem *)net_raw;
+    const int t = threadIdx.x, og = t & 7, sg = t >> 3;   // outputs og + 8 j, samples sg + 16 j
+    for (int i = t; i < H * kLdX; i += kNetThreads) {
+        const int j = i / kLdX, f = i % kLdX;
+        S.w1[j][f] = f < IN ? bf(w16, oW1 + j * IN + f) : 0.f;
     }
-    for (int i = t; i < NP; i += blockDim.x) atomicAdd(&grad[i], G[i]);
-    // block-reduce the loss
-    __shared__ double lred[kGradThreads];
-    lred[t] = lsum;
+    for (int i = t; i < H * H; i += kNetThreads) S.w2[i / H][i % H] = bf(w16, oW2 + i);
+    for (int i = t; i < H; i += kNetThreads) {
+        S.b1[i] = bf(w16, oB1 + i);
+        S.b2[i] = bf(w16, oB2 + i);
+        S.w3[i] = bf(w16, oW3 + i);
+    }
+    const float b3 = bf(w16, oB3);
+    for (int i = t; i < kNetTile; i += kNetThreads) S.x[i][IN] = 0.f;
+    // gradient shares: W2 (8 x 8) and W1 (8 x 4) over half of the samples,
+    // W3, b1 and b2 of the thread's eight units over its samples
+    float g2[8][8], g1[8][4], gw3[8], gb2[8], gb1[8], gb3 = 0.f;
+    double lsum = 0.0;
+    if constexpr (GRAD) {
+#pragma unroll
+        for (int a = 0; a < 8; ++a) {
+#pragma unroll
+            for (int b = 0; b < 8; ++b) g2[a][b] = 0.f;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) g1[a][b] = 0.f;
+            gw3[a] = gb2[a] = gb1[a] = 0.f;
+        }
+    }
+    const int half = t >> 6, u = t & 63, ua = u & 7, ub = u >> 3;   // weight-gradient tiles
+    for (int64_t base = (int64_t)blockIdx.x * kNetTile; base < m; base += (int64_t)gridDim.x * kNetTile) {
+        const int nt = (int)min((int64_t)kNetTile, m - base);
+        __syncthreads();
+        for (int i = t; i < kNetTile * IN; i += kNetThreads) {
+            const int r = i / IN, f = i - r * IN;
+            float v = 0.f;
+            if (r < nt) v = idx ? feat[(int64_t)idx[base + r] * IN + f] : feat[base * IN + i];
+            S.x[r][f] = v;
+        }
+        __syncthreads();
+        float acc[8][8];   // [output][sample]
+        // ---- layer 1
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+            for (int b = 0; b < 8; ++b) acc[a][b] = S.b1[og + 8 * a];
+#pragma unroll 1
+        for (int k = 0; k < kLdX; k += 4) {
+            float4 w[8];
+#pragma unroll
+            for (int a = 0; a < 8; ++a) w[a] = *(const float4 *)&S.w1[og + 8 * a][k];
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                const float4 x = *(const float4 *)&S.x[sg + 16 * b][k];
+#pragma unroll
+                for (int a = 0; a < 8; ++a) fma4(acc[a][b], w[a], x);
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+            for (int b = 0; b < 8; ++b) S.h1[sg + 16 * b][og + 8 * a] = fmaxf(acc[a][b], 0.f);
+        __syncthreads();
+        // ---- layer 2
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+            for (int b = 0; b < 8; ++b) acc[a][b] = S.b2[og + 8 * a];
+#pragma unroll 1
+        for (int k = 0; k < H; k += 4) {
+            float4 w[8];
+#pragma unroll
+            for (int a = 0; a < 8; ++a) w[a] = *(const float4 *)&S.w2[og + 8 * a][k];
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                const float4 x = *(const float4 *)&S.h1[sg + 16 * b][k];
+#pragma unroll
+                for (int a = 0; a < 8; ++a) fma4(acc[a][b], w[a], x);
+            }
+        }
+        // ---- output: the eight lanes of a sample sum their units
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            float y = 0.f;
+#pragma unroll
+            for (int a = 0; a < 8; ++a) {
+                acc[a][b] = fmaxf(acc[a][b], 0.f);
+                y = fmaf(S.w3[og + 8 * a], acc[a][b], y);
+            }
+            y += __shfl_xor_sync(0xffffffffu, y, 1);
+            y += __shfl_xor_sync(0xffffffffu, y, 2);
+            y += __shfl_xor_sync(0xffffffffu, y, 4);
+            y += b3;
+            const int r = sg + 16 * b;
+            if constexpr (!GRAD) {
+                if (og == 0 && r < nt) {
+                    // with lvl: the search radius side(lvl) * exp(y + margin)
+                    if (lvl) y = (float)(box / (double)(1u << lvl[base + r])) * expf(y + margin);
+                    out[base + r] = y;
+                }
+            } else {
+                float e = 0.f;
+                if (r < nt) e = y - target[idx ? (int64_t)idx[base + r] : base + r];
+                const float dy = 2.f * e * scale;
+                if (og == 0) {
+                    lsum += (double)e * (double)e * (double)scale;
+                    gb3 += dy;
+                }
+#pragma unroll
+                for (int a = 0; a < 8; ++a) {
+                    const float d = acc[a][b] > 0.f ? dy * S.w3[og + 8 * a] : 0.f;
+                    gw3[a] = fmaf(dy, acc[a][b], gw3[a]);
+                    gb2[a] += d;
+                    S.d2[r][og + 8 * a] = d;
+                }
+            }
+        }
+        if constexpr (GRAD) {
+            __syncthreads();
+            // ---- W2's gradient: units {4 ua, 32 + 4 ua} .. x {4 ub, 32 + 4 ub} ..
+#pragma unroll 1
+            for (int r = half * (kNetTile / 2); r < (half + 1) * (kNetTile / 2); ++r) {
+                const float4 p = *(const float4 *)&S.d2[r][4 * ua], q = *(const float4 *)&S.d2[r][32 + 4 * ua];
+                const float4 v = *(const float4 *)&S.h1[r][4 * ub], w = *(const float4 *)&S.h1[r][32 + 4 * ub];
+                const float d[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+                const float h[8] = {v.x, v.y, v.z, v.w, w.x, w.y, w.z, w.w};
+#pragma unroll
+                for (int a = 0; a < 8; ++a)
+#pragma unroll
+                    for (int b = 0; b < 8; ++b) g2[a][b] = fmaf(d[a], h[b], g2[a][b]);
+            }
+            // ---- back through W2: units {4 og, 32 + 4 og} .., samples sg + 16 b
+#pragma unroll
+            for (int a = 0; a < 8; ++a)
+#pragma unroll
+                for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
+#pragma unroll 1
+            for (int o = 0; o < H; o += 4) {
+                float4 x[8];
+#pragma unroll
+                for (int b = 0; b < 8; ++b) x[b] = *(const float4 *)&S.d2[sg + 16 * b][o];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const float4 p = *(const float4 *)&S.w2[o + c][4 * og], q = *(const float4 *)&S.w2[o + c][32 + 4 * og];
+                    const float w[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+#pragma unroll
+                    for (int b = 0; b < 8; ++b) {
+                        const float d = c == 0 ? x[b].x : c == 1 ? x[b].y : c == 2 ? x[b].z : x[b].w;
+#pragma unroll
+                        for (int a = 0; a < 8; ++a) acc[a][b] = fmaf(w[a], d, acc[a][b]);
+                    }
+                }
+            }
+            __syncthreads();   // every read of h1 as activations is done
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                float4 *lo = (float4 *)&S.h1[sg + 16 * b][4 * og], *hi = (float4 *)&S.h1[sg + 16 * b][32 + 4 * og];
+                const float4 p = *lo, q = *hi;
+                const float h[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+                float d[8];
+#pragma unroll
+                for (int a = 0; a < 8; ++a) {
+                    d[a] = h[a] > 0.f ? acc[a][b] : 0.f;
+                    gb1[a] += d[a];
+                }
+                *lo = make_float4(d[0], d[1], d[2], d[3]);
+                *hi = make_float4(d[4], d[5], d[6], d[7]);
+            }
+            __syncthreads();
+            // ---- W1's gradient: units {4 ua, 32 + 4 ua} .. x features 4 ub ..
+            if (ub < kLdX / 4) {
+#pragma unroll 1
+                for (int r = half * (kNetTile / 2); r < (half + 1) * (kNetTile / 2); ++r) {
+                    const float4 p = *(const float4 *)&S.h1[r][4 * ua], q = *(const float4 *)&S.h1[r][32 + 4 * ua];
+                    const float4 v = *(const float4 *)&S.x[r][4 * ub];
+                    const float d[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+                    const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int a = 0; a < 8; ++a)
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) g1[a][b] = fmaf(d[a], x[b], g1[a][b]);
+                }
+            }
+        }
+    }
+    if constexpr (GRAD) {
+        // the block's share: the threads' parts meet in shared memory
+        __syncthreads();
+        float *G = &S.h1[0][0];
+        static_assert(sizeof(S.h1) >= sizeof(float) * NP, "a gradient fits the activations' space");
+        for (int i = t; i < NP; i += kNetThreads) G[i] = 0.f;
+        __syncthreads();
+        for (int h = 0; h < 2; ++h) {
+            if (half == h) {
+#pragma unroll
+                for (int a = 0; a < 8; ++a) {
+                    const int ra = (a < 4 ? 4 * ua : 28 + 4 * ua) + a;
+#pragma unroll
+                    for (int b = 0; b < 8; ++b) G[oW2 + ra * H + (b < 4 ? 4 * ub : 28 + 4 * ub) + b] += g2[a][b];
+#pragma unroll
+                    for (int b = 0; b < 4; ++b)
+                        if (4 * ub + b < IN) G[oW1 + ra * IN + 4 * ub + b] += g1[a][b];
+                }
+            }
+            __syncthreads();
+        }
+        // units' sums: the four lanes of a warp that share og, then the warps
+#pragma unroll
+        for (int a = 0; a < 8; ++a) {
+            float v[3] = {gw3[a], gb2[a], gb1[a]};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                v[c] += __shfl_xor_sync(0xffffffffu, v[c], 8);
+                v[c] += __shfl_xor_sync(0xffffffffu, v[c], 16);
+            }
+            if ((t & 31) < 8) {
+                atomicAdd(&G[oW3 + og + 8 * a], v[0]);
+                atomicAdd(&G[oB2 + og + 8 * a], v[1]);
+                atomicAdd(&G[oB1 + (a < 4 ? 4 * og : 28 + 4 * og) + a], v[2]);
+            }
+        }
+        if (og == 0) atomicAdd(&G[oB3], gb3);
+        for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+        if ((t & 31) == 0) atomicAdd(loss, lsum);
+        __syncthreads();
+        for (int i = t; i < NP; i += kNetThreads) part[(int64_t)blockIdx.x * NP + i] = G[i];
+    }
+}
+
+// grad = the sum of the blocks' shares, in fp64: eight warps per 32
+// parameters, each over every eighth share.
+__global__ void __launch_bounds__(256) grad_sum_kernel(const float *__restrict__ part, int blocks, float *__restrict__ grad)
+{
+    __shared__ double s[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
+    double v = 0.0;
+    if (i < NP)
+#pragma unroll 4
+        for (int b = w; b < blocks; b += 8) v += (double)part[(int64_t)b * NP + i];
+    s[w][lane] = v;
     __syncthreads();
-    if (t == 0) {
-        double a = 0.0;
-        for (int u = 0; u < kGradThreads; ++u) a += lred[u];
-        atomicAdd(loss, a);
+    if (w == 0 && i < NP) {
+        for (int k = 1; k < 8; ++k) v += s[k][lane];
+        grad[i] = (float)v;
     }
 }
 
@@ -338,21 +494,38 @@ __global__ void to_bf16_kernel(const float *__restrict__ w, __nv_bfloat16 *__res
         w16[i] = __float2bfloat16_rn(w[i]);
 }
 
-size_t grad_smem_bytes()
+// Blocks of the network kernels: a tile each, as many as are resident (two
+// per SM with gradients, three without).
+int64_t net_blocks(hop_ctx *c, int64_t m, int per_sm)
 {
-    return sizeof(float) * (2 * NP + kGradThreads * IN + 4 * kGradThreads * H + kGradThreads);
+    return std::max<int64_t>(1, std::min<int64_t>((m + kNetTile - 1) / kNetTile, (int64_t)c->num_sms * per_sm));
 }
 
+// grad = the gradient (written whole), *loss += its loss.
 int grad_launch(hop_ctx *c, const float *feat, const float *target, const uint32_t *idx, int64_t m,
                 float scale, float *grad, double *loss)
 {
-    const size_t smem = grad_smem_bytes();
-    HOP_CUDA(c, cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int64_t blocks = (m + kGradThreads - 1) / kGradThreads;
-    blocks = std::min<int64_t>(blocks, (int64_t)c->num_sms * 2);
-    blocks = std::max<int64_t>(blocks, 1);
-    mlp_grad_kernel<<<(unsigned)blocks, kGradThreads, smem, c->stream>>>(
-        (const __nv_bfloat16 *)c->mlp->w16, feat, target, idx, m, scale, grad, loss);
+    const int64_t blocks = net_blocks(c, m, 2);
+    float *part = (float *)ctx_buf(c, S_MLP_PART, (size_t)blocks * NP * sizeof(float));
+    if (!part) return HOP_ENOMEM;
+    constexpr size_t smem = net_smem<true>();
+    HOP_CUDA(c, cudaFuncSetAttribute(mlp_net_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    mlp_net_kernel<true><<<(unsigned)blocks, kNetThreads, smem, c->stream>>>(
+        (const __nv_bfloat16 *)c->mlp->w16, feat, target, idx, m, scale, part, loss, nullptr, nullptr, 1.0, 0.f);
+    HOP_LAUNCH(c);
+    grad_sum_kernel<<<(NP + 31) / 32, 256, 0, c->stream>>>(part, (int)blocks, grad);
+    HOP_LAUNCH(c);
+    return HOP_OK;
+}
+
+// out[s] = MLP(feat[s]); with lvl != null the search radius side(lvl[s]) *
+// exp(MLP + margin) instead.
+int forward_launch(hop_ctx *c, const float *feat, int64_t m, float *out, const uint8_t *lvl, double box, float margin)
+{
+    constexpr size_t smem = net_smem<false>();
+    HOP_CUDA(c, cudaFuncSetAttribute(mlp_net_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    mlp_net_kernel<false><<<(unsigned)net_blocks(c, m, 3), kNetThreads, smem, c->stream>>>(
+        (const __nv_bfloat16 *)c->mlp->w16, feat, nullptr, nullptr, m, 0.f, nullptr, nullptr, out, lvl, box, margin);
     HOP_LAUNCH(c);
     return HOP_OK;
 }
@@ -384,12 +557,7 @@ void mlp_free(hop_ctx *c)
 
 int mlp_forward_dev(hop_ctx *c, const float *feat, int64_t m, float *out)
 {
-    int64_t blocks = std::min<int64_t>((m + 127) / 128, (int64_t)c->num_sms * 8);
-    blocks = std::max<int64_t>(blocks, 1);
-    mlp_fwd_kernel<<<(unsigned)blocks, 128, 0, c->stream>>>((const __nv_bfloat16 *)c->mlp->w16, feat, m,
-                                                           out, nullptr, 1.0, 0.f);
-    HOP_LAUNCH(c);
-    return HOP_OK;
+    return forward_launch(c, feat, m, out, nullptr, 1.0, 0.f);
 }
 
 namespace {
@@ -435,12 +603,7 @@ int mlp_radius(hop_ctx *c, const void *spos, const uint64_t *keys, const uint32_
     int rc = chunk_features(c, spos, keys, cellT, Ld, n, p->pos_is_f64 != 0, p->box, qpw, feat, lvl,
                             nullptr, nullptr);
     if (rc) return rc;
-    int64_t blocks = std::min<int64_t>((nc + 127) / 128, (int64_t)c->num_sms * 8);
-    blocks = std::max<int64_t>(blocks, 1);
-    mlp_fwd_kernel<<<(unsigned)blocks, 128, 0, c->stream>>>((const __nv_bfloat16 *)c->mlp->w16, feat, nc,
-                                                           chunk_r, lvl, p->box, c->mlp->log_margin);
-    HOP_LAUNCH(c);
-    return HOP_OK;
+    return forward_launch(c, feat, nc, chunk_r, lvl, p->box, c->mlp->log_margin);
 }
 
 // Batched pass: features of every chunk (with the cell side of its own
@@ -516,7 +679,6 @@ int hop_mlp_grad(hop_ctx *c, const float *feat, const float *target, int64_t m, 
     HOP_CUDA(c, cudaSetDevice(c->device));
     double *dl = (double *)ctx_buf(c, S_MISC, 256);
     if (!dl) return HOP_ENOMEM;
-    HOP_CUDA(c, cudaMemsetAsync(grad, 0, sizeof(float) * NP, c->stream));
     HOP_CUDA(c, cudaMemsetAsync(dl, 0, sizeof(double), c->stream));
     int rc = grad_launch(c, feat, target, nullptr, m, 1.f / (float)m, grad, dl);
     if (rc) return rc;
@@ -552,7 +714,6 @@ int hop_mlp_train(hop_ctx *c, const float *feat, const float *target, int64_t m,
         HOP_CUDA(c, cudaMemsetAsync(dl, 0, sizeof(double), c->stream));
         for (int64_t b = 0; b < m; b += batch) {
             const int64_t bs = std::min<int64_t>(batch, m - b);
-            HOP_CUDA(c, cudaMemsetAsync(c->mlp->g, 0, sizeof(float) * NP, c->stream));
             // loss of each batch is its mean; weight it by bs/m for the epoch mean
             int rc = grad_launch(c, feat, target, perm + b, bs, 1.f / (float)bs, c->mlp->g, dl);
             if (rc) return rc;
