@@ -71,7 +71,7 @@ __global__ void keys_seg_kernel(const T *__restrict__ pos, int64_t n, const SegD
 
 // Sorted float4 records; with kout set, also the sorted keys without the
 // subvolume field (the Morton key within the particle's own box).  The
-// kSposPad records from n on are NaN (no distance test accepts them), so that
+// kSposPad records from n on are infinite (no distance test accepts them), so that
 // particles can be read in runs of eight without a bound.
 template <typename T>
 __global__ void gather_kernel(const T *__restrict__ pos, const uint32_t *__restrict__ perm,
@@ -79,7 +79,7 @@ __global__ void gather_kernel(const T *__restrict__ pos, const uint32_t *__restr
                               const uint64_t *__restrict__ kin, uint64_t *__restrict__ kout)
 {
     if (blockIdx.x == 0 && threadIdx.x < kSposPad)
-        spos[n + threadIdx.x] = make_rec((T)NAN, (T)NAN, (T)NAN, 0u);
+        spos[n + threadIdx.x] = make_rec((T)INFINITY, (T)INFINITY, (T)INFINITY, 0u);
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
          s += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t p = perm[s];

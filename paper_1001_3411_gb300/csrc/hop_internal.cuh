@@ -19,7 +19,7 @@ constexpr int kMaxLevel = 16;
 constexpr int kMaxDens = 128;    // Ndens limit (search buffer is 4 * Ndens + slack)
 constexpr int kHistBins = 32;    // 1/8-octave bins of d^2 used for selection
 
-constexpr int kSposPad = 16;     // NaN records after the sorted positions (the last run and one past it)
+constexpr int kSposPad = 16;     // infinite records after the sorted positions (the last run and one past it)
 
 // Device error word bits (atomicOr'ed by kernels, read by the host).
 enum : uint32_t {

@@ -13,12 +13,14 @@
 //   2. Boxes, down to eight particles.  Of those, the nodes that meet the
 //      group's box grown by R are opened, then the 64-particle nodes below
 //      them; what is left is a list of runs of eight particles.
-//   3. Evaluation.  Lane p of a query reads particle p of each run, so the
-//      four queries share one 128-byte line; d^2 and sorted index of those
-//      within R go to the lane's own list, one column of a [slot][lane]
-//      array: no two lanes meet in a bank and no ballot is needed.  When a
-//      list is nearly full, the query's limit drops to the upper edge of the
-//      bin holding its Ndens-th entry.
+//   3. Evaluation.  The lanes read 16 runs at a time (four independent
+//      16-byte loads each, the next 16 runs' in flight) and put the particles
+//      within R of the group's box, fewer than half, in a tile in shared
+//      memory.  Lane p of a query takes every eighth of the tile; d^2 and
+//      sorted index of those within R go to the lane's own list, one column
+//      of a [slot][lane] array: no two lanes meet in a bank and no ballot is
+//      needed.  When a list is nearly full, the query's limit drops to the
+//      upper edge of the bin holding its Ndens-th entry.
 //   4. Selection.  A histogram of the query's lists (32 bins linear in d^2,
 //      16-bit counts) places the entries up to the Ndens-th
 //      bin, bin by bin, in one array (a counting sort).  The exact Ndens-th
@@ -31,22 +33,22 @@
 // Ndens-th distance -- it hands over to the warp-per-query kernel
 // (knn_cg.cu), which runs after it over the list of such queries.
 //
-// What bounds it: shared-memory wavefronts (72 % of peak; every run is read
-// by the four queries' lanes, 16 bytes each) and instruction issue (60 % busy
-// at 16 warps per SM, 1.6k warp instructions per particle); DRAM and tensor
-// cores play no part.  Four queries share the walk and the reads that a warp
-// per query repeats for each.  The code is kept small on purpose (loops not
-// unrolled, one call site of what is long, rare parts out of line): at 55 KB
-// instead of 42 KB instruction-cache misses were the largest stall and the
-// 16.8M-particle kNN took 48.3 ms instead of 37.7.  Runs come through
-// cp.async, three steps ahead: with loads into registers the loop held 60
-// register moves per step and took 77 ms.
-// Kernel time, with learned first radius unless stated, against a cell
-// listing per four queries (and a warp per query): 16.8M particles 68.4 ->
-// 37.7 ms (82.1), 64 subvolumes of 22M together 86.2 -> 53.1 ms (111.8), 3M
-// with Ndens = Nhop = 65 (closed form) 15.3 -> 10.2 ms (22.2), 2.1M with the
-// plain radius, whose start is cut to what the boxes show to be enough, 53.8
-// -> 20.5 ms (59.2).
+// What bounds it: instruction issue and shared-memory wavefronts (58 % of
+// issue slots and 66 % of wavefronts at 16 warps per SM, 1.35k warp
+// instructions per particle); DRAM and tensor cores play no part.  Four
+// queries share the walk and the reads that a warp per query repeats for
+// each.  The code is kept small on purpose (loops not unrolled, one call site
+// of what is long, rare parts out of line): at 55 KB instead of 42 KB
+// instruction-cache misses were the largest stall and the 16.8M-particle kNN
+// took 48.3 ms instead of 37.7.  Evaluating every particle of the runs (108
+// per group) straight from cp.async buffers took 37.7 ms where the tile takes
+// 33.6: a 16-byte read costs four wavefronts whether or not the four queries
+// read the same words.
+// Kernel time, with learned first radius unless stated (in brackets a warp
+// per query): 16.8M particles 33.6 ms (82.1), 64 subvolumes of 22M together
+// 46.5 ms (111.8), 3M with Ndens = Nhop = 65 (closed form) 9.2 ms (22.2), 2.1M
+// with the plain radius, whose start is cut to what the boxes show to be
+// enough, 20.4 ms (59.2), 4,913 particles 0.37 ms (0.99).
 //
 // Results equal those of the other kNN kernels bit for bit: the same
 // per-component minimum-image differences, the same fused d^2, the same
@@ -68,6 +70,8 @@ constexpr int kGqN2 = 96;              // 512-particle nodes held
 constexpr int kGqN1 = 192;             // 64-particle nodes held at once
 constexpr int kGqN0 = 256;             // runs of eight particles held at once
 constexpr int kGqBins = 32;            // histogram bins, linear in d^2
+constexpr int kGqCutBins = 16;         // the same for a cut during the search
+constexpr int kGqTile = 144;           // particles staged: 16 runs, and up to 15 left over
 constexpr int kGqTries = 96;
 
 struct GqDev {
@@ -100,9 +104,13 @@ struct GqSmem {
     static constexpr int bst = hist + kGqBins * 64;                 // [kGqQ][kGqBins + 2] u16 bin starts
     static constexpr int u2 = (bst + kGqQ * (kGqBins + 2) * 2 + 15) & ~15;   // the unit's 512-particle nodes
     static constexpr int t0 = u2 + kGqN2 * 4;                       // a search's runs (read 16 bytes at a time) ...
-    static constexpr int t1 = t0 + (kGqN0 + 8) * 4;                 // ... 64-particle nodes ...
+    static constexpr int t1 = t0 + (kGqN0 + 16) * 4;                 // ... 64-particle nodes ...
     static constexpr int t2 = t1 + kGqN1 * 4;                       // ... and 512-particle nodes
-    static constexpr int search_end = t2 + kGqN2 * 4;
+    static constexpr int thist = t2 + kGqN2 * 4;                    // the histogram of a cut during the search
+    static constexpr int search_end = thist + kGqCutBins * 64;
+    // the particles in reach of a batch of runs share the space of hist and bst
+    static constexpr int tile = hist;
+    static_assert(kGqTile * 16 <= u2 - hist, "the tile fits");
     static_assert(t0 % 16 == 0, "runs are read 16 bytes at a time");
     // Row stride of the sorted arrays: 8 mod 32, so that the four queries'
     // lanes (eight consecutive words each) read distinct banks.
@@ -114,28 +122,19 @@ struct GqSmem {
     }
 };
 
-static_assert(kGqBins * 64 == 4 * 512, "the histogram's space holds four steps of four runs");
-
 extern __shared__ __align__(16) unsigned char gq_smem[];
 
 // Shared-memory byte address of an offset into gq_smem.
 __device__ __forceinline__ uint32_t gq_addr(uint32_t o) { return (uint32_t)__cvta_generic_to_shared(gq_smem + o); }
 
-__device__ __forceinline__ void copy16_async(uint32_t dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N> __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-// Appends (d2, run) to the lane's list when d2 <= tau: one predicated store
+// Appends (d2, sorted index) to the lane's list when d2 <= tau: one predicated store
 // and one predicated add.
-__device__ __forceinline__ void gq_keep(uint32_t &lp, float d2, float tau, uint32_t run)
+__device__ __forceinline__ void gq_keep(uint32_t &lp, float d2, float tau, uint32_t s)
 {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.le.f32 p, %1, %2;\n\t@p st.shared.v2.b32 [%0], {%3, %4};\n\t"
                  "@p add.u32 %0, %0, 256;\n\t}"
                  : "+r"(lp)
-                 : "f"(d2), "f"(tau), "r"(__float_as_uint(d2)), "r"(run)
+                 : "f"(d2), "f"(tau), "r"(__float_as_uint(d2)), "r"(s)
                  : "memory");
 }
 
@@ -228,11 +227,32 @@ __device__ __forceinline__ int oct_sum(int v)
 
 // Bin of a d^2 <= tau: the integer part of d^2 * scale, left in the low bits
 // of a float (one instruction, exact product, rounded towards zero); scale
-// keeps it below kGqBins.
-__device__ __forceinline__ float gq_scale(float tau) { return fminf(__fdividef(kGqBins - 0.01f, tau), 5e37f); }
-__device__ __forceinline__ int gq_bin(float d2, float scale)
+// keeps it below BINS.
+template <int BINS> __device__ __forceinline__ float gq_scale(float tau)
 {
-    return (int)(__float_as_uint(__fmaf_rz(d2, scale, 8388608.f)) - 0x4b000000u);
+    return fminf(__fdividef(BINS - 0.01f, tau), 5e37f);
+}
+__device__ __forceinline__ uint32_t gq_bin_bits(float d2, float scale)   // 0x4b000000 + the bin
+{
+    return __float_as_uint(__fmaf_rz(d2, scale, 8388608.f));
+}
+__device__ __forceinline__ int gq_bin(float d2, float scale) { return (int)(gq_bin_bits(d2, scale) - 0x4b000000u); }
+// The address of a lane's 16-bit histogram column, less what gq_bin_bits *
+// 64 adds to the bin's row.
+__device__ __forceinline__ uint32_t gq_column(const uint16_t *hist, int lane)
+{
+    return (uint32_t)__cvta_generic_to_shared(hist) + 2u * (uint32_t)lane - 0x4b000000u * 64u;
+}
+// With `on`, adds one to a lane's histogram entry; returns what it held.
+__device__ __forceinline__ uint32_t gq_next(uint32_t addr, bool on)
+{
+    uint32_t v = 0;
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tsetp.ne.b32 p, %2, 0;\n\t@p ld.shared.u16 %0, [%1];\n\t"
+                 "add.u32 t, %0, 1;\n\t@p st.shared.u16 [%1], t;\n\t}"
+                 : "+r"(v)
+                 : "r"(addr), "r"((int)on)
+                 : "memory");
+    return v;
 }
 // A value that only later bins exceed.
 __device__ __forceinline__ float gq_edge(int bin, float scale) { return __fdividef((float)(bin + 1), scale) * 1.000002f; }
@@ -245,56 +265,56 @@ __device__ __forceinline__ float gq_edge(int bin, float scale) { return __fdivid
 struct GqFound {
     uint32_t k, o;
 };
-template <bool PLACE>
+template <int BINS, bool PLACE>
 __device__ __forceinline__ GqFound gq_count(const float2 *list, int cnt, int cmax, uint16_t *hist,
                                             uint16_t *bst, float scale, int k, int n_out, int lane)
 {
     const int q = lane >> 3, p = lane & 7;
 #pragma unroll
-    for (int i = 0; i < kGqBins * 64 / 512; ++i) reinterpret_cast<uint4 *>(hist)[i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 0; i < BINS * 64 / 512; ++i) reinterpret_cast<uint4 *>(hist)[i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
     __syncwarp();
-    uint16_t *col = hist + lane;
+    const uint32_t col = gq_column(hist, lane);
 #pragma unroll 1
     for (int i = 0; i < cmax; i += 2) {
         // (a column has an even number of slots)
         const float v0 = list[i * 32].x, v1 = list[(i + 1) * 32].x;
-        if (i < cnt) ++col[gq_bin(v0, scale) * 32];
-        if (i + 1 < cnt) ++col[gq_bin(v1, scale) * 32];
+        gq_next(col + gq_bin_bits(v0, scale) * 64, i < cnt);
+        gq_next(col + gq_bin_bits(v1, scale) * 64, i + 1 < cnt);
     }
     __syncwarp();
-    // lane p holds bins p, p + 8, p + 16, p + 24 of its query, each one read
-    // of 16 bytes (the query's eight lanes)
-    uint4 w[4];
-    int t[4], st[4];
+    // lane p holds bins p, p + 8 .. of its query, each one read of 16 bytes
+    // (the query's eight lanes)
+    constexpr int J = BINS / 8;
+    uint4 w[J];
+    int t[J], st[J];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < J; ++j) {
         w[j] = *reinterpret_cast<const uint4 *>(hist + (p + 8 * j) * 32 + q * 8);
         const uint32_t s = w[j].x + w[j].y + w[j].z + w[j].w;
         t[j] = (int)((s & 0xffffu) + (s >> 16));
     }
-    {
-        uint32_t a = (uint32_t)t[0] | ((uint32_t)t[1] << 16), b = (uint32_t)t[2] | ((uint32_t)t[3] << 16);
+    int all = 0;
+#pragma unroll
+    for (int j = 0; j < J; j += 2) {
+        // two bins' prefixes over the lanes at once, 16 bits each
+        uint32_t a = (uint32_t)t[j] | ((uint32_t)t[j + 1] << 16);
 #pragma unroll
         for (int o = 1; o < 8; o <<= 1) {
-            const uint32_t ya = __shfl_up_sync(kAll, a, o, 8), yb = __shfl_up_sync(kAll, b, o, 8);
-            if (p >= o) {
-                a += ya;
-                b += yb;
-            }
+            const uint32_t y = __shfl_up_sync(kAll, a, o, 8);
+            if (p >= o) a += y;
         }
-        const uint32_t sa = __shfl_sync(kAll, a, 7, 8), sb = __shfl_sync(kAll, b, 7, 8);
-        const int n0 = sa & 0xffffu, n1 = n0 + (int)(sa >> 16), n2 = n1 + (int)(sb & 0xffffu);
-        st[0] = (int)(a & 0xffffu) - t[0];
-        st[1] = n0 + (int)(a >> 16) - t[1];
-        st[2] = n1 + (int)(b & 0xffffu) - t[2];
-        st[3] = n2 + (int)(b >> 16) - t[3];
-        if constexpr (PLACE)
-            if (p == 7) bst[q * (kGqBins + 2) + kGqBins] = (uint16_t)(n2 + (int)(sb >> 16));
+        const uint32_t s = __shfl_sync(kAll, a, 7, 8);
+        st[j] = all + (int)(a & 0xffffu) - t[j];
+        all += (int)(s & 0xffffu);
+        st[j + 1] = all + (int)(a >> 16) - t[j + 1];
+        all += (int)(s >> 16);
     }
+    if constexpr (PLACE)
+        if (p == 7) bst[q * (BINS + 2) + BINS] = (uint16_t)all;
     auto find = [&](int rank) {
         uint32_t v = 0;
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < J; ++j)
             if (st[j] < rank && rank <= st[j] + t[j])
                 v = ((uint32_t)(p + 8 * j) << 20) | ((uint32_t)st[j] << 10) | (uint32_t)(st[j] + t[j]);
         const uint32_t m = (__ballot_sync(kAll, v != 0u) >> (q * 8)) & 0xffu;
@@ -306,7 +326,7 @@ __device__ __forceinline__ GqFound gq_count(const float2 *list, int cnt, int cma
     f.o = n_out > 0 ? find(n_out) : 0u;
     if constexpr (PLACE) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
+        for (int j = 0; j < J; ++j) {
             uint32_t r = (uint32_t)st[j];
             auto next = [&](uint32_t x) {
                 const uint32_t out = r * 0x10001u + (x << 16);
@@ -319,7 +339,7 @@ __device__ __forceinline__ GqFound gq_count(const float2 *list, int cnt, int cma
             o.z = next(w[j].z);
             o.w = next(w[j].w);
             *reinterpret_cast<uint4 *>(hist + (p + 8 * j) * 32 + q * 8) = o;
-            bst[q * (kGqBins + 2) + p + 8 * j] = (uint16_t)st[j];
+            bst[q * (BINS + 2) + p + 8 * j] = (uint16_t)st[j];
         }
         __syncwarp();
     }
@@ -337,10 +357,10 @@ struct Tight {
 __device__ __noinline__ Tight gq_tighten(uint32_t wo, int cnt, bool which, float tau, int k, int lane)
 {
     float2 *list = (float2 *)(gq_smem + wo + GqSmem::list) + lane;
-    uint16_t *hist = (uint16_t *)(gq_smem + wo + GqSmem::hist);
+    uint16_t *hist = (uint16_t *)(gq_smem + wo + GqSmem::thist);
     const int cmax = (int)__reduce_max_sync(kAll, which ? (unsigned)cnt : 0u);
-    const float scale = gq_scale(tau);
-    const GqFound f = gq_count<false>(list, which ? cnt : 0, cmax, hist, nullptr, scale, k, 0, lane);
+    const float scale = gq_scale<kGqCutBins>(tau);
+    const GqFound f = gq_count<kGqCutBins, false>(list, which ? cnt : 0, cmax, hist, nullptr, scale, k, 0, lane);
     if (which && f.k) {
         tau = fminf(tau, gq_edge((int)(f.k >> 20), scale));
         int m = 0;
@@ -419,10 +439,8 @@ __device__ __forceinline__ int gq_open(const BoxTree &t, int lv, const Region &r
     for (int u = 0; u < 4; ++u) {
         const int j = i + 4 * u + (lane >> 3);
         node[u] = list[min(j, n - 1)] * 8 + (lane & 7);
-        if (i + 4 * u < n) {
-            l[u] = lo[node[u]];
-            h[u] = hi[node[u]];
-        }
+        l[u] = lo[node[u]];
+        h[u] = hi[node[u]];
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -473,8 +491,8 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
     unsigned char *wb = gq_smem + wo;
     float2 *list = (float2 *)(wb + L::list) + lane;
     const uint32_t list0 = gq_addr(wo + L::list) + lane * 8;
-    const uint32_t full = list0 + (kGqSlots - 4) * 256;   // a list beyond it has no room for four more
-    const uint32_t stage_st = gq_addr(wo + L::hist) + lane * 16;
+    const uint32_t full = list0 + (kGqSlots - 2) * 256;   // a list beyond it has no room for two more
+    float4 *tile = (float4 *)(wb + L::tile);
     uint16_t *hist = (uint16_t *)(wb + L::hist);
     uint16_t *bst = (uint16_t *)(wb + L::bst);
     uint32_t *U2 = (uint32_t *)(wb + L::u2), *T0 = (uint32_t *)(wb + L::t0), *T1 = (uint32_t *)(wb + L::t1),
@@ -590,7 +608,7 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
                 uint32_t lp = list0;   // the end of the lane's list
                 float tau = member ? R * R : -1.f;
                 bool crowd = false;
-                int i2 = 0, i1 = 0, n1 = 0;
+                int i2 = 0, i1 = 0, n1 = 0, cand = 0;
                 for (;;) {
                     int n0 = 0;
                     // 16 nodes at a time: 512-particle ones while the list
@@ -618,67 +636,92 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
                         }
                     }
                     if (n0 == 0) break;
-                    cand_acc += (unsigned long long)(8 * n0) * (unsigned long long)(__popc(__ballot_sync(kAll, member)) >> 3);
-                    // up to a multiple of four with runs past the last particle
-                    if (lane < 4) T0[n0 + lane] = a.pad_run;
+                    // up to a multiple of 16 with runs past the last particle
+                    if (lane < 16) T0[n0 + lane] = a.pad_run;
                     __syncwarp();
-                    const int steps = (n0 + 3) >> 2;
                     const float4 *sp = a.spos + p;
-                    // step j stages four runs in slot j mod 4 (the histogram's
-                    // space), one particle per lane, three steps ahead
-                    auto fetch = [&](int j) {
-                        if (j < steps) copy16_async(stage_st + (j & 3) * 512, sp + (size_t)(T0[4 * j + q] * 8));
-                        copy_commit();
-                    };
-                    int j = 0;
-                    while (j < steps) {
-                        fetch(j);
-                        fetch(j + 1);
-                        fetch(j + 2);
-                        bool over = false;
-                        for (; j < steps && !over; ++j) {
-                            copy_wait<2>();
-                            __syncwarp();
-                            fetch(j + 3);
-                            const uint4 id = reinterpret_cast<const uint4 *>(T0)[j];
-                            const float4 *st = (const float4 *)(wb + L::hist) + (j & 3) * 32 + p;
-                            float4 c[4] = {st[0], st[8], st[16], st[24]};
-                            if (rg.shifted) {
-                                const float half = 0.5f * box;
+                    float4 v[4];
+                    uint32_t run[4];
+                    auto load = [&](int j) {
 #pragma unroll
-                                for (int u = 0; u < 4; ++u) {
-                                    if (rg.wx && c[u].x >= half) c[u].x -= box;
-                                    if (rg.wy && c[u].y >= half) c[u].y -= box;
-                                    if (rg.wz && c[u].z >= half) c[u].z -= box;
-                                }
-                            }
-                            const uint32_t run[4] = {id.x, id.y, id.z, id.w};
+                        for (int u = 0; u < 4; ++u) {
+                            run[u] = T0[j + 4 * u + q] * 8;
+                            v[u] = sp[run[u]];
+                        }
+                    };
+                    load(0);
+                    int m = 0;
+#pragma unroll 1
+                    for (int j = 0; j < n0; j += 16) {
+                        if (rg.shifted) {
+                            const float half = 0.5f * box, bx = rg.wx ? box : 0.f, by = rg.wy ? box : 0.f,
+                                        bz = rg.wz ? box : 0.f;
 #pragma unroll
                             for (int u = 0; u < 4; ++u) {
-                                const float dx = c[u].x - fx, dy = c[u].y - fy, dz = c[u].z - fz;
-                                float d2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                                // a run at the end of a subvolume also holds particles of the next
-                                if constexpr (SEG)
-                                    if (run[u] * 8 + p - base >= end - base) d2 = INFINITY;
-                                gq_keep(lp, d2, tau, run[u]);
+                                if (v[u].x >= half) v[u].x -= bx;
+                                if (v[u].y >= half) v[u].y -= by;
+                                if (v[u].z >= half) v[u].z -= bz;
                             }
-                            over = __any_sync(kAll, lp > full);
                         }
-                        copy_wait<0>();
+                        // a lane's particles in reach of the box go to the tile
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            float4 c = v[u];
+                            const float gx = Region::gap(c.x, c.x, rg.lx, rg.hx), gy = Region::gap(c.y, c.y, rg.ly, rg.hy),
+                                        gz = Region::gap(c.z, c.z, rg.lz, rg.hz);
+                            bool in = gx * gx + gy * gy + gz * gz <= rg.r2c;
+                            // a run at the end of a subvolume also holds particles of the next
+                            if constexpr (SEG) in = in && run[u] + p - base < end - base;
+                            const uint32_t bal = __ballot_sync(kAll, in);
+                            c.w = __uint_as_float(run[u] + p);
+                            if (in) tile[m + __popc(bal & lt)] = c;
+                            m += __popc(bal);
+                        }
+                        const bool last = j + 16 >= n0;
+                        if (!last) load(j + 16);
+                        cand += m & (last ? 0xff : 0xf0);
+                        if (last) {
+                            // up to a multiple of 16 with entries no test accepts
+                            const float nan = __int_as_float(0x7fc00000);
+                            if (lane < ((16 - (m & 15)) & 15)) tile[m + lane] = make_float4(nan, nan, nan, 0.f);
+                            m = (m + 15) & ~15;
+                        }
                         __syncwarp();
-                        if (over) {
-                            const Tight t = gq_tighten(wo, (int)(lp - list0) >> 8, member && !crowd, tau, k, lane);
-                            lp = list0 + t.cnt * 256;
-                            tau = t.tau;
-                            // a list that stays full: a crowd at the limit
-                            if ((__ballot_sync(kAll, lp > full) >> (q * 8)) & 0xffu) {
-                                crowd = true;
-                                lp = list0;
-                                tau = -1.f;
+                        int r = 0;
+                        while (r + 16 <= m) {
+                            bool over = false;
+#pragma unroll 1
+                            for (; r + 16 <= m && !over; r += 16) {
+                                const float4 c = tile[r + p], d = tile[r + 8 + p];
+                                const float cx = c.x - fx, cy = c.y - fy, cz = c.z - fz;
+                                const float dx = d.x - fx, dy = d.y - fy, dz = d.z - fz;
+                                gq_keep(lp, fmaf(cx, cx, fmaf(cy, cy, cz * cz)), tau, __float_as_uint(c.w));
+                                gq_keep(lp, fmaf(dx, dx, fmaf(dy, dy, dz * dz)), tau, __float_as_uint(d.w));
+                                over = __any_sync(kAll, lp > full);
+                            }
+                            if (over) {
+                                __syncwarp();
+                                const Tight t = gq_tighten(wo, (int)(lp - list0) >> 8, member && !crowd, tau, k, lane);
+                                lp = list0 + t.cnt * 256;
+                                tau = t.tau;
+                                // a list that stays full: a crowd at the limit
+                                if ((__ballot_sync(kAll, lp > full) >> (q * 8)) & 0xffu) {
+                                    crowd = true;
+                                    lp = list0;
+                                    tau = -1.f;
+                                }
                             }
                         }
+                        // what is left (fewer than 16) moves to the front
+                        m -= r;
+                        float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (lane < m) c = tile[r + lane];
+                        __syncwarp();
+                        if (lane < m) tile[lane] = c;
                     }
+                    __syncwarp();
                 }
+                cand_acc += (unsigned long long)cand * (unsigned long long)(__popc(__ballot_sync(kAll, member)) >> 3);
                 int cnt = (int)(lp - list0) >> 8;
                 // ------------- selection
                 const int tot = oct_sum(cnt);
@@ -689,8 +732,8 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
                     GqFound f;
                     for (int it = 0;; ++it) {
                         cmax = (int)__reduce_max_sync(kAll, ok ? (unsigned)cnt : 0u);
-                        scale = gq_scale(tau);
-                        f = gq_count<true>(list, ok ? cnt : 0, cmax, hist, bst, scale, k, n_out, lane);
+                        scale = gq_scale<kGqBins>(tau);
+                        f = gq_count<kGqBins, true>(list, ok ? cnt : 0, cmax, hist, bst, scale, k, n_out, lane);
                         const bool over = ok && (int)(f.k & 1023u) > a.capq;
                         if (!__any_sync(kAll, over)) break;
                         if (it == 3) {
@@ -705,18 +748,19 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
                         cnt = t.cnt;
                         tau = t.tau;
                     }
-                    const int bk = ok ? (int)(f.k >> 20) : -1, below = (int)((f.k >> 10) & 1023u),
+                    const int bk = (int)(f.k >> 20), below = (int)((f.k >> 10) & 1023u),
                               upto = ok ? (int)(f.k & 1023u) : 0;
-                    uint16_t *col = hist + lane;
+                    const uint32_t col = gq_column(hist, lane), last_bin = 0x4b000000u + (uint32_t)bk;
+                    const int cnt_ok = ok ? cnt : 0;
 #pragma unroll 2
                     for (int i = 0; i < cmax; ++i) {
                         const float2 v = list[i * 32];
-                        const int b = gq_bin(v.x, scale);
-                        if (i < cnt && b <= bk) {
-                            const uint32_t pos = col[b * 32];
-                            col[b * 32] = (uint16_t)(pos + 1);
+                        const uint32_t b = gq_bin_bits(v.x, scale);
+                        const bool on = i < cnt_ok && b <= last_bin;
+                        const uint32_t pos = gq_next(col + b * 64, on);
+                        if (on) {
                             Dd[pos] = v.x;
-                            Ds[pos] = __float_as_uint(v.y) * 8 + p;
+                            Ds[pos] = __float_as_uint(v.y);
                         }
                     }
                     __syncwarp();
@@ -744,11 +788,11 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
 #pragma unroll 1
                     for (int e = p; e < upto; e += 8) {
                         const float v = Dd[e];
-                        const float w = m4<float>(sqrtf(v) * inv_h) * 4294967296.0f + 0.5f;
-                        uint32_t u = __float2uint_rz(w);
-                        if (!(v < vk)) u = 0u;
-                        wsum += u;
-                        if (v < vk && w >= 4294967296.0f) wsum += 1u;
+                        // m4(), both of its pieces computed
+                        const float x = sqrtf(v) * inv_h, y = 2.f - x;
+                        const float wi = 1.f - 1.5f * x * x + 0.75f * x * x * x, wo_ = 0.25f * y * y * y;
+                        const float w = (x < 1.f ? wi : wo_) * 4294967296.0f + 0.5f;
+                        if (v < vk) wsum += (unsigned long long)__float2uint_rz(w) + (w >= 4294967296.0f ? 1u : 0u);
                     }
                     __syncwarp();
 #pragma unroll
@@ -771,25 +815,37 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
                         const uint16_t *t = bst + q * (kGqBins + 2);
                         uint32_t *row = a.nbr_s + (size_t)sq * a.ld_out;
 #pragma unroll 1
+                        int sum = 0;
                         for (int e = p; e < upto_o; e += 8) {
                             const float v = Dd[e];
-                            const uint32_t se = Ds[e];
                             const int b = gq_bin(v, scale);
                             const int h0 = t[b], h1 = t[b + 1];
-                            int rank = h0, same = 0;
+                            int rank = h0;
 #pragma unroll 2
-                            for (int h = h0; h < h1; ++h) {
-                                const float u = Dd[h];
-                                rank += u < v;
-                                same += u == v;
-                            }
-                            if (same > 1) {
-                                const uint32_t oe = __float_as_uint(a.spos[se].w);
+                            for (int h = h0; h < h1; ++h) rank += Dd[h] < v;
+                            if (rank < n_out) row[rank] = Ds[e];
+                            sum += rank;
+                        }
+                        __syncwarp();
+                        // the ranks are 0 .. upto_o - 1 unless two distances
+                        // are equal; only then rank again, equal ones by index
+                        const bool ties = oct_sum(sum) != upto_o * (upto_o - 1) / 2;
+                        if (__any_sync(kAll, ties)) {
 #pragma unroll 1
-                                for (int h = h0; h < h1; ++h)
-                                    rank += Dd[h] == v && __float_as_uint(a.spos[Ds[h]].w) < oe;
+                            for (int e = p; ties && e < upto_o; e += 8) {
+                                const float v = Dd[e];
+                                const uint32_t se = Ds[e], oe = __float_as_uint(a.spos[se].w);
+                                const int b = gq_bin(v, scale);
+                                const int h0 = t[b], h1 = t[b + 1];
+                                int rank = h0;
+#pragma unroll 1
+                                for (int h = h0; h < h1; ++h) {
+                                    const float u = Dd[h];
+                                    rank += u < v;
+                                    if (u == v) rank += __float_as_uint(a.spos[Ds[h]].w) < oe;
+                                }
+                                if (rank < n_out) row[rank] = se;
                             }
-                            if (rank < n_out) row[rank] = se;
                         }
                     }
                     __syncwarp();
