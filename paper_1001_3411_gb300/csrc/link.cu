@@ -25,7 +25,11 @@ __global__ void dkey_kernel(const float *__restrict__ dens, const uint32_t *__re
     }
 }
 
-// hop_i = argmax of the key over the first n_hop entries of row i.
+// hop_i = argmax of the key over the first n_hop entries of row i.  VEC: rows
+// start on 16 bytes and n_hop is a multiple of four; a thread then reads its
+// row in 16-byte parts, whose keys are gathered independently.  Bound by the
+// gathers (8 bytes each, mostly from L2).
+template <bool VEC>
 __global__ void hop_kernel(const uint64_t *__restrict__ dkey, const uint32_t *__restrict__ nbr,
                            int ld, int64_t n, int n_hop, uint32_t *__restrict__ hop,
                            uint32_t *__restrict__ chain, uint32_t *__restrict__ err)
@@ -33,14 +37,33 @@ __global__ void hop_kernel(const uint64_t *__restrict__ dkey, const uint32_t *__
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t *row = nbr + i * (int64_t)ld;
-        uint32_t best = row[0];
-        bool bad = best >= (uint64_t)n;
-        uint64_t bk = bad ? 0 : dkey[best];
-        for (int t = 1; t < n_hop; ++t) {
-            const uint32_t j = row[t];
-            if (j >= (uint64_t)n) { bad = true; break; }
-            const uint64_t kj = dkey[j];
-            if (kj > bk) { bk = kj; best = j; }
+        uint32_t best = 0;
+        uint64_t bk = 0;
+        bool bad = false;
+        if constexpr (VEC) {
+            const uint4 *r4 = (const uint4 *)row;
+#pragma unroll 4
+            for (int t = 0; t < n_hop / 4; ++t) {
+                const uint4 v = r4[t];
+                const uint32_t j[4] = {v.x, v.y, v.z, v.w};
+                uint64_t kj[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const bool in = j[u] < (uint64_t)n;
+                    bad |= !in;
+                    kj[u] = in ? dkey[j[u]] : 0ull;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if ((t == 0 && u == 0) || kj[u] > bk) { bk = kj[u]; best = j[u]; }
+            }
+        } else {
+            for (int t = 0; t < n_hop; ++t) {
+                const uint32_t j = row[t];
+                if (j >= (uint64_t)n) { bad = true; break; }
+                const uint64_t kj = dkey[j];
+                if (t == 0 || kj > bk) { bk = kj; best = j; }
+            }
         }
         if (bad) {
             atomicOr(err, kErrBadIndex);
@@ -49,6 +72,15 @@ __global__ void hop_kernel(const uint64_t *__restrict__ dkey, const uint32_t *__
         hop[i] = best;
         chain[i] = best;
     }
+}
+
+template <typename... A> void hop_launch(int blocks, cudaStream_t st, const uint64_t *dkey, const uint32_t *nbr, int ld,
+                                         int64_t n, int n_hop, A... a)
+{
+    if (n_hop % 4 == 0 && ld % 4 == 0 && (uintptr_t)nbr % 16 == 0)
+        hop_kernel<true><<<blocks, 256, 0, st>>>(dkey, nbr, ld, n, n_hop, a...);
+    else
+        hop_kernel<false><<<blocks, 256, 0, st>>>(dkey, nbr, ld, n, n_hop, a...);
 }
 
 // Path halving: every pointer moves to its grandparent while walking up.
@@ -272,11 +304,10 @@ __global__ void fill_u64_kernel(uint64_t *p, int64_t n, uint64_t v)
         p[i] = v;
 }
 
+// Results in the caller's order: one value per particle each.
 __global__ void scatter_kernel(const uint32_t *__restrict__ perm, int64_t n,
                                const float *__restrict__ dens_s, float *__restrict__ dens,
                                const int32_t *__restrict__ group_s, int32_t *__restrict__ group,
-                               const uint32_t *__restrict__ nbr_s, int ld_s,
-                               uint32_t *__restrict__ nbr, int ld, int n_cols,
                                const uint32_t *__restrict__ chain_s, uint32_t *__restrict__ chain)
 {
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n;
@@ -285,10 +316,31 @@ __global__ void scatter_kernel(const uint32_t *__restrict__ perm, int64_t n,
         if (dens) dens[o] = dens_s[s];
         if (group) group[o] = group_s[s];
         if (chain) chain[o] = perm[chain_s[s]];
-        if (nbr) {
-            const uint32_t *src = nbr_s + s * (int64_t)ld_s;
-            uint32_t *dst = nbr + (int64_t)o * ld;
-            for (int t = 0; t < n_cols; ++t) dst[t] = perm[src[t]];
+    }
+}
+
+// Neighbour rows in the caller's order, W entries (1 or 4: 16 bytes) per
+// thread, so that a row is read and written by consecutive lanes: HBM-bound
+// where a thread per row touches a sector for every entry.  parts = entries
+// of a row / W, ld_s and ld multiples of W, both arrays on W * 4 bytes.
+template <int W>
+__global__ void scatter_rows_kernel(const uint32_t *__restrict__ perm, int64_t n, const uint32_t *__restrict__ nbr_s,
+                                    int ld_s, uint32_t *__restrict__ nbr, int ld, int parts)
+{
+    const int64_t items = n * parts, stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < items; i += stride) {
+        const int64_t s = items < (int64_t(1) << 32) ? (int64_t)((uint32_t)i / (uint32_t)parts) : i / parts;
+        const int t = (int)(i - s * parts);
+        const uint32_t o = perm[s];
+        if constexpr (W == 4) {
+            uint4 v = reinterpret_cast<const uint4 *>(nbr_s + s * (int64_t)ld_s)[t];
+            v.x = perm[v.x];
+            v.y = perm[v.y];
+            v.z = perm[v.z];
+            v.w = perm[v.w];
+            reinterpret_cast<uint4 *>(nbr + (int64_t)o * ld)[t] = v;
+        } else {
+            nbr[(int64_t)o * ld + t] = perm[nbr_s[s * (int64_t)ld_s + t]];
         }
     }
 }
@@ -320,7 +372,7 @@ int hop_links(hop_ctx *c, const uint64_t *dkey, const uint32_t *nbr, int ld, int
         if (!hop) return HOP_ENOMEM;
     }
     HOP_CUDA(c, cudaMemsetAsync(flag, 0, 8, c->stream));
-    hop_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(dkey, nbr, ld, n, n_hop, hop, chain, flag);
+    hop_launch(grid_for(c, n), c->stream, dkey, nbr, ld, n, n_hop, hop, chain, flag);
     HOP_LAUNCH(c);
     chain_halving_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(chain, n, flag);
     HOP_LAUNCH(c);
@@ -455,7 +507,7 @@ int edges_max_table(hop_ctx *c, const uint64_t *pair, const double *sum, int64_t
 int hop_links_async(hop_ctx *c, const uint64_t *dkey, const uint32_t *nbr, int ld, int64_t n,
                     int n_hop, uint32_t *hop, uint32_t *chain)
 {
-    hop_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(dkey, nbr, ld, n, n_hop, hop, chain, c->d_err);
+    hop_launch(grid_for(c, n), c->stream, dkey, nbr, ld, n, n_hop, hop, chain, c->d_err);
     HOP_LAUNCH(c);
     chain_halving_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(chain, n, c->d_err);
     HOP_LAUNCH(c);
@@ -508,10 +560,21 @@ int scatter_outputs(hop_ctx *c, const uint32_t *perm, int64_t n, const float *de
                     const int32_t *group_s, int32_t *group, const uint32_t *nbr_s, int ld_s,
                     uint32_t *nbr, int ld, int n_cols, const uint32_t *chain_s, uint32_t *chain)
 {
-    scatter_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(perm, n, dens_s, dens, group_s, group,
-                                                         nbr_s, ld_s, nbr, ld, n_cols, chain_s,
-                                                         chain);
-    HOP_LAUNCH(c);
+    if (dens || group || chain) {
+        scatter_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(perm, n, dens_s, dens, group_s, group, chain_s, chain);
+        HOP_LAUNCH(c);
+    }
+    if (nbr && n_cols > 0) {
+        const bool vec = n_cols % 4 == 0 && ld_s % 4 == 0 && ld % 4 == 0 && (uintptr_t)nbr_s % 16 == 0 &&
+                         (uintptr_t)nbr % 16 == 0;
+        const int parts = vec ? n_cols / 4 : n_cols;
+        const int blocks = grid_for(c, n * parts);
+        if (vec)
+            scatter_rows_kernel<4><<<blocks, 256, 0, c->stream>>>(perm, n, nbr_s, ld_s, nbr, ld, parts);
+        else
+            scatter_rows_kernel<1><<<blocks, 256, 0, c->stream>>>(perm, n, nbr_s, ld_s, nbr, ld, parts);
+        HOP_LAUNCH(c);
+    }
     return HOP_OK;
 }
 
@@ -577,7 +640,7 @@ extern "C" int hop_link_static(const float *dens, const uint32_t *nbr, int32_t l
     // the array keeps the previous call's contents: the error word starts at zero
     if (cudaMemsetAsync(flag, 0, 8, st) != cudaSuccess) return HOP_ECUDA;
     dkey_kernel<<<blocks, 256, 0, st>>>(dens, nullptr, n, dkey);
-    hop_kernel<<<blocks, 256, 0, st>>>(dkey, nbr, ld_nbr, n, n_hop, hop, chain, flag);
+    hop_launch(blocks, st, dkey, nbr, ld_nbr, n, n_hop, hop, chain, flag);
     chain_halving_kernel<<<blocks, 256, 0, st>>>(chain, n, flag);
     chain_root_kernel<<<blocks, 256, 0, st>>>(chain, n, flag);
     chain_check_kernel<<<blocks, 256, 0, st>>>(hop, chain, n, flag);
