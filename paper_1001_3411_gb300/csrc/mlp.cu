@@ -20,53 +20,91 @@ constexpr int oW1 = 0, oB1 = H * IN, oW2 = oB1 + H, oB2 = oW2 + H * H, oW3 = oB2
 static_assert(oB3 + 1 == NP, "parameter layout");
 __device__ __forceinline__ float bf(const __nv_bfloat16 *w, int i) { return __bfloat162float(w[i]); }
 
-// The first radius of every chunk in one pass, 32 chunks per warp: each
+// The first radius of every chunk in one pass, 32 chunks per warp.  Each
 // lane finds its chunk's stencil level and centre cell (the same arithmetic
-// as chunk_stencil), the warp looks up the 27 stencil cells of one chunk at
-// a time (27 lanes), and each lane turns its chunk's counts into a radius.
-// NET: the learned radius, R = side * exp(MLP + margin), the network run
-// with its activations in registers.  !NET: the closed form from the
+// as chunk_stencil) and spreads the three coordinates of each axis into
+// Morton bits once.  The 32 x 27 stencil cells are then looked up as one flat
+// list, kRadU independent cells per lane and step: this part is bound by the
+// latency of the table reads and, in halos, of the searches below the dense
+// level, so the searches of a lane's cells advance together.
+// NET: the learned radius, R = side * exp(MLP + margin), the network as two
+// small GEMMs of the warp's 32 chunks (an 8 x 8 register tile per lane, FP32-
+// bound: 184 FMA instructions per chunk).  !NET: the closed form from the
 // stencil total, R = side * cbrt(81 k / (4 pi total)) * exp(margin), the
 // chunk's k-th-neighbour distance if the 27 cells held the mean density of
 // their total.
-// Weights sit in shared memory as fp32 values of the bf16 copy, laid out
-// so that a lane reads four consecutive outputs' weights at once.
+// Measured (one chunk's cells at a time, the network one chunk per lane, in
+// brackets): learned, 4.2M chunks of 16.8M particles 3.06 ms (3.98), issue
+// 52 % busy; closed form, 750k chunks of 3M particles 0.31 ms (0.48).  Nine
+// cells at once gave the same time.
 constexpr int kRadThreads = 128;
 constexpr int kRadWarps = kRadThreads / 32;
-constexpr int kFeatStride = IN + 2;   // 29: lane-strided feature rows hit distinct banks
-static_assert(H % 16 == 0, "hidden width in blocks of 16");
+constexpr int kRadU = 3;              // cells a lane looks up at once
+constexpr int kRadLog = 256;          // log(1 + count) from a table up to this count
+constexpr int kLdX = 28, kLdH = 68;   // row strides: features (padded with a zero), hidden units
+static_assert((27 * 32) % (32 * kRadU) == 0, "whole steps");
 
-struct RadWeights {
-    float w1t[IN][H];   // w1t[f][j] = W1[j][f]
-    float b1[H];
-    float w2t[H][H];    // w2t[i][o] = W2[o][i]
-    float b2[H];
-    float w3[H];
-    float b3;
+struct RadChunk {
+    uint2 code[3][3];     // spread coordinates: axis, offset -1 / 0 / +1
+    int64_t cell0;        // the subvolume's table
+    int l, ld;            // stencil level, dense level
 };
+struct __align__(16) RadWarp {
+    union {
+        RadChunk ch[32];
+        float h[32][kLdH];
+    };
+    float f[32][kLdX];    // log(1 + count); the counts' bits without the network
+};
+struct __align__(16) RadWeights {
+    float w1[H][kLdX], w2[H][kLdH];
+    float b1[H], b2[H], w3[H], b3;
+    float lg[kRadLog];
+};
+// (rows are read 16 bytes at a time)
+static_assert(sizeof(RadWeights) % 16 == 0 && sizeof(RadWarp) % 16 == 0 && offsetof(RadWarp, f) % 16 == 0 &&
+                  offsetof(RadWeights, w2) % 16 == 0 && kLdX % 4 == 0 && kLdH % 4 == 0,
+              "alignment of the rows");
+template <bool NET> constexpr size_t rad_smem()
+{
+    return NET ? sizeof(RadWeights) + kRadWarps * sizeof(RadWarp) : kRadWarps * sizeof(RadWarp);
+}
+
+__device__ __forceinline__ void fma4(float &a, const float4 &u, const float4 &v)
+{
+    a = fmaf(u.x, v.x, a);
+    a = fmaf(u.y, v.y, a);
+    a = fmaf(u.z, v.z, a);
+    a = fmaf(u.w, v.w, a);
+}
 
 template <bool NET>
-__global__ void __launch_bounds__(kRadThreads, 4)
+__global__ void __launch_bounds__(kRadThreads, 3)
 radius_kernel(const __nv_bfloat16 *__restrict__ w16, const float4 *__restrict__ spos,
               const uint64_t *__restrict__ keys, const uint32_t *__restrict__ cellT, int Ld,
               int64_t n, int64_t n_chunks, int Q, float box, float inv_box,
               const SegDesc *__restrict__ seg, int B, float margin, int k, float *__restrict__ chunk_r)
 {
-    __shared__ __align__(16) RadWeights Ws;
-    __shared__ float F[kRadWarps][32][kFeatStride];
-    __shared__ uint32_t T[kRadWarps][32];
+    extern __shared__ __align__(16) unsigned char rad_raw[];
+    RadWeights &W = *(RadWeights *)rad_raw;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    RadWarp &S = *((RadWarp *)(rad_raw + (NET ? sizeof(RadWeights) : 0)) + w);
     if constexpr (NET) {
-        for (int i = threadIdx.x; i < H * IN; i += blockDim.x) Ws.w1t[i % IN][i / IN] = bf(w16, oW1 + i);
-        for (int i = threadIdx.x; i < H * H; i += blockDim.x) Ws.w2t[i % H][i / H] = bf(w16, oW2 + i);
-        for (int i = threadIdx.x; i < H; i += blockDim.x) {
-            Ws.b1[i] = bf(w16, oB1 + i);
-            Ws.b2[i] = bf(w16, oB2 + i);
-            Ws.w3[i] = bf(w16, oW3 + i);
+        for (int i = threadIdx.x; i < H * kLdX; i += kRadThreads) {
+            const int j = i / kLdX, f = i % kLdX;
+            W.w1[j][f] = f < IN ? bf(w16, oW1 + j * IN + f) : 0.f;
         }
-        if (threadIdx.x == 0) Ws.b3 = bf(w16, oB3);
+        for (int i = threadIdx.x; i < H * H; i += kRadThreads) W.w2[i / H][i % H] = bf(w16, oW2 + i);
+        for (int i = threadIdx.x; i < H; i += kRadThreads) {
+            W.b1[i] = bf(w16, oB1 + i);
+            W.b2[i] = bf(w16, oB2 + i);
+            W.w3[i] = bf(w16, oW3 + i);
+        }
+        if (threadIdx.x == 0) W.b3 = bf(w16, oB3);
+        for (int i = threadIdx.x; i < kRadLog; i += kRadThreads) W.lg[i] = log1pf((float)i);
+        S.f[lane][IN] = 0.f;
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t stride = (int64_t)gridDim.x * kRadWarps * 32;
     for (int64_t base = ((int64_t)blockIdx.x * kRadWarps + w) * 32; base < n_chunks; base += stride) {
         const int nc = (int)min((int64_t)32, n_chunks - base);
@@ -100,82 +138,155 @@ radius_kernel(const __nv_bfloat16 *__restrict__ w16, const float4 *__restrict__ 
         while (l > 2 && bx / (float)(1 << l) < ext) --l;
         const int G = 1 << l;
         const float sc = ibx * (float)G;
-        const int cx = min((int)floorf((lx + hx) * 0.5f * sc), G - 1);
-        const int cy = min((int)floorf((ly + hy) * 0.5f * sc), G - 1);
-        const int cz = min((int)floorf((lz + hz) * 0.5f * sc), G - 1);
+        const int c0[3] = {min((int)floorf((lx + hx) * 0.5f * sc), G - 1), min((int)floorf((ly + hy) * 0.5f * sc), G - 1),
+                           min((int)floorf((lz + hz) * 0.5f * sc), G - 1)};
         const float side = (float)((double)bx / (double)G);
-        // ---- the 27 stencil counts of each chunk, one chunk at a time
-        const int dx = lane % 3 - 1, dy = (lane / 3) % 3 - 1, dz = lane / 9 - 1;
-        for (int j = 0; j < nc; ++j) {
-            const int lj = __shfl_sync(0xffffffffu, l, j), ldj = __shfl_sync(0xffffffffu, ld, j);
-            const int xj = __shfl_sync(0xffffffffu, cx, j), yj = __shfl_sync(0xffffffffu, cy, j),
-                      zj = __shfl_sync(0xffffffffu, cz, j);
-            const int64_t c0 = __shfl_sync(0xffffffffu, cell0, j);
-            uint32_t cnt = 0;
-            if (lane < IN) {
-                const int Gj = 1 << lj;
-                const int rx = (xj + dx + Gj) % Gj, ry = (yj + dy + Gj) % Gj, rz = (zj + dz + Gj) % Gj;
-                uint32_t a, b;
-                cell_range(cellT + c0, keys, ldj, lj, morton3((uint32_t)rx, (uint32_t)ry, (uint32_t)rz), a, b);
-                cnt = b - a;
-                if constexpr (NET) F[w][j][lane] = log1pf((float)cnt);
+        {
+            RadChunk &c = S.ch[lane];
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    const uint32_t x = (uint32_t)(c0[a] + d - 1) & (uint32_t)(G - 1);
+                    c.code[a][d] = make_uint2(spread3_8(x) << a, spread3_8(x >> 8) << a);
+                }
+            c.cell0 = cell0;
+            c.l = l;
+            c.ld = ld;
+        }
+        __syncwarp();
+        // ---- the stencil counts, kRadU cells per lane and step
+#pragma unroll 1
+        for (int i0 = 0; i0 < 27 * 32; i0 += 32 * kRadU) {
+            uint32_t a[kRadU], b[kRadU], ha[kRadU], hb[kRadU];
+            uint64_t k0[kRadU], k1[kRadU];
+            int cj[kRadU], cc[kRadU];
+#pragma unroll
+            for (int u = 0; u < kRadU; ++u) {
+                const int i = i0 + 32 * u + lane;
+                cj[u] = i / 27;
+                cc[u] = i - 27 * cj[u];
+                const RadChunk &c = S.ch[cj[u]];
+                const int dz = cc[u] / 9, r = cc[u] - 9 * dz, dy = r / 3, dx = r - 3 * dy;
+                const uint2 x = c.code[0][dx], y = c.code[1][dy], z = c.code[2][dz];
+                const uint64_t code = ((uint64_t)(x.y | y.y | z.y) << 24) | (x.x | y.x | z.x);
+                const uint32_t *t = cellT + c.cell0;
+                const int up = 3 * (c.l - c.ld);
+                if (up <= 0) {
+                    a[u] = t[code << -up];
+                    b[u] = t[(code + 1) << -up];
+                    ha[u] = a[u];
+                    hb[u] = b[u];
+                    k0[u] = k1[u] = 0;
+                } else {
+                    // below the dense level: first keys >= k0 and >= k1 in the
+                    // dense cell's range
+                    const uint64_t pc = code >> up;
+                    const int ksh = 3 * (kMaxLevel - c.l);
+                    a[u] = b[u] = t[pc];
+                    ha[u] = hb[u] = t[pc + 1];
+                    k0[u] = code << ksh;
+                    k1[u] = (code + 1) << ksh;
+                }
             }
-            if constexpr (!NET) {
-                const uint32_t tot = __reduce_add_sync(0xffffffffu, cnt);
-                if (lane == 0) T[w][j] = tot;
+            for (;;) {
+                bool more = false;
+                uint64_t x[kRadU], y[kRadU];
+#pragma unroll
+                for (int u = 0; u < kRadU; ++u) {
+                    x[u] = y[u] = 0;
+                    if (a[u] < ha[u]) x[u] = keys[(a[u] + ha[u]) >> 1];
+                    if (b[u] < hb[u]) y[u] = keys[(b[u] + hb[u]) >> 1];
+                }
+#pragma unroll
+                for (int u = 0; u < kRadU; ++u) {
+                    if (a[u] < ha[u]) {
+                        const uint32_t m = (a[u] + ha[u]) >> 1;
+                        if (x[u] < k0[u]) a[u] = m + 1; else ha[u] = m;
+                    }
+                    if (b[u] < hb[u]) {
+                        const uint32_t m = (b[u] + hb[u]) >> 1;
+                        if (y[u] < k1[u]) b[u] = m + 1; else hb[u] = m;
+                    }
+                    more = more || a[u] < ha[u] || b[u] < hb[u];
+                }
+                if (!__any_sync(0xffffffffu, more)) break;
+            }
+#pragma unroll
+            for (int u = 0; u < kRadU; ++u) {
+                const uint32_t cnt = b[u] - a[u];
+                if constexpr (NET)
+                    S.f[cj[u]][cc[u]] = cnt < (uint32_t)kRadLog ? W.lg[cnt] : log1pf((float)cnt);
+                else
+                    S.f[cj[u]][cc[u]] = __uint_as_float(cnt);
             }
         }
         __syncwarp();
         if constexpr (!NET) {
             if (lane < nc) {
-                const double r = (double)side * cbrt(81.0 * k / (4.0 * 3.14159265358979323846 * (double)max(T[w][lane], 1u)));
+                uint32_t tot = 0;
+                for (int c = 0; c < IN; ++c) tot += __float_as_uint(S.f[lane][c]);
+                const double r = (double)side * cbrt(81.0 * k / (4.0 * 3.14159265358979323846 * (double)max(tot, 1u)));
                 chunk_r[base + lane] = (float)(r * exp((double)margin));
             }
             __syncwarp();
             continue;
         }
-        // ---- the network for the lane's chunk
-        if (lane < nc) {
-            const float *x = F[w][lane];
-            float h[H];
+        // ---- the network: outputs og + 8 a, chunks sg + 4 b
+        const int og = lane & 7, sg = lane >> 3;
+        float acc[8][8];
 #pragma unroll
-            for (int j = 0; j < H; ++j) h[j] = Ws.b1[j];
-            for (int f = 0; f < IN; ++f) {
-                const float xf = x[f];
-                const float4 *r = (const float4 *)Ws.w1t[f];
+        for (int a = 0; a < 8; ++a)
 #pragma unroll
-                for (int j4 = 0; j4 < H / 4; ++j4) {
-                    const float4 wv = r[j4];
-                    h[4 * j4 + 0] = fmaf(wv.x, xf, h[4 * j4 + 0]);
-                    h[4 * j4 + 1] = fmaf(wv.y, xf, h[4 * j4 + 1]);
-                    h[4 * j4 + 2] = fmaf(wv.z, xf, h[4 * j4 + 2]);
-                    h[4 * j4 + 3] = fmaf(wv.w, xf, h[4 * j4 + 3]);
-                }
+            for (int b = 0; b < 8; ++b) acc[a][b] = W.b1[og + 8 * a];
+#pragma unroll 1
+        for (int kk = 0; kk < kLdX; kk += 4) {
+            float4 wv[8];
+#pragma unroll
+            for (int a = 0; a < 8; ++a) wv[a] = *(const float4 *)&W.w1[og + 8 * a][kk];
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                const float4 x = *(const float4 *)&S.f[sg + 4 * b][kk];
+#pragma unroll
+                for (int a = 0; a < 8; ++a) fma4(acc[a][b], wv[a], x);
             }
-#pragma unroll
-            for (int j = 0; j < H; ++j) h[j] = fmaxf(h[j], 0.f);
-            float y = Ws.b3;
-            for (int ob = 0; ob < H; ob += 16) {
-                float acc[16];
-#pragma unroll
-                for (int m = 0; m < 16; ++m) acc[m] = Ws.b2[ob + m];
-#pragma unroll
-                for (int i = 0; i < H; ++i) {
-                    const float4 *r = (const float4 *)&Ws.w2t[i][ob];
-#pragma unroll
-                    for (int k4 = 0; k4 < 4; ++k4) {
-                        const float4 wv = r[k4];
-                        acc[4 * k4 + 0] = fmaf(wv.x, h[i], acc[4 * k4 + 0]);
-                        acc[4 * k4 + 1] = fmaf(wv.y, h[i], acc[4 * k4 + 1]);
-                        acc[4 * k4 + 2] = fmaf(wv.z, h[i], acc[4 * k4 + 2]);
-                        acc[4 * k4 + 3] = fmaf(wv.w, h[i], acc[4 * k4 + 3]);
-                    }
-                }
-#pragma unroll
-                for (int m = 0; m < 16; ++m) y = fmaf(Ws.w3[ob + m], fmaxf(acc[m], 0.f), y);
-            }
-            chunk_r[base + lane] = side * expf(y + margin);
         }
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+            for (int b = 0; b < 8; ++b) S.h[sg + 4 * b][og + 8 * a] = fmaxf(acc[a][b], 0.f);
+        __syncwarp();
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+#pragma unroll
+            for (int b = 0; b < 8; ++b) acc[a][b] = W.b2[og + 8 * a];
+#pragma unroll 1
+        for (int kk = 0; kk < H; kk += 4) {
+            float4 wv[8];
+#pragma unroll
+            for (int a = 0; a < 8; ++a) wv[a] = *(const float4 *)&W.w2[og + 8 * a][kk];
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                const float4 x = *(const float4 *)&S.h[sg + 4 * b][kk];
+#pragma unroll
+                for (int a = 0; a < 8; ++a) fma4(acc[a][b], wv[a], x);
+            }
+        }
+        // lane (og, sg) ends with the output of chunk sg + 4 og
+        float out = 0.f;
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            float y = 0.f;
+#pragma unroll
+            for (int a = 0; a < 8; ++a) y = fmaf(W.w3[og + 8 * a], fmaxf(acc[a][b], 0.f), y);
+            y += __shfl_xor_sync(0xffffffffu, y, 1);
+            y += __shfl_xor_sync(0xffffffffu, y, 2);
+            y += __shfl_xor_sync(0xffffffffu, y, 4);
+            if (og == b) out = y;
+        }
+        const int mine = sg + 4 * og;
+        const float sd = __shfl_sync(0xffffffffu, side, mine);
+        if (mine < nc) chunk_r[base + mine] = sd * expf(out + W.b3 + margin);
         __syncwarp();
     }
 }
@@ -197,7 +308,6 @@ radius_kernel(const __nv_bfloat16 *__restrict__ w16, const float4 *__restrict__ 
 // 3237 us with one sample per thread (rows 64 apart, every lane in one bank;
 // shares added by atomics), 374 us now, of an FP32 floor of 140 us.
 constexpr int kNetThreads = 128, kNetTile = 128;
-constexpr int kLdX = 28, kLdH = 68;          // row strides: features (padded with a zero), hidden units
 struct NetSmem {
     float w1[H][kLdX];
     float w2[H][kLdH];
@@ -206,15 +316,10 @@ struct NetSmem {
     float h1[kNetTile][kLdH];                // h1, then d loss / d pre-activation 1
     float d2[kNetTile][kLdH];                // d loss / d pre-activation 2 (GRAD only, the last member)
 };
+static_assert(offsetof(NetSmem, w2) % 16 == 0 && offsetof(NetSmem, x) % 16 == 0 && offsetof(NetSmem, h1) % 16 == 0 &&
+                  offsetof(NetSmem, d2) % 16 == 0,
+              "alignment of the rows");
 template <bool GRAD> constexpr size_t net_smem() { return GRAD ? sizeof(NetSmem) : offsetof(NetSmem, d2); }
-
-__device__ __forceinline__ void fma4(float &a, const float4 &u, const float4 &v)
-{
-    a = fmaf(u.x, v.x, a);
-    a = fmaf(u.y, v.y, a);
-    a = fmaf(u.z, v.z, a);
-    a = fmaf(u.w, v.w, a);
-}
 
 template <bool GRAD>
 __global__ void __launch_bounds__(kNetThreads, 2)
@@ -562,15 +667,20 @@ int mlp_forward_dev(hop_ctx *c, const float *feat, int64_t m, float *out)
 
 namespace {
 
-int radius_fused(hop_ctx *c, const void *spos, const uint64_t *keys, const uint32_t *cellT, int Ld,
-                 int64_t n, int64_t n_chunks, int qpw, double box, const SegDesc *seg, int B, float *chunk_r)
+template <bool NET>
+int radius_launch(hop_ctx *c, const void *spos, const uint64_t *keys, const uint32_t *cellT, int Ld, int64_t n,
+                  int64_t n_chunks, int qpw, double box, const SegDesc *seg, int B, int k, float margin, float *chunk_r)
 {
+    constexpr size_t smem = rad_smem<NET>();
+    HOP_CUDA(c, cudaFuncSetAttribute(radius_kernel<NET>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    HOP_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, radius_kernel<NET>, kRadThreads, smem));
     int64_t blocks = (n_chunks + kRadThreads - 1) / kRadThreads;
-    blocks = std::min<int64_t>(blocks, (int64_t)c->num_sms * 4);
+    blocks = std::min<int64_t>(blocks, (int64_t)c->num_sms * std::max(per_sm, 1));
     blocks = std::max<int64_t>(blocks, 1);
-    radius_kernel<true><<<(unsigned)blocks, kRadThreads, 0, c->stream>>>(
-        (const __nv_bfloat16 *)c->mlp->w16, (const float4 *)spos, keys, cellT, Ld, n, n_chunks, qpw,
-        (float)box, (float)(1.0 / box), seg, B, c->mlp->log_margin, 0, chunk_r);
+    radius_kernel<NET><<<(unsigned)blocks, kRadThreads, smem, c->stream>>>(
+        NET ? (const __nv_bfloat16 *)c->mlp->w16 : nullptr, (const float4 *)spos, keys, cellT, Ld, n, n_chunks, qpw,
+        (float)box, (float)(1.0 / box), seg, B, margin, k, chunk_r);
     HOP_LAUNCH(c);
     return HOP_OK;
 }
@@ -582,21 +692,14 @@ int radius_closed(hop_ctx *c, const void *spos, const uint64_t *keys, const uint
                   int64_t n_chunks, int qpw, double box, const SegDesc *seg, int B, int k, float log_margin,
                   float *chunk_r)
 {
-    int64_t blocks = (n_chunks + kRadThreads - 1) / kRadThreads;
-    blocks = std::min<int64_t>(blocks, (int64_t)c->num_sms * 4);
-    blocks = std::max<int64_t>(blocks, 1);
-    radius_kernel<false><<<(unsigned)blocks, kRadThreads, 0, c->stream>>>(
-        nullptr, (const float4 *)spos, keys, cellT, Ld, n, n_chunks, qpw, (float)box, (float)(1.0 / box), seg, B,
-        log_margin, k, chunk_r);
-    HOP_LAUNCH(c);
-    return HOP_OK;
+    return radius_launch<false>(c, spos, keys, cellT, Ld, n, n_chunks, qpw, box, seg, B, k, log_margin, chunk_r);
 }
 
 int mlp_radius(hop_ctx *c, const void *spos, const uint64_t *keys, const uint32_t *cellT, int Ld,
                int64_t n, const hop_params *p, int qpw, float *chunk_r)
 {
     const int64_t nc = (n + qpw - 1) / qpw;
-    if (!p->pos_is_f64) return radius_fused(c, spos, keys, cellT, Ld, n, nc, qpw, p->box, nullptr, 0, chunk_r);
+    if (!p->pos_is_f64) return radius_launch<true>(c, spos, keys, cellT, Ld, n, nc, qpw, p->box, nullptr, 0, 0, c->mlp->log_margin, chunk_r);
     float *feat = (float *)ctx_buf(c, S_MLP_TMP, nc * IN * sizeof(float));
     uint8_t *lvl = (uint8_t *)ctx_buf(c, S_CHUNK_LVL, nc);
     if (!feat || !lvl) return HOP_ENOMEM;
@@ -613,7 +716,7 @@ int mlp_radius_seg(hop_ctx *c, const void *spos, const uint64_t *keys, const uin
 {
     if (!c->mlp->loaded) return ctx_fail(c, HOP_ENOMODEL, "no radius network loaded (hop_mlp_load)");
     (void)k;
-    return radius_fused(c, spos, keys, cellT, 0, 0, n_chunks, qpw, 1.0, seg, B, chunk_r);
+    return radius_launch<true>(c, spos, keys, cellT, 0, 0, n_chunks, qpw, 1.0, seg, B, 0, c->mlp->log_margin, chunk_r);
 }
 
 extern "C" {
