@@ -65,6 +65,7 @@ enum Slot {
     S_SUB_C,                            // subhalos: arrays over chains and boundaries
     S_KNN_HAND,                         // queries that the grouped kNN hands over
     S_BOX,                              // bounding boxes over the sorted particles
+    S_SPOS_F,                           // sorted float64 positions rounded to float32
     S_MLP_PART,                         // the blocks' shares of a network gradient
     S_COUNT
 };
@@ -435,9 +436,11 @@ struct KnnArgs {
 };
 int knn_launch(hop_ctx *c, const KnnArgs &a, bool f64, int qpw, int cpr);
 int knn32_launch(hop_ctx *c, const KnnArgs &a, int cpr);   // knn32.cu: one query per lane, float32
-// knn_gq.cu: float32, radius chunks of 4, 8 or 16 queries; four queries per
-// warp, the ones it does not take handed over to knn_wq_launch
-int knn_gq_launch(hop_ctx *c, const KnnArgs &a, int qpw, int cpr);
+// knn_gq.cu: four queries per warp, the ones it does not take handed over to knn_wq_launch
+// (float64: to knn_hand_f64_launch, knn.cu)
+int knn_gq_launch(hop_ctx *c, const KnnArgs &a, bool f64, int qpw, int cpr);
+int knn_hand_f64_launch(hop_ctx *c, const KnnArgs &a, int qpw, int cpr, const uint32_t *hand,
+                        const unsigned long long *hand_n, unsigned long long *counter);
 // knn_cg.cu: one warp per query, over a list of *hand_n sorted indices;
 // `counter` is a device word that is zero on entry
 int knn_wq_launch(hop_ctx *c, const KnnArgs &a, int qpw, int cpr, const uint32_t *hand,

@@ -464,6 +464,9 @@ template <typename T> struct KnnDev {
     unsigned long long *chunk_counter;
     unsigned long long *counters;
     uint32_t *err;
+    const uint32_t *hand;               // when set: the queries (sorted index), one per warp ...
+    const unsigned long long *hand_n;   // ... their number ...
+    int qpw;                            // ... and the queries per radius chunk
 };
 
 // Shared-memory layout of one warp (byte offsets), used by kernel and host.
@@ -535,8 +538,8 @@ __global__ void __launch_bounds__(kKnnThreads, 4) knn_kernel(KnnDev<T> a)
         unsigned long long ch = 0;
         if (lane == 0) ch = atomicAdd(a.chunk_counter, 1ull);
         ch = __shfl_sync(FULL, ch, 0);
-        if ((int64_t)ch >= a.n_chunks) break;
-        ++warp_acc;
+        if ((int64_t)ch >= (a.hand ? (int64_t)*a.hand_n : a.n_chunks)) break;
+        if (!a.hand) ++warp_acc;
         int64_t s_first, n_end, seg_base;
         T box, half, inv_box, norm;
         const uint32_t *cellT;
@@ -557,7 +560,7 @@ __global__ void __launch_bounds__(kKnnThreads, 4) knn_kernel(KnnDev<T> a)
         } else {
             seg_base = 0;
             n_end = a.n;
-            s_first = (int64_t)ch * Q;
+            s_first = a.hand ? (int64_t)a.hand[ch] : (int64_t)ch * Q;
             box = a.box;
             half = a.half_box;
             inv_box = a.inv_box;
@@ -578,7 +581,7 @@ __global__ void __launch_bounds__(kKnnThreads, 4) knn_kernel(KnnDev<T> a)
         }
         __syncwarp();
 
-        T R = a.chunk_r ? (T)a.chunk_r[ch] : (T)plain_r;
+        T R = a.chunk_r ? (T)a.chunk_r[a.hand ? s_first / a.qpw : (int64_t)ch] : (T)plain_r;
         if (!(R > T(0))) R = box * T(1e-6);
         T tau = R * R;
         int cnt = 0;
@@ -1054,7 +1057,9 @@ __global__ void __launch_bounds__(kKnnThreads, 4) knn_kernel(KnnDev<T> a)
 
 template <typename T, int P> size_t knn_smem_per_warp(int buf) { return WarpSmem<T, P>::total(buf); }
 
-template <typename T, int P, bool SEG> int knn_run(hop_ctx *c, const KnnArgs &a, int cpr)
+template <typename T, int P, bool SEG>
+int knn_run(hop_ctx *c, const KnnArgs &a, int cpr, const uint32_t *hand = nullptr,
+            const unsigned long long *hand_n = nullptr, unsigned long long *counter = nullptr, int qpw = 1)
 {
     constexpr int Q = 32 / P;
     KnnDev<T> d;
@@ -1085,9 +1090,12 @@ template <typename T, int P, bool SEG> int knn_run(hop_ctx *c, const KnnArgs &a,
     d.dens_s = a.dens_s;
     d.rk_s = a.rk_s;
     d.counters = c->d_counters;
-    d.chunk_counter = c->d_counters + kCntNum;
+    d.chunk_counter = hand ? counter : c->d_counters + kCntNum;
     d.err = c->d_err;
-    HOP_CUDA(c, cudaMemsetAsync(d.chunk_counter, 0, sizeof(unsigned long long), c->stream));
+    d.hand = hand;
+    d.hand_n = hand_n;
+    d.qpw = qpw;
+    if (!hand) HOP_CUDA(c, cudaMemsetAsync(d.chunk_counter, 0, sizeof(unsigned long long), c->stream));
     // as many warps per block (4, 2 or 1) as fit in the opt-in shared memory
     int max_smem = 0;
     HOP_CUDA(c, cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
@@ -1113,6 +1121,12 @@ template <typename T, int P, bool SEG> int knn_run(hop_ctx *c, const KnnArgs &a,
 
 }  // namespace
 
+int knn_hand_f64_launch(hop_ctx *c, const KnnArgs &a, int qpw, int cpr, const uint32_t *hand,
+                        const unsigned long long *hand_n, unsigned long long *counter)
+{
+    return knn_run<double, 32, false>(c, a, cpr, hand, hand_n, counter, qpw);
+}
+
 int knn_launch(hop_ctx *c, const KnnArgs &a, bool f64, int qpw, int cpr)
 {
     if (a.k < 2 || a.k > kMaxDens) return ctx_fail(c, HOP_EINVAL, "n_dens out of range");
@@ -1120,7 +1134,10 @@ int knn_launch(hop_ctx *c, const KnnArgs &a, bool f64, int qpw, int cpr)
     if (qpw == 32 && !f64) return knn32_launch(c, a, cpr);   // one query per lane
     // float32 with 4, 8 or 16 queries per warp: the grouped kernel, unless a
     // candidate-buffer factor was set (the single-scan kernel below)
-    if (!f64 && c->capf == 0 && (qpw == 4 || qpw == 8 || qpw == 16)) return knn_gq_launch(c, a, qpw, cpr);
+    if (!f64 && c->capf == 0 && (qpw == 4 || qpw == 8 || qpw == 16)) return knn_gq_launch(c, a, false, qpw, cpr);
+    // float64, whatever the queries per warp: the same kernel (the radius is
+    // per chunk of that many)
+    if (f64 && c->capf == 0 && !a.seg) return knn_gq_launch(c, a, true, qpw, cpr);
     if (a.seg) {
         // batched passes: float32 positions, 4, 8, 16 or 32 queries per warp
         if (f64) return ctx_fail(c, HOP_EINVAL, "batched passes take float32 positions");

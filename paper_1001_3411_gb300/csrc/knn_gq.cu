@@ -1,6 +1,7 @@
 // Certified cell-stencil kNN fused with the M4 cubic-spline density (HOP
-// step 1, Parallel HOP Sec. 2) for float32 positions: four queries per warp,
-// eight lanes per query.
+// step 1, Parallel HOP Sec. 2): four queries per warp, eight lanes per query.
+// It serves float32 positions at 4, 8 and 16 queries per radius chunk and
+// float64 positions at any number (searched in float32, decided in float64).
 //
 // A warp takes a unit of 16 consecutive Morton-sorted particles and serves
 // them in four groups of four.  Consecutive ones farther apart than the
@@ -28,10 +29,14 @@
 //      the array, and an entry's place in the neighbour list is the start of
 //      its bin plus its rank in it by (d^2, original index).
 // A query is certified when at least Ndens particles lie within R; the
-// others search again with a larger R.  What this kernel does not take -- a
-// ball that wraps around the box, more nodes than it lists, a crowd at the
-// Ndens-th distance -- it hands over to the warp-per-query kernel
-// (knn_cg.cu), which runs after it over the list of such queries.
+// others search again with a larger R.  A group whose region crosses both a
+// face and L/2 is served one query at a time.  What this kernel does not take
+// -- a ball that wraps around the box, more nodes than it lists, a crowd at
+// the Ndens-th distance, float64 distances too close for float32 to bin -- it
+// hands over to a warp-per-query kernel (knn_cg.cu; float64: knn.cu), which
+// runs after it over the list of such queries.  Such a query takes 0.3 ms
+// however few there are, so radii reach the largest that does not wrap before
+// one is handed over (4,913 particles: 0.37 -> 0.08 ms).
 //
 // What bounds it: instruction issue and shared-memory wavefronts (58 % of
 // issue slots and 66 % of wavefronts at 16 warps per SM, 1.35k warp
@@ -48,7 +53,8 @@
 // per query): 16.8M particles 33.6 ms (82.1), 64 subvolumes of 22M together
 // 46.5 ms (111.8), 3M with Ndens = Nhop = 65 (closed form) 9.2 ms (22.2), 2.1M
 // with the plain radius, whose start is cut to what the boxes show to be
-// enough, 20.4 ms (59.2), 4,913 particles 0.37 ms (0.99).
+// enough, 19.1 ms (59.2), 4,913 particles 0.08 ms (0.99), 32,768 float64
+// particles 0.72 ms (5.2, the single-scan kernel).
 //
 // Results equal those of the other kNN kernels bit for bit: the same
 // per-component minimum-image differences, the same fused d^2, the same
@@ -58,6 +64,7 @@
 
 #include <algorithm>
 #include <math.h>
+#include <type_traits>
 
 namespace {
 
@@ -76,12 +83,14 @@ constexpr int kGqTries = 96;
 
 struct GqDev {
     const float4 *spos;
+    const double4 *spos64;             // F64: the positions themselves
     BoxTree tree;
     uint32_t n, pad_run;               // pad_run: a run past the last particle
     int64_t n_tasks;                   // units of 16 queries, in `split` parts each
     int split;
     int qpw;                           // queries per radius chunk
     float box, norm;
+    double box64, norm64;
     int k, n_out, ld_out, capq;
     const float *chunk_r;
     float plain_r;
@@ -115,9 +124,9 @@ struct GqSmem {
     // Row stride of the sorted arrays: 8 mod 32, so that the four queries'
     // lanes (eight consecutive words each) read distinct banks.
     __host__ __device__ static int stride(int capq) { return (capq + 23) / 32 * 32 + 8; }
-    __host__ __device__ static int total(int capq)
+    __host__ __device__ static int total(int capq, bool f64)
     {
-        const int sel = t0 + kGqQ * stride(capq) * 8;
+        const int sel = t0 + kGqQ * stride(capq) * (f64 ? 12 : 8);
         return ((search_end > sel ? search_end : sel) + 15) & ~15;
     }
 };
@@ -347,14 +356,14 @@ __device__ __forceinline__ GqFound gq_count(const float2 *list, int cnt, int cma
 }
 
 // Drops the limit of every query that holds at least k entries (and is in
-// `which`) to the upper edge of the bin of its k-th, and its lists to the
-// entries up to it.  Out of line: only lists that are nearly full, or a
+// `which`) to the upper edge of the bin of its k-th (plus slack), and its
+// lists to the entries up to it.  Out of line: only lists that are nearly full, or a
 // crowded k-th bin, need it.
 struct Tight {
     int cnt;
     float tau;
 };
-__device__ __noinline__ Tight gq_tighten(uint32_t wo, int cnt, bool which, float tau, int k, int lane)
+__device__ __noinline__ Tight gq_tighten(uint32_t wo, int cnt, bool which, float tau, float slack, int k, int lane)
 {
     float2 *list = (float2 *)(gq_smem + wo + GqSmem::list) + lane;
     uint16_t *hist = (uint16_t *)(gq_smem + wo + GqSmem::thist);
@@ -362,7 +371,7 @@ __device__ __noinline__ Tight gq_tighten(uint32_t wo, int cnt, bool which, float
     const float scale = gq_scale<kGqCutBins>(tau);
     const GqFound f = gq_count<kGqCutBins, false>(list, which ? cnt : 0, cmax, hist, nullptr, scale, k, 0, lane);
     if (which && f.k) {
-        tau = fminf(tau, gq_edge((int)(f.k >> 20), scale));
+        tau = fminf(tau, gq_edge((int)(f.k >> 20), scale) + slack);
         int m = 0;
 #pragma unroll 1
         for (int i = 0; i < cnt; ++i) {
@@ -479,15 +488,31 @@ __device__ __noinline__ float gq_grow(int k, int tot)
     return fmaxf(1.25f, 1.1f * cbrtf((float)k / (float)max(tot, 1)));
 }
 
-template <bool SEG>
-__global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
+// Exact squared minimum-image distance of two double-precision particles, as
+// the single-scan kernel rounds it.
+__device__ __forceinline__ double gq_d2_f64(const double4 &c, double x, double y, double z, double box)
+{
+    const double half = 0.5 * box;
+    const double dx = wrapdiff(c.x, x, box, half), dy = wrapdiff(c.y, y, box, half), dz = wrapdiff(c.z, z, box, half);
+    return fma(dx, dx, fma(dy, dy, dz * dz));
+}
+
+// F64: the search runs on positions rounded to float; a squared distance
+// found that way is within `err` of the exact one (the bound is the two
+// coordinates' rounding, the frame shift's, and the float arithmetic).  The
+// entries up to the bin after the Ndens-th's therefore hold the exact Ndens
+// nearest as long as a bin is wider than 2 err; their distances are computed
+// again in double, and an entry's place is ranked over its own and the two
+// neighbouring bins.
+template <bool SEG, bool F64>
+__global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(const GqDev a)
 {
     using L = GqSmem;
     int lane;
     asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));   // (kept in a register)
     const int q = lane >> 3, p = lane & 7;
     const uint32_t lt = (1u << lane) - 1u;
-    const uint32_t wo = (uint32_t)L::total(a.capq) * (threadIdx.x >> 5);   // the warp's shared memory
+    const uint32_t wo = (uint32_t)L::total(a.capq, F64) * (threadIdx.x >> 5);   // the warp's shared memory
     unsigned char *wb = gq_smem + wo;
     float2 *list = (float2 *)(wb + L::list) + lane;
     const uint32_t list0 = gq_addr(wo + L::list) + lane * 8;
@@ -497,8 +522,9 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
     uint16_t *bst = (uint16_t *)(wb + L::bst);
     uint32_t *U2 = (uint32_t *)(wb + L::u2), *T0 = (uint32_t *)(wb + L::t0), *T1 = (uint32_t *)(wb + L::t1),
              *T2 = (uint32_t *)(wb + L::t2);
-    float *Dd = (float *)(wb + L::t0) + q * L::stride(a.capq);                     // the query's entries, bin by bin
-    uint32_t *Ds = (uint32_t *)(wb + L::t0) + (kGqQ + q) * L::stride(a.capq);
+    using D2 = std::conditional_t<F64, double, float>;
+    D2 *Dd = (D2 *)(wb + L::t0) + q * L::stride(a.capq);                     // the query's entries, bin by bin
+    uint32_t *Ds = (uint32_t *)(wb + L::t0) + (kGqQ * (int)sizeof(D2) / 4 + q) * L::stride(a.capq);
     const int k = a.k, n_out = a.nbr_s ? a.n_out : 0;
     unsigned long long cand_acc = 0;
     uint32_t search_acc = 0, retry_acc = 0, warp_acc = 0;
@@ -539,12 +565,10 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
             ux = v.x;
             uy = v.y;
             uz = v.z;
-            float r;
-            if (a.chunk_r) {
-                r = a.chunk_r[ch0 + (su - base) / (uint32_t)a.qpw];
-            } else {
-                r = gq_plain_radius(a.tree, v, su, base, end, k, plain_r);
-            }
+            // (a first radius whose ball wraps around the box, as of a chunk
+            // across a jump of the Morton curve, gives way to the plain one)
+            float r = a.chunk_r ? a.chunk_r[ch0 + (su - base) / (uint32_t)a.qpw] : INFINITY;
+            if (2.f * r >= 0.5f * box) r = gq_plain_radius(a.tree, v, su, base, end, k, plain_r);
             if (!(r > 0.f)) r = box * 1e-6f;
             r = fmaxf(r, __shfl_xor_sync(kAll, r, 1));
             r4 = fmaxf(r, __shfl_xor_sync(kAll, r, 2));
@@ -567,15 +591,19 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
         const float ex = qx - __shfl_up_sync(kAll, qx, 8), ey = qy - __shfl_up_sync(kAll, qy, 8),
                     ez = qz - __shfl_up_sync(kAll, qz, 8);
         const uint32_t cuts = __ballot_sync(kAll, p == 0 && q > 0 && q < nq && ex * ex + ey * ey + ez * ez > R0 * R0);
-        int g0 = 0;
-        while (g0 < nq) {
-            const uint32_t rest = cuts & (kAll << (g0 * 8)) & ~(1u << (g0 * 8));
-            const int g1 = rest ? (__ffs(rest) - 1) >> 3 : nq;
-            bool member = q >= g0 && q < g1;   // still to be served
-            g0 = g1;
-            float R = R0;
-            int tries = 0;
-            for (;;) {
+        uint32_t todo = (1u << (8 * nq - 1)) * 2u - 1u;   // the lanes of the queries still to be served
+        float rq = R0;                                     // the query's radius
+        bool alone = false;
+        int tries = 0;
+        {
+            while (todo) {
+                // from the first one up to the next cut, or the first alone
+                const int g0 = __ffs(todo) - 1;
+                const uint32_t later = cuts & ~((2u << g0) - 1u);
+                uint32_t set = todo & (later ? (later & (0u - later)) - 1u : kAll);
+                if (alone) set = 0xffu << g0;
+                const bool member = (set >> lane) & 1u;
+                const float R = warp_max(member ? rq : 0.f);
                 // ------------- the 512-particle nodes that meet the region
                 Region rg;
                 float fx = qx, fy = qy, fz = qz;
@@ -600,14 +628,26 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
                     }
                 }
                 if (n2 < 0) {
-                    if (member && p == 0) a.hand[atomicAdd(a.hand_n, 1ull)] = sq;
-                    break;
+                    // several queries' region that crosses both a face and L/2,
+                    // or meets too many nodes: the first one alone
+                    alone = !alone && set != (0xffu << g0);
+                    if (!alone) {
+                        if (member && p == 0) a.hand[atomicAdd(a.hand_n, 1ull)] = sq;
+                        todo &= ~set;
+                    }
+                    continue;
                 }
+                alone = false;
                 ++search_acc;
                 // ------------- open them and evaluate the runs
                 uint32_t lp = list0;   // the end of the lane's list
                 float tau = member ? R * R : -1.f;
                 bool crowd = false;
+                float slack = 0.f;   // F64: 2 err
+                if constexpr (F64) {
+                    const float d = box * 2.38418579e-7f;   // 2^-22 of the box per component
+                    slack = 2.f * (3.47f * R * d + 3.f * d * d + R * R * 4.76837158e-7f);
+                }
                 int i2 = 0, i1 = 0, n1 = 0, cand = 0;
                 for (;;) {
                     int n0 = 0;
@@ -701,7 +741,7 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
                             }
                             if (over) {
                                 __syncwarp();
-                                const Tight t = gq_tighten(wo, (int)(lp - list0) >> 8, member && !crowd, tau, k, lane);
+                                const Tight t = gq_tighten(wo, (int)(lp - list0) >> 8, member && !crowd, tau, slack, k, lane);
                                 lp = list0 + t.cnt * 256;
                                 tau = t.tau;
                                 // a list that stays full: a crowd at the limit
@@ -730,11 +770,26 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
                     int cmax = 0;
                     float scale = 0.f;
                     GqFound f;
+                    int upto = 0, upto_o = 0;
+                    const uint16_t *t = bst + q * (kGqBins + 2);
                     for (int it = 0;; ++it) {
                         cmax = (int)__reduce_max_sync(kAll, ok ? (unsigned)cnt : 0u);
                         scale = gq_scale<kGqBins>(tau);
                         f = gq_count<kGqBins, true>(list, ok ? cnt : 0, cmax, hist, bst, scale, k, n_out, lane);
-                        const bool over = ok && (int)(f.k & 1023u) > a.capq;
+                        upto = (int)(f.k & 1023u);
+                        upto_o = (int)(f.o & 1023u);
+                        if constexpr (F64) {
+                            upto = t[min((int)(f.k >> 20) + 2, kGqBins)];
+                            upto_o = t[min((int)(f.o >> 20) + 2, kGqBins)];
+                            if (ok && slack > 0.9f * tau * (1.f / kGqBins)) {
+                                // bins too narrow for float distances
+                                ok = false;
+                                crowd = true;
+                            } else if (ok && (int)(f.k >> 20) == kGqBins - 1 && tau >= R * R) {
+                                ok = false;   // not certain that R reaches the exact Ndens-th: a larger one
+                            }
+                        }
+                        const bool over = ok && upto > a.capq;
                         if (!__any_sync(kAll, over)) break;
                         if (it == 3) {
                             // the bin stays crowded
@@ -744,13 +799,21 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
                             }
                             break;
                         }
-                        const Tight t = gq_tighten(wo, cnt, over, tau, k, lane);
-                        cnt = t.cnt;
-                        tau = t.tau;
+                        const Tight c = gq_tighten(wo, cnt, over, tau, slack, k, lane);
+                        cnt = c.cnt;
+                        tau = c.tau;
                     }
-                    const int bk = (int)(f.k >> 20), below = (int)((f.k >> 10) & 1023u),
-                              upto = ok ? (int)(f.k & 1023u) : 0;
-                    const uint32_t col = gq_column(hist, lane), last_bin = 0x4b000000u + (uint32_t)bk;
+                    const int bk = (int)(f.k >> 20);
+                    const int below = F64 ? t[max(bk - 1, 0)] : (int)((f.k >> 10) & 1023u);
+                    if (!ok) upto = upto_o = 0;
+                    const uint32_t col = gq_column(hist, lane), last_bin = 0x4b000000u + (uint32_t)bk + (F64 ? 1u : 0u);
+                    double q64x = 0.0, q64y = 0.0, q64z = 0.0;
+                    if constexpr (F64) {
+                        const double4 v = a.spos64[sq];
+                        q64x = v.x;
+                        q64y = v.y;
+                        q64z = v.z;
+                    }
                     const int cnt_ok = ok ? cnt : 0;
 #pragma unroll 2
                     for (int i = 0; i < cmax; ++i) {
@@ -759,37 +822,44 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
                         const bool on = i < cnt_ok && b <= last_bin;
                         const uint32_t pos = gq_next(col + b * 64, on);
                         if (on) {
-                            Dd[pos] = v.x;
+                            if constexpr (F64)
+                                Dd[pos] = gq_d2_f64(a.spos64[__float_as_uint(v.y)], q64x, q64y, q64z, a.box64);
+                            else
+                                Dd[pos] = v.x;
                             Ds[pos] = __float_as_uint(v.y);
                         }
                     }
                     __syncwarp();
                     // the exact k-th d^2: the largest of its bin with fewer
                     // than k smaller entries
-                    float vk = -1.f;
+                    D2 vk = D2(-1);
 #pragma unroll 1
                     for (int e = below + p; e < upto; e += 8) {
-                        const float v = Dd[e];
+                        const D2 v = Dd[e];
                         int l = below;
 #pragma unroll 2
                         for (int h = below; h < upto; ++h) l += Dd[h] < v;
-                        if (l < k) vk = fmaxf(vk, v);
+                        if (l < k) vk = max(vk, v);
                     }
                     __syncwarp();
-                    vk = fmaxf(vk, __shfl_xor_sync(kAll, vk, 1));
-                    vk = fmaxf(vk, __shfl_xor_sync(kAll, vk, 2));
-                    vk = fmaxf(vk, __shfl_xor_sync(kAll, vk, 4));
+                    vk = max(vk, __shfl_xor_sync(kAll, vk, 1));
+                    vk = max(vk, __shfl_xor_sync(kAll, vk, 2));
+                    vk = max(vk, __shfl_xor_sync(kAll, vk, 4));
                     // density: fixed-point (2^-32) sum of w(2 r / r_k) over
                     // entries with d^2 < r_k^2; a weight of 1 is one more
                     // than the conversion's largest value
-                    const float rk = sqrtf(vk);
-                    const float inv_h = vk > 0.f ? 2.f / rk : 0.f;
+                    const D2 rk = sqrt(vk);
+                    const D2 inv_h = vk > D2(0) ? D2(2) / rk : D2(0);
                     unsigned long long wsum = 0;
 #pragma unroll 1
                     for (int e = p; e < upto; e += 8) {
-                        const float v = Dd[e];
+                        const D2 v = Dd[e];
+                        if constexpr (F64) {
+                            if (v < vk) wsum += (unsigned long long)(m4<double>(sqrt(v) * inv_h) * 4294967296.0 + 0.5);
+                            continue;
+                        }
                         // m4(), both of its pieces computed
-                        const float x = sqrtf(v) * inv_h, y = 2.f - x;
+                        const float x = sqrtf((float)v) * (float)inv_h, y = 2.f - x;
                         const float wi = 1.f - 1.5f * x * x + 0.75f * x * x * x, wo_ = 0.25f * y * y * y;
                         const float w = (x < 1.f ? wi : wo_) * 4294967296.0f + 0.5f;
                         if (v < vk) wsum += (unsigned long long)__float2uint_rz(w) + (w >= 4294967296.0f ? 1u : 0u);
@@ -799,27 +869,42 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
                     for (int o = 1; o < 8; o <<= 1) wsum += __shfl_xor_sync(kAll, wsum, o);
                     if (ok && p == 0) {
                         float dens;
-                        if (vk > 0.f) {
-                            const float h = rk * 0.5f;
-                            dens = (float)(norm * ((float)wsum * 2.3283064365386963e-10f) / (h * h * h));
+                        if (vk > D2(0)) {
+                            const D2 h = rk * D2(0.5);
+                            if constexpr (F64)
+                                dens = (float)(a.norm64 * ((double)wsum * 2.3283064365386963e-10) / (h * h * h));
+                            else
+                                dens = (float)(norm * ((float)wsum * 2.3283064365386963e-10f) / (h * h * h));
                         } else {
                             dens = INFINITY;
                         }
                         a.dens_s[sq] = dens;
-                        if (a.rk_s) a.rk_s[sq] = rk;
+                        if (a.rk_s) a.rk_s[sq] = (float)rk;
                     }
                     // the n_out nearest by (d^2, original index): the start of
                     // the entry's bin and its rank in it
                     if (n_out > 0) {
-                        const int upto_o = ok ? (int)(f.o & 1023u) : 0;
-                        const uint16_t *t = bst + q * (kGqBins + 2);
                         uint32_t *row = a.nbr_s + (size_t)sq * a.ld_out;
 #pragma unroll 1
+                        // the entries that may come before or after entry e
+                        auto around = [&](int e, D2 v, int &h0, int &h1) {
+                            if constexpr (F64) {
+                                // its bin from its place, then one bin either way
+                                int b = 0;
+                                while (b < kGqBins - 1 && t[b + 1] <= e) ++b;
+                                h0 = t[max(b - 1, 0)];
+                                h1 = min((int)t[min(b + 2, kGqBins)], upto_o);
+                            } else {
+                                const int b = gq_bin(v, scale);
+                                h0 = t[b];
+                                h1 = t[b + 1];
+                            }
+                        };
                         int sum = 0;
                         for (int e = p; e < upto_o; e += 8) {
-                            const float v = Dd[e];
-                            const int b = gq_bin(v, scale);
-                            const int h0 = t[b], h1 = t[b + 1];
+                            const D2 v = Dd[e];
+                            int h0, h1;
+                            around(e, v, h0, h1);
                             int rank = h0;
 #pragma unroll 2
                             for (int h = h0; h < h1; ++h) rank += Dd[h] < v;
@@ -833,14 +918,14 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
                         if (__any_sync(kAll, ties)) {
 #pragma unroll 1
                             for (int e = p; ties && e < upto_o; e += 8) {
-                                const float v = Dd[e];
+                                const D2 v = Dd[e];
                                 const uint32_t se = Ds[e], oe = __float_as_uint(a.spos[se].w);
-                                const int b = gq_bin(v, scale);
-                                const int h0 = t[b], h1 = t[b + 1];
+                                int h0, h1;
+                                around(e, v, h0, h1);
                                 int rank = h0;
 #pragma unroll 1
                                 for (int h = h0; h < h1; ++h) {
-                                    const float u = Dd[h];
+                                    const D2 u = Dd[h];
                                     rank += u < v;
                                     if (u == v) rank += __float_as_uint(a.spos[Ds[h]].w) < oe;
                                 }
@@ -851,13 +936,18 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
                     __syncwarp();
                 }
                 if (member && crowd && p == 0) a.hand[atomicAdd(a.hand_n, 1ull)] = (uint32_t)sq;
-                member = member && !ok && !crowd;
-                if (!__any_sync(kAll, member)) break;
-                // the others: too few within R
-                ++retry_acc;
-                ++tries;
-                const float grow = member ? gq_grow(k, tot) : 1.25f;
-                R *= fminf(warp_max(grow), 8.f);
+                todo &= ~__ballot_sync(kAll, ok || (member && crowd));
+                // the others of the set hold too few within R: a larger one, at
+                // first not beyond the largest this kernel takes
+                if (todo & set) {
+                    ++retry_acc;
+                    ++tries;
+                    if (member && !ok && !crowd) {
+                        const float most = 0.2499f * box;
+                        rq = R * fminf(gq_grow(k, tot), 8.f);
+                        if (R < 0.99f * most) rq = fminf(rq, most);
+                    }
+                }
                 __syncwarp();
             }
         }
@@ -871,12 +961,31 @@ __global__ void __launch_bounds__(kGqWarps * 32, 4) knn_gq_kernel(const GqDev a)
     }
 }
 
-template <bool SEG> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int qpw, int cpr)
+// Rounded copies of double-precision particles, the padding included.
+__global__ void to_float4_kernel(const double4 *__restrict__ in, int64_t n, float4 *__restrict__ out)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const double4 v = in[i];
+        out[i] = make_float4((float)v.x, (float)v.y, (float)v.z, __uint_as_float((uint32_t)__double_as_longlong(v.w)));
+    }
+}
+
+template <bool SEG, bool F64> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int qpw, int cpr)
 {
     GqDev d;
-    const int rc = box_tree_build(c, (const float4 *)ka.spos, ka.n, &d.tree);
-    if (rc) return rc;
+    d.spos64 = nullptr;
     d.spos = (const float4 *)ka.spos;
+    if constexpr (F64) {
+        const int64_t m = ka.n + kSposPad;
+        float4 *f = (float4 *)ctx_buf(c, S_SPOS_F, (size_t)m * sizeof(float4));
+        if (!f) return HOP_ENOMEM;
+        to_float4_kernel<<<grid_for(c, m), 256, 0, c->stream>>>((const double4 *)ka.spos, m, f);
+        HOP_LAUNCH(c);
+        d.spos = f;
+        d.spos64 = (const double4 *)ka.spos;
+    }
+    const int rc = box_tree_build(c, d.spos, ka.n, &d.tree);
+    if (rc) return rc;
     d.n = (uint32_t)ka.n;
     d.pad_run = (uint32_t)((ka.n + 7) / 8);
     // a warp takes a whole unit, except where that would leave warps idle:
@@ -889,6 +998,8 @@ template <bool SEG> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int qpw, int c
     d.qpw = qpw;
     d.box = (float)ka.box;
     d.norm = (float)(ka.box * ka.box * ka.box / ((double)(ka.n_norm > 0 ? ka.n_norm : ka.n) * 3.14159265358979323846));
+    d.box64 = ka.box;
+    d.norm64 = ka.box * ka.box * ka.box / ((double)(ka.n_norm > 0 ? ka.n_norm : ka.n) * 3.14159265358979323846);
     d.k = ka.k;
     d.n_out = ka.n_out;
     d.ld_out = ka.ld_out;
@@ -907,8 +1018,8 @@ template <bool SEG> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int qpw, int c
     d.hand = (uint32_t *)ctx_buf(c, S_KNN_HAND, (size_t)ka.n * sizeof(uint32_t));
     if (!d.hand) return HOP_ENOMEM;
     HOP_CUDA(c, cudaMemsetAsync(d.task_counter, 0, 3 * sizeof(unsigned long long), c->stream));
-    const size_t smem = (size_t)GqSmem::total(d.capq) * kGqWarps;
-    auto kern = knn_gq_kernel<SEG>;
+    const size_t smem = (size_t)GqSmem::total(d.capq, F64) * kGqWarps;
+    auto kern = knn_gq_kernel<SEG, F64>;
     HOP_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     HOP_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kGqWarps * 32, smem));
@@ -917,14 +1028,15 @@ template <bool SEG> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int qpw, int c
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * c->num_sms, need));
     kern<<<(unsigned)blocks, kGqWarps * 32, smem, c->stream>>>(d);
     HOP_LAUNCH(c);
+    if constexpr (F64) return knn_hand_f64_launch(c, ka, qpw, cpr, d.hand, d.hand_n, d.hand_n + 1);
     return knn_wq_launch(c, ka, qpw, cpr, d.hand, d.hand_n, d.hand_n + 1);
 }
 
 }  // namespace
 
-int knn_gq_launch(hop_ctx *c, const KnnArgs &a, int qpw, int cpr)
+int knn_gq_launch(hop_ctx *c, const KnnArgs &a, bool f64, int qpw, int cpr)
 {
-    if (qpw != 4 && qpw != 8 && qpw != 16)
-        return ctx_fail(c, HOP_EINVAL, "the grouped kNN takes radius chunks of 4, 8 or 16 queries");
-    return a.seg ? knn_gq_run<true>(c, a, qpw, cpr) : knn_gq_run<false>(c, a, qpw, cpr);
+    if (qpw < 1) return ctx_fail(c, HOP_EINVAL, "radius chunks hold at least one query");
+    if (f64) return knn_gq_run<false, true>(c, a, qpw, cpr);
+    return a.seg ? knn_gq_run<true, false>(c, a, qpw, cpr) : knn_gq_run<false, false>(c, a, qpw, cpr);
 }

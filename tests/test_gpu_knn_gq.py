@@ -92,3 +92,27 @@ def test_subvolumes_at_odd_offsets(hop, sizes, qpw):
             hop.apply_tuning(8, 1, 0)
     for key in ("dens", "nbr", "group"):
         assert torch.equal(out[0][key], out[1][key]), key
+
+
+F64_CASES = {
+    "plummer": lambda: synth.workload("plummer32k"),
+    "lattice": lambda: synth.lattice_box(16, dtype=np.float64),
+    "uniform": lambda: synth.uniform_box(20011, 5, dtype=np.float64),
+    "tiny": lambda: synth.uniform_box(130, 6, dtype=np.float64),
+    # distances far below a float's spacing at the coordinates' size
+    "tight": lambda: np.concatenate([0.7 + 1e-7 * np.random.default_rng(4).random((300, 3)),
+                                     np.random.default_rng(5).random((3000, 3))]),
+}
+
+
+@pytest.mark.parametrize("qpw", [1, 8, 32])
+@pytest.mark.parametrize("case", list(F64_CASES))
+def test_float64(hop, case, qpw):
+    _both(hop, F64_CASES[case](), qpw=qpw, pos_is_f64=1)
+
+
+@pytest.mark.parametrize("box", [1e-3, 250.0])
+def test_float64_boxes_and_lists(hop, box):
+    pos = (synth.nfw_box(20001, 31, dtype=np.float64)[0] * box) % box
+    for k, ld, mode in ((64, 64, 0), (65, 65, 1), (128, 16, 1), (2, 2, 0)):
+        _both(hop, pos, box=box, ld=ld, n_dens=k, n_hop=min(ld, k), n_merge=1, radius_mode=mode, pos_is_f64=1)
