@@ -141,7 +141,7 @@ struct BatchGraph {
 namespace {
 
 constexpr int kProtoBodyKernels = 3;     // hook, compress, loop condition
-constexpr int kBoruvkaBodyKernels = 6;   // fill, best edge, target, hook, compress, loop condition
+constexpr int kBoruvkaBodyKernels = 7;   // reset, best edge (3), hook, compress, loop condition
 
 // Host-side description of one batched pass.
 struct BatchPlan {

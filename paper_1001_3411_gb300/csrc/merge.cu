@@ -3,15 +3,18 @@
 //  M1  chains = roots (chain[i] == i) with density >= delta_outer, numbered
 //      densely by a scan; every boundary endpoint is such a root.
 //  M2  proto-halos: root density >= delta_peak.
-//  M3  edges sorted once in the strict merge order (s desc, lo asc, hi asc,
-//      lo/hi the roots' original indices) by two stable radix sorts, so an
-//      edge's position is its rank.
+//  M3  edges in the strict merge order: s desc, then lo asc, hi asc (lo / hi
+//      the roots' original indices).  Nothing is sorted: a component's best
+//      edge is the largest s (bits of a double >= 0 order like its value)
+//      and, among the edges with it, the smallest (lo, hi), which names the
+//      edge.  That is two more passes over the edges per round and spares two
+//      sorts of 8 radix passes each.
 //  M4  proto-halos joined by a direct boundary s >= 2 delta_saddle:
 //      connected components (hook to the smaller root + compress, until no
 //      edge joins two roots).  Each component is an owned set.
 //  M5  sub-peak chains: Boruvka rounds on the maximum spanning forest of the
 //      boundary graph with all owned sets contracted.  In a round every
-//      unowned component picks its best edge (smallest rank) to another
+//      unowned component picks its best edge to another
 //      component not both owned; it hooks to the other side (owned targets
 //      absorb it; a mutual pick keeps the smaller label as root).  Owned sets
 //      never pick, so no two owned sets meet.  Under a strict edge order the
@@ -59,13 +62,11 @@ __global__ void root_list_kernel(const uint32_t *__restrict__ chain, const uint6
     }
 }
 
-// Edge endpoints -> dense chain ids; sort key for (lo_orig, hi_orig).
-__global__ void edge_prep_kernel(const uint64_t *__restrict__ ekey, const double *__restrict__ esum,
-                                 DevCount mc, int64_t n, const uint32_t *__restrict__ chain,
+// Edge endpoints -> dense chain ids, and the edge's name (lo_orig, hi_orig).
+__global__ void edge_prep_kernel(const uint64_t *__restrict__ ekey, DevCount mc, int64_t n, const uint32_t *__restrict__ chain,
                                  const uint32_t *__restrict__ cid, const uint64_t *__restrict__ dkey,
                                  float d_o, uint32_t *__restrict__ ea, uint32_t *__restrict__ eb,
-                                 uint64_t *__restrict__ k1, uint32_t *__restrict__ v1,
-                                 uint32_t *__restrict__ err, int64_t c_cap)
+                                 uint64_t *__restrict__ ename, uint32_t *__restrict__ err, int64_t c_cap)
 {
     const int64_t m = mc.get();
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
@@ -76,40 +77,13 @@ __global__ void edge_prep_kernel(const uint64_t *__restrict__ ekey, const double
         if (bad || cid[lo] >= (uint64_t)c_cap || cid[hi] >= (uint64_t)c_cap) {
             atomicOr(err, bad ? kErrBadIndex : kErrChainCap);
             ea[e] = eb[e] = 0;
-            k1[e] = 0;
-            v1[e] = (uint32_t)e;
+            ename[e] = 0;
             continue;
         }
         const uint32_t olo = key_orig(dkey[lo]), ohi = key_orig(dkey[hi]);
         ea[e] = cid[lo];
         eb[e] = cid[hi];
-        k1[e] = olo < ohi ? (((uint64_t)olo << 32) | ohi) : (((uint64_t)ohi << 32) | olo);
-        v1[e] = (uint32_t)e;
-        (void)esum;
-    }
-}
-
-__global__ void edge_key2_kernel(const double *__restrict__ esum, const uint32_t *__restrict__ order,
-                                 DevCount mc, uint64_t *__restrict__ k2)
-{
-    const int64_t m = mc.get();
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < m;
-         t += (int64_t)gridDim.x * blockDim.x)
-        k2[t] = ~(uint64_t)__double_as_longlong(esum[order[t]]);
-}
-
-__global__ void edge_permute_kernel(const uint32_t *__restrict__ order, DevCount mc,
-                                    const uint32_t *__restrict__ ea, const uint32_t *__restrict__ eb,
-                                    const double *__restrict__ esum, uint32_t *__restrict__ sa,
-                                    uint32_t *__restrict__ sb, double *__restrict__ ss)
-{
-    const int64_t m = mc.get();
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < m;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t e = order[t];
-        sa[t] = ea[e];
-        sb[t] = eb[e];
-        ss[t] = esum[e];
+        ename[e] = olo < ohi ? (((uint64_t)olo << 32) | ohi) : (((uint64_t)ohi << 32) | olo);
     }
 }
 
@@ -119,14 +93,6 @@ __global__ void iota_kernel(uint32_t *p, DevCount nc)
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
         p[i] = (uint32_t)i;
-}
-
-__global__ void fill_kernel(uint32_t *p, DevCount nc, uint32_t v)
-{
-    const int64_t n = nc.get();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = v;
 }
 
 __global__ void proto_hook_kernel(const uint32_t *__restrict__ sa, const uint32_t *__restrict__ sb,
@@ -154,51 +120,63 @@ __global__ void compress_kernel(uint32_t *parent, DevCount cc)
         parent[c] = find_root(parent, (uint32_t)c);
 }
 
-// Boruvka: every unowned component's smallest-rank eligible edge.
+// Boruvka: every unowned component's best edge, named by its sum and its
+// (lo, hi).  bs = 0: none (sums are at least 2 delta_outer > 0 where edges
+// come from boundaries; an edge of sum 0 still beats none by its name).
+struct Best {
+    unsigned long long *s, *name;
+    uint32_t *tgt;
+};
+
+__global__ void best_reset_kernel(DevCount cc, Best b)
+{
+    const int64_t C = cc.get();
+    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < C; c += (int64_t)gridDim.x * blockDim.x) {
+        b.s[c] = 0ull;
+        b.name[c] = ~0ull;
+        b.tgt[c] = kNone;
+    }
+}
+
+// Step 0: the largest sum; 1: the smallest name among the edges with it; 2:
+// the other side of that edge.
+template <int STEP>
 __global__ void best_edge_kernel(const uint32_t *__restrict__ sa, const uint32_t *__restrict__ sb,
-                                 DevCount mc, const uint32_t *__restrict__ parent,
-                                 const uint8_t *__restrict__ own, uint32_t *__restrict__ best)
+                                 const double *__restrict__ ss, const uint64_t *__restrict__ ename, DevCount mc,
+                                 const uint32_t *__restrict__ parent, const uint8_t *__restrict__ own, Best b)
 {
     const int64_t m = mc.get();
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < m;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t ca = parent[sa[t]], cb = parent[sb[t]];
-        if (ca == cb) continue;
-        const bool oa = own[ca], ob = own[cb];
-        if (oa && ob) continue;
-        if (!oa) atomicMin(&best[ca], (uint32_t)t);
-        if (!ob) atomicMin(&best[cb], (uint32_t)t);
-    }
-}
-
-__global__ void target_kernel(const uint32_t *__restrict__ sa, const uint32_t *__restrict__ sb,
-                              DevCount cc, const uint32_t *__restrict__ parent,
-                              const uint8_t *__restrict__ own, const uint32_t *__restrict__ best,
-                              uint32_t *__restrict__ tgt)
-{
-    const int64_t C = cc.get();
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < C;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t y = kNone;
-        if (parent[x] == (uint32_t)x && !own[x] && best[x] != kNone) {
-            const uint32_t t = best[x];
-            const uint32_t ca = parent[sa[t]], cb = parent[sb[t]];
-            y = ca == (uint32_t)x ? cb : ca;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < m; t += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t c[2] = {parent[sa[t]], parent[sb[t]]};
+        if (c[0] == c[1]) continue;
+        const bool o[2] = {own[c[0]] != 0, own[c[1]] != 0};
+        if (o[0] && o[1]) continue;
+        const unsigned long long v = (unsigned long long)__double_as_longlong(ss[t]);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            if (o[i]) continue;
+            if constexpr (STEP == 0) {
+                if (b.s[c[i]] < v) atomicMax(&b.s[c[i]], v);
+            } else if (b.s[c[i]] == v) {
+                if constexpr (STEP == 1) {
+                    atomicMin(&b.name[c[i]], (unsigned long long)ename[t]);
+                } else if (b.name[c[i]] == ename[t]) {
+                    b.tgt[c[i]] = c[1 - i];
+                }
+            }
         }
-        tgt[x] = y;
     }
 }
 
-__global__ void hook_kernel(DevCount cc, const uint8_t *__restrict__ own,
-                            const uint32_t *__restrict__ best, const uint32_t *__restrict__ tgt,
-                            uint32_t *parent, uint32_t *changed)
+__global__ void hook_kernel(DevCount cc, const uint8_t *__restrict__ own, Best b, uint32_t *parent, uint32_t *changed)
 {
     const int64_t C = cc.get();
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < C;
          x += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t y = tgt[x];
+        const uint32_t y = b.tgt[x];
         if (y == kNone) continue;
-        if (!own[y] && best[y] == best[x] && (uint32_t)x < y) continue;  // mutual: smaller stays root
+        // mutual: smaller stays root
+        if (!own[y] && b.s[y] == b.s[x] && b.name[y] == b.name[x] && (uint32_t)x < y) continue;
         parent[x] = y;
         *changed = 1u;
     }
@@ -336,27 +314,21 @@ int merge_groups(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, int64_
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += align256(bytes); return o; };
     const size_t o_ckey = take(Cp * 8), o_own = take(Cp), o_parent = take(Cp * 4),
-                 o_best = take(Cp * 4), o_tgt = take(Cp * 4), o_gpeak = take(Cp * 8),
+                 o_bs = take(Cp * 8), o_bn = take(Cp * 8), o_tgt = take(Cp * 4), o_gpeak = take(Cp * 8),
                  o_flag = take((Cp + 1) * 4), o_grank = take(Cp * 4), o_ea = take(mp * 4),
-                 o_eb = take(mp * 4), o_sa = take(mp * 4), o_sb = take(mp * 4), o_ss = take(mp * 8),
-                 o_k1 = take(mp * 8), o_k1b = take(mp * 8), o_v1 = take(mp * 4),
-                 o_v1b = take(mp * 4), o_gk = take(Cp * 8), o_gkb = take(Cp * 8),
+                 o_eb = take(mp * 4), o_name = take(mp * 8), o_gk = take(Cp * 8), o_gkb = take(Cp * 8),
                  o_gv = take(Cp * 4), o_gvb = take(Cp * 4);
-    const size_t sort_tmp = std::max(radix_sort_scratch_bytes(mp), radix_sort_scratch_bytes(Cp));
-    const size_t o_tmp = take(sort_tmp);
+    const size_t o_tmp = take(radix_sort_scratch_bytes(Cp));
     char *base = (char *)ctx_buf(c, S_MERGE, off);
     if (!base) return HOP_ENOMEM;
     uint64_t *ckey = (uint64_t *)(base + o_ckey);
     uint8_t *own = (uint8_t *)(base + o_own);
-    uint32_t *parent = (uint32_t *)(base + o_parent), *best = (uint32_t *)(base + o_best),
-             *tgt = (uint32_t *)(base + o_tgt), *flag = (uint32_t *)(base + o_flag),
-             *grank = (uint32_t *)(base + o_grank);
+    uint32_t *parent = (uint32_t *)(base + o_parent), *tgt = (uint32_t *)(base + o_tgt),
+             *flag = (uint32_t *)(base + o_flag), *grank = (uint32_t *)(base + o_grank);
     unsigned long long *gpeak = (unsigned long long *)(base + o_gpeak);
-    uint32_t *ea = (uint32_t *)(base + o_ea), *eb = (uint32_t *)(base + o_eb),
-             *sa = (uint32_t *)(base + o_sa), *sb = (uint32_t *)(base + o_sb);
-    double *ss = (double *)(base + o_ss);
-    uint64_t *k1 = (uint64_t *)(base + o_k1), *k1b = (uint64_t *)(base + o_k1b);
-    uint32_t *v1 = (uint32_t *)(base + o_v1), *v1b = (uint32_t *)(base + o_v1b);
+    const Best best{(unsigned long long *)(base + o_bs), (unsigned long long *)(base + o_bn), tgt};
+    uint32_t *ea = (uint32_t *)(base + o_ea), *eb = (uint32_t *)(base + o_eb);
+    uint64_t *ename = (uint64_t *)(base + o_name);
     uint64_t *gk = (uint64_t *)(base + o_gk), *gkb = (uint64_t *)(base + o_gkb);
     uint32_t *gv = (uint32_t *)(base + o_gv), *gvb = (uint32_t *)(base + o_gvb);
     void *tmp = base + o_tmp;
@@ -365,18 +337,11 @@ int merge_groups(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, int64_
     root_list_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(chain, dkey, n, d_o, d_p, cid, ckey, own, Cp,
                                                             d_merr);
     HOP_LAUNCH(c);
-    // M3: strict order
+    // M3: endpoints and names
+    const DevCount Cc{C, nullptr}, mc{m, nullptr};
     if (m > 0) {
-        edge_prep_kernel<<<grid_for(c, m), 256, 0, c->stream>>>(edge_key, edge_sum, DevCount{m, nullptr}, n, chain, cid,
-                                                               dkey, d_o, ea, eb, k1, v1, d_merr, Cp);
-        HOP_LAUNCH(c);
-        rc = radix_sort_u64(c, k1, k1b, v1, v1b, m, 0, 64, tmp);
-        if (rc) return rc;
-        edge_key2_kernel<<<grid_for(c, m), 256, 0, c->stream>>>(edge_sum, v1, DevCount{m, nullptr}, k1);
-        HOP_LAUNCH(c);
-        rc = radix_sort_u64(c, k1, k1b, v1, v1b, m, 0, 64, tmp);
-        if (rc) return rc;
-        edge_permute_kernel<<<grid_for(c, m), 256, 0, c->stream>>>(v1, DevCount{m, nullptr}, ea, eb, edge_sum, sa, sb, ss);
+        edge_prep_kernel<<<grid_for(c, m), 256, 0, c->stream>>>(edge_key, mc, n, chain, cid, dkey, d_o, ea, eb, ename,
+                                                               d_merr, Cp);
         HOP_LAUNCH(c);
     }
     // M4: proto-halo components
@@ -385,8 +350,8 @@ int merge_groups(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, int64_
     int rounds = 0;
     for (; m > 0 && rounds < kMaxRounds; ++rounds) {
         HOP_CUDA(c, cudaMemsetAsync(d_changed, 0, 4, c->stream));
-        proto_hook_kernel<<<grid_for(c, m), 256, 0, c->stream>>>(sa, sb, ss, DevCount{m, nullptr}, 2.0 * (double)d_s, own,
-                                                                parent, d_changed);
+        proto_hook_kernel<<<grid_for(c, m), 256, 0, c->stream>>>(ea, eb, edge_sum, mc, 2.0 * (double)d_s, own, parent,
+                                                                d_changed);
         HOP_LAUNCH(c);
         compress_kernel<<<grid_for(c, C), 256, 0, c->stream>>>(parent, DevCount{C, nullptr});
         HOP_LAUNCH(c);
@@ -399,13 +364,15 @@ int merge_groups(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, int64_
     // M5: Boruvka over sub-peak chains
     for (rounds = 0; m > 0 && rounds < kMaxRounds; ++rounds) {
         HOP_CUDA(c, cudaMemsetAsync(d_changed, 0, 4, c->stream));
-        fill_kernel<<<grid_for(c, C), 256, 0, c->stream>>>(best, DevCount{C, nullptr}, kNone);
+        best_reset_kernel<<<grid_for(c, C), 256, 0, c->stream>>>(Cc, best);
         HOP_LAUNCH(c);
-        best_edge_kernel<<<grid_for(c, m), 256, 0, c->stream>>>(sa, sb, DevCount{m, nullptr}, parent, own, best);
+        best_edge_kernel<0><<<grid_for(c, m), 256, 0, c->stream>>>(ea, eb, edge_sum, ename, mc, parent, own, best);
         HOP_LAUNCH(c);
-        target_kernel<<<grid_for(c, C), 256, 0, c->stream>>>(sa, sb, DevCount{C, nullptr}, parent, own, best, tgt);
+        best_edge_kernel<1><<<grid_for(c, m), 256, 0, c->stream>>>(ea, eb, edge_sum, ename, mc, parent, own, best);
         HOP_LAUNCH(c);
-        hook_kernel<<<grid_for(c, C), 256, 0, c->stream>>>(DevCount{C, nullptr}, own, best, tgt, parent, d_changed);
+        best_edge_kernel<2><<<grid_for(c, m), 256, 0, c->stream>>>(ea, eb, edge_sum, ename, mc, parent, own, best);
+        HOP_LAUNCH(c);
+        hook_kernel<<<grid_for(c, C), 256, 0, c->stream>>>(Cc, own, best, parent, d_changed);
         HOP_LAUNCH(c);
         compress_kernel<<<grid_for(c, C), 256, 0, c->stream>>>(parent, DevCount{C, nullptr});
         HOP_LAUNCH(c);
@@ -452,10 +419,13 @@ namespace {
 struct RoundArgs {
     const uint32_t *sa, *sb;
     const double *ss;
+    const uint64_t *ename;
     DevCount m, C;
     double two_ds;
     const uint8_t *own;
-    uint32_t *parent, *best, *tgt, *changed;
+    uint32_t *parent;
+    Best best;
+    uint32_t *changed;
     int64_t cmax, mmax;
 };
 
@@ -473,13 +443,15 @@ int proto_round(hop_ctx *c, void *p)
 int boruvka_round(hop_ctx *c, void *p)
 {
     const RoundArgs &r = *(const RoundArgs *)p;
-    fill_kernel<<<grid_for(c, r.cmax), 256, 0, c->stream>>>(r.best, r.C, kNone);
+    best_reset_kernel<<<grid_for(c, r.cmax), 256, 0, c->stream>>>(r.C, r.best);
     HOP_LAUNCH(c);
-    best_edge_kernel<<<grid_for(c, r.mmax), 256, 0, c->stream>>>(r.sa, r.sb, r.m, r.parent, r.own, r.best);
+    best_edge_kernel<0><<<grid_for(c, r.mmax), 256, 0, c->stream>>>(r.sa, r.sb, r.ss, r.ename, r.m, r.parent, r.own, r.best);
     HOP_LAUNCH(c);
-    target_kernel<<<grid_for(c, r.cmax), 256, 0, c->stream>>>(r.sa, r.sb, r.C, r.parent, r.own, r.best, r.tgt);
+    best_edge_kernel<1><<<grid_for(c, r.mmax), 256, 0, c->stream>>>(r.sa, r.sb, r.ss, r.ename, r.m, r.parent, r.own, r.best);
     HOP_LAUNCH(c);
-    hook_kernel<<<grid_for(c, r.cmax), 256, 0, c->stream>>>(r.C, r.own, r.best, r.tgt, r.parent, r.changed);
+    best_edge_kernel<2><<<grid_for(c, r.mmax), 256, 0, c->stream>>>(r.sa, r.sb, r.ss, r.ename, r.m, r.parent, r.own, r.best);
+    HOP_LAUNCH(c);
+    hook_kernel<<<grid_for(c, r.cmax), 256, 0, c->stream>>>(r.C, r.own, r.best, r.parent, r.changed);
     HOP_LAUNCH(c);
     compress_kernel<<<grid_for(c, r.cmax), 256, 0, c->stream>>>(r.parent, r.C);
     HOP_LAUNCH(c);
@@ -498,28 +470,23 @@ int merge_groups_graph(hop_ctx *c, const MergeGraphArgs &a)
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += align256(bytes); return o; };
     const size_t o_cid = take((n + 1) * 4), o_ckey = take(Cmax * 8), o_own = take(Cmax),
-                 o_parent = take(Cmax * 4), o_best = take(Cmax * 4), o_tgt = take(Cmax * 4),
+                 o_parent = take(Cmax * 4), o_bs = take(Cmax * 8), o_bn = take(Cmax * 8), o_tgt = take(Cmax * 4),
                  o_gpeak = take(Cmax * 8), o_flag = take((Cmax + 1) * 4), o_grank = take(Cmax * 4),
-                 o_ea = take(mmax * 4), o_eb = take(mmax * 4), o_sa = take(mmax * 4),
-                 o_sb = take(mmax * 4), o_ss = take(mmax * 8), o_k1 = take(mmax * 8),
-                 o_k1b = take(mmax * 8), o_v1 = take(mmax * 4), o_v1b = take(mmax * 4),
-                 o_gk = take(Cmax * 8), o_gkb = take(Cmax * 8), o_gv = take(Cmax * 4),
+                 o_ea = take(mmax * 4), o_eb = take(mmax * 4), o_name = take(mmax * 8), o_gk = take(Cmax * 8), o_gkb = take(Cmax * 8), o_gv = take(Cmax * 4),
                  o_gvb = take(Cmax * 4), o_start = take((a.B + 1) * 4);
-    const size_t o_tmp = take(std::max(radix_sort_scratch_bytes(mmax), radix_sort_scratch_bytes(Cmax)));
+    const size_t o_tmp = take(radix_sort_scratch_bytes(Cmax));
     char *base = (char *)ctx_buf(c, S_MERGE, off);
     if (!base) return HOP_ENOMEM;
     uint32_t *cid = (uint32_t *)(base + o_cid);
     uint64_t *ckey = (uint64_t *)(base + o_ckey);
     uint8_t *own = (uint8_t *)(base + o_own);
-    uint32_t *parent = (uint32_t *)(base + o_parent), *best = (uint32_t *)(base + o_best),
-             *tgt = (uint32_t *)(base + o_tgt), *flag = (uint32_t *)(base + o_flag),
-             *grank = (uint32_t *)(base + o_grank), *seg_start = (uint32_t *)(base + o_start);
+    uint32_t *parent = (uint32_t *)(base + o_parent), *tgt = (uint32_t *)(base + o_tgt),
+             *flag = (uint32_t *)(base + o_flag), *grank = (uint32_t *)(base + o_grank),
+             *seg_start = (uint32_t *)(base + o_start);
     unsigned long long *gpeak = (unsigned long long *)(base + o_gpeak);
-    uint32_t *ea = (uint32_t *)(base + o_ea), *eb = (uint32_t *)(base + o_eb),
-             *sa = (uint32_t *)(base + o_sa), *sb = (uint32_t *)(base + o_sb);
-    double *ss = (double *)(base + o_ss);
-    uint64_t *k1 = (uint64_t *)(base + o_k1), *k1b = (uint64_t *)(base + o_k1b);
-    uint32_t *v1 = (uint32_t *)(base + o_v1), *v1b = (uint32_t *)(base + o_v1b);
+    const Best best{(unsigned long long *)(base + o_bs), (unsigned long long *)(base + o_bn), tgt};
+    uint32_t *ea = (uint32_t *)(base + o_ea), *eb = (uint32_t *)(base + o_eb);
+    uint64_t *ename = (uint64_t *)(base + o_name);
     uint64_t *gk = (uint64_t *)(base + o_gk), *gkb = (uint64_t *)(base + o_gkb);
     uint32_t *gv = (uint32_t *)(base + o_gv), *gvb = (uint32_t *)(base + o_gvb);
     void *tmp = base + o_tmp;
@@ -534,22 +501,14 @@ int merge_groups_graph(hop_ctx *c, const MergeGraphArgs &a)
     root_list_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(a.chain, a.dkey, n, a.d_o, a.d_p, cid, ckey, own,
                                                             Cmax, c->d_err);
     HOP_LAUNCH(c);
-    // M3: strict edge order
-    edge_prep_kernel<<<grid_for(c, mmax), 256, 0, c->stream>>>(a.edge_key, a.edge_sum, a.m, n, a.chain, cid,
-                                                              a.dkey, a.d_o, ea, eb, k1, v1, c->d_err, Cmax);
-    HOP_LAUNCH(c);
-    rc = radix_sort_u64_dev(c, k1, k1b, v1, v1b, a.m, 0, 64, tmp);
-    if (rc) return rc;
-    edge_key2_kernel<<<grid_for(c, mmax), 256, 0, c->stream>>>(a.edge_sum, v1, a.m, k1);
-    HOP_LAUNCH(c);
-    rc = radix_sort_u64_dev(c, k1, k1b, v1, v1b, a.m, 0, 64, tmp);
-    if (rc) return rc;
-    edge_permute_kernel<<<grid_for(c, mmax), 256, 0, c->stream>>>(v1, a.m, ea, eb, a.edge_sum, sa, sb, ss);
+    // M3: endpoints and names of the edges
+    edge_prep_kernel<<<grid_for(c, mmax), 256, 0, c->stream>>>(a.edge_key, a.m, n, a.chain, cid, a.dkey, a.d_o, ea, eb,
+                                                              ename, c->d_err, Cmax);
     HOP_LAUNCH(c);
     // M4, M5: device-bounded rounds
     iota_kernel<<<grid_for(c, Cmax), 256, 0, c->stream>>>(parent, C);
     HOP_LAUNCH(c);
-    RoundArgs r{sa, sb, ss, a.m, C, 2.0 * (double)a.d_s, own, parent, best, tgt, d_changed, Cmax, mmax};
+    RoundArgs r{ea, eb, a.edge_sum, ename, a.m, C, 2.0 * (double)a.d_s, own, parent, best, d_changed, Cmax, mmax};
     rc = graph_while(c, d_changed, d_round1, kMaxRounds, kErrMergeLoop, proto_round, &r);
     if (rc) return rc;
     rc = graph_while(c, d_changed, d_round2, kMaxRounds, kErrMergeLoop, boruvka_round, &r);

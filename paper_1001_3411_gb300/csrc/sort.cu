@@ -317,6 +317,125 @@ __global__ void __launch_bounds__(kSortThreads, 3) radix_onesweep_kernel(
     }
 }
 
+// All passes of a sort of at most kSmallSort pairs in one launch of one block.
+// Each pass is that of the tiled sort: the warps rank their items (32 *
+// ITEMS consecutive ones, held in registers) per digit with ballots, a scan
+// over (digit, warp) places them, and they are exchanged through shared
+// memory.  Bound by latency: a pass of the tiled sort costs a launch, the
+// clearing of its status words and a look-back, 10 us whatever the size.
+// Measured in whole passes: 4,913 particles (6 passes here, 8 over the groups)
+// 760 -> 531 us, with the merge's edge sorts gone as well.
+constexpr int kSmallThreads = 512, kSmallWarps = kSmallThreads / 32;
+constexpr int kSmallItems = 16;
+constexpr int kSmallSort = kSmallThreads * kSmallItems;
+constexpr int small_sort_smem(int items) { return kSmallWarps * 256 * 2 + kSmallThreads * items * 12; }
+
+template <int ITEMS>
+__global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(uint64_t *__restrict__ keys, uint32_t *__restrict__ vals,
+                                                                   int n, int begin_bit, int npass)
+{
+    extern __shared__ __align__(16) unsigned char ss_raw[];
+    uint64_t *skey = (uint64_t *)ss_raw;
+    uint32_t *sval = (uint32_t *)(skey + kSmallThreads * ITEMS);
+    uint16_t *cnt = (uint16_t *)(sval + kSmallThreads * ITEMS);   // [warp][digit]
+    __shared__ uint32_t sw[33];
+    const uint32_t lane = lane_id(), warp = threadIdx.x >> 5, lt = lanemask_lt();
+    const int first = (int)warp * 32 * ITEMS + (int)lane;
+    uint64_t key[ITEMS];
+    uint32_t val[ITEMS];
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int i = first + r * 32;
+        key[r] = i < n ? keys[i] : 0ull;
+        val[r] = i < n ? vals[i] : 0u;
+    }
+    uint16_t *mine = cnt + warp * 256;
+    for (int p = 0; p < npass; ++p) {
+        const int shift = begin_bit + 8 * p;
+        for (int t = threadIdx.x; t < kSmallWarps * 256 / 8; t += kSmallThreads)
+            reinterpret_cast<uint4 *>(cnt)[t] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        uint32_t rnk[ITEMS];
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) {
+            const bool valid = first + r * 32 < n;
+            const uint32_t d = valid ? (uint32_t)((key[r] >> shift) & 255u) : 256u;
+            uint32_t peers = __ballot_sync(0xffffffffu, valid);
+            if (!valid) peers = ~peers;
+#pragma unroll
+            for (int b = 0; b < 8; ++b) {
+                const uint32_t vb = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+                peers &= ((d >> b) & 1u) ? vb : ~vb;
+            }
+            const uint32_t leader = __ffs(peers) - 1;
+            uint32_t prior = 0;
+            if (valid && lane == leader) {
+                prior = mine[d];
+                mine[d] = (uint16_t)(prior + __popc(peers));
+            }
+            prior = __shfl_sync(0xffffffffu, prior, leader);
+            rnk[r] = prior + __popc(peers & lt);
+            __syncwarp();
+        }
+        __syncthreads();
+        // digit threadIdx.x >> 1: half of the warps' runs each, then the
+        // digits' starts
+        {
+            static_assert(kSmallThreads == 2 * 256, "two threads per digit");
+            const int d = threadIdx.x >> 1, w0 = (threadIdx.x & 1) * (kSmallWarps / 2);
+            uint32_t c[kSmallWarps / 2], run = 0;
+#pragma unroll
+            for (int w = 0; w < kSmallWarps / 2; ++w) {
+                c[w] = cnt[(w0 + w) * 256 + d];
+                run += c[w];
+            }
+            uint32_t tot;
+            uint32_t at = block_exclusive_scan(run, sw, &tot);   // (digit, half) order
+#pragma unroll
+            for (int w = 0; w < kSmallWarps / 2; ++w) {
+                cnt[(w0 + w) * 256 + d] = (uint16_t)at;
+                at += c[w];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) {
+            if (first + r * 32 < n) {
+                const uint32_t to = mine[(uint32_t)((key[r] >> shift) & 255u)] + rnk[r];
+                skey[to] = key[r];
+                sval[to] = val[r];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < ITEMS; ++r) {
+            const int i = first + r * 32;
+            if (i < n) {
+                key[r] = skey[i];
+                val[r] = sval[i];
+            }
+        }
+        // (the next pass writes skey only after its own barriers)
+    }
+#pragma unroll
+    for (int r = 0; r < ITEMS; ++r) {
+        const int i = first + r * 32;
+        if (i < n) {
+            keys[i] = key[r];
+            vals[i] = val[r];
+        }
+    }
+}
+
+template <int ITEMS> int small_sort(hop_ctx *c, uint64_t *keys, uint32_t *vals, int n, int begin_bit, int npass)
+{
+    constexpr int smem = small_sort_smem(ITEMS);
+    HOP_CUDA(c, cudaFuncSetAttribute(small_sort_kernel<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    small_sort_kernel<ITEMS><<<1, kSmallThreads, smem, c->stream>>>(keys, vals, n, begin_bit, npass);
+    HOP_LAUNCH(c);
+    return HOP_OK;
+}
+
 __global__ void iota_kernel(uint32_t *out, int64_t n)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -392,7 +511,13 @@ size_t radix_sort_scratch_bytes(int64_t n)
 int radix_sort_u64(hop_ctx *c, uint64_t *&keys, uint64_t *&keys_alt, uint32_t *&vals,
                    uint32_t *&vals_alt, int64_t n, int begin_bit, int end_bit, void *scratch)
 {
-    if (n <= 1) return HOP_OK;
+    if (n <= 1 || end_bit <= begin_bit) return HOP_OK;
+    if (n <= kSmallSort) {
+        const int npass = (end_bit - begin_bit + 7) / 8;
+        if (npass > kMaxPasses) return ctx_fail(c, HOP_EINVAL, "radix sort over more than 64 key bits");
+        return n <= 4 * kSmallThreads ? small_sort<4>(c, keys, vals, (int)n, begin_bit, npass)
+                                      : small_sort<kSmallItems>(c, keys, vals, (int)n, begin_bit, npass);
+    }
     return radix_sort_u64_dev(c, keys, keys_alt, vals, vals_alt, DevCount{n, nullptr}, begin_bit,
                               end_bit, scratch);
 }
