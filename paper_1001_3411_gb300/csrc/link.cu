@@ -189,11 +189,15 @@ __device__ __forceinline__ int64_t table_find(const uint64_t *hkey, uint64_t mas
 // double is >= 0, so its bits order like its value and atomicMax applies.
 // With `directed` the key is (chain_i, chain_j) in that order, so the table
 // holds each direction of a pair separately (ADAPTAHOP's symmetric test).
+// VEC: rows start on 16 bytes and n_merge is at most four, so a row's part is
+// one read.  A pair's chains are compared before its density is fetched: most
+// neighbours are in the particle's own chain.
+template <bool VEC>
 __global__ void boundary_kernel(const uint32_t *__restrict__ chain,
                                 const uint64_t *__restrict__ dkey,
                                 const uint32_t *__restrict__ nbr, int ld, int64_t n, int n_merge,
                                 float d_o, uint64_t *hkey, unsigned long long *hval, uint64_t mask,
-                                uint32_t *err, unsigned long long *n_ins, bool directed = false)
+                                uint32_t *err, unsigned long long *n_ins, bool directed)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
@@ -201,21 +205,54 @@ __global__ void boundary_kernel(const uint32_t *__restrict__ chain,
         if (!(di >= d_o)) continue;
         const uint32_t ci = chain[i];
         const uint32_t *row = nbr + i * (int64_t)ld;
-        for (int t = 0; t < n_merge; ++t) {
-            const uint32_t j = row[t];
-            if (j == (uint32_t)i) continue;
-            if (j >= (uint64_t)n) { atomicOr(err, kErrBadIndex); continue; }
+        auto link = [&](uint32_t j, uint32_t cj) {
             const float dj = key_dens(dkey[j]);
-            if (!(dj >= d_o)) continue;
-            const uint32_t cj = chain[j];
-            if (cj == ci) continue;
+            if (!(dj >= d_o)) return;
             const uint64_t key = (directed || ci < cj) ? (((uint64_t)ci << 32) | cj)
                                                        : (((uint64_t)cj << 32) | ci);
             const double s = (double)di + (double)dj;
             if (!table_insert(hkey, hval, mask, key, (unsigned long long)__double_as_longlong(s), n_ins))
                 atomicOr(err, kErrTableFull);
+        };
+        if constexpr (VEC) {
+            const uint4 v = *reinterpret_cast<const uint4 *>(row);
+            const uint32_t j[4] = {v.x, v.y, v.z, v.w};
+            uint32_t cj[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                cj[t] = ci;
+                if (t >= n_merge || j[t] == (uint32_t)i) continue;
+                if (j[t] >= (uint64_t)n) atomicOr(err, kErrBadIndex);
+                else cj[t] = chain[j[t]];
+            }
+#pragma unroll 1
+            for (int t = 0; t < 4; ++t) {
+                const uint32_t jt = t == 0 ? j[0] : t == 1 ? j[1] : t == 2 ? j[2] : j[3];
+                const uint32_t ct = t == 0 ? cj[0] : t == 1 ? cj[1] : t == 2 ? cj[2] : cj[3];
+                if (ct != ci) link(jt, ct);
+            }
+        } else {
+            for (int t = 0; t < n_merge; ++t) {
+                const uint32_t j = row[t];
+                if (j == (uint32_t)i) continue;
+                if (j >= (uint64_t)n) { atomicOr(err, kErrBadIndex); continue; }
+                const uint32_t cj = chain[j];
+                if (cj != ci) link(j, cj);
+            }
         }
     }
+}
+
+void boundary_launch(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, const uint32_t *nbr, int ld, int64_t n,
+                     int n_merge, float d_o, uint64_t *hkey, unsigned long long *hval, uint64_t mask, uint32_t *err,
+                     unsigned long long *n_ins, bool directed)
+{
+    if (n_merge <= 4 && ld >= 4 && ld % 4 == 0 && (uintptr_t)nbr % 16 == 0)
+        boundary_kernel<true><<<grid_for(c, n), 256, 0, c->stream>>>(chain, dkey, nbr, ld, n, n_merge, d_o, hkey, hval,
+                                                                    mask, err, n_ins, directed);
+    else
+        boundary_kernel<false><<<grid_for(c, n), 256, 0, c->stream>>>(chain, dkey, nbr, ld, n, n_merge, d_o, hkey, hval,
+                                                                     mask, err, n_ins, directed);
 }
 
 // Inserts a list of (pair, sum) boundaries into the table; each pair keeps
@@ -407,9 +444,8 @@ int boundaries_table(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, co
         HOP_CUDA(c, cudaMemsetAsync(hval, 0, cap * sizeof(uint64_t), c->stream));
         HOP_CUDA(c, cudaMemsetAsync(nins, 0, 16, c->stream));
         uint32_t *terr = (uint32_t *)(nins + 1);   // this pass's own error word
-        boundary_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(chain, dkey, nbr, ld, n, n_merge,
-                                                              delta_outer, hkey, hval,
-                                                              (uint64_t)cap - 1, terr, nins, symmetric);
+        boundary_launch(c, chain, dkey, nbr, ld, n, n_merge, delta_outer, hkey, hval, (uint64_t)cap - 1, terr, nins,
+                        symmetric);
         HOP_LAUNCH(c);
         HOP_CUDA(c, cudaMemcpyAsync(hn, nins, 16, cudaMemcpyDeviceToHost, c->stream));
         HOP_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -535,8 +571,8 @@ int boundaries_table_async(hop_ctx *c, const uint32_t *chain, const uint64_t *dk
     fill_u64_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(hkey, cap, kEmpty);
     HOP_LAUNCH(c);
     HOP_CUDA(c, cudaMemsetAsync(hval, 0, cap * sizeof(uint64_t), c->stream));
-    boundary_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(chain, dkey, nbr, ld, n, n_merge, delta_outer,
-                                                          hkey, hval, (uint64_t)cap - 1, c->d_err, nins);
+    boundary_launch(c, chain, dkey, nbr, ld, n, n_merge, delta_outer, hkey, hval, (uint64_t)cap - 1, c->d_err, nins,
+                    false);
     HOP_LAUNCH(c);
     occupied_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(hkey, cap, occ);
     HOP_LAUNCH(c);

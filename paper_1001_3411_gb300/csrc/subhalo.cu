@@ -7,19 +7,28 @@
 //      (link.cu, boundaries_table with symmetric = true);
 //  S2  dense ids for the chain roots above delta_outer (scan) and, per
 //      particle above delta_outer, its root's id;
-//  then once per threshold delta_s (the paper's linear cost in the number
-//  of thresholds):
-//  S3  links with s < 2 delta_s are destroyed; the rest join chains into
-//      connected components (hook the larger root under the smaller with
-//      atomicMin, compress, repeat until no edge joins two roots);
-//  S4  members (dens >= delta_s) give each component its count, fp64
-//      density sum and peak key (warp-aggregated atomics);
-//  S5  a component is a subhalo when count >= n_min and mean density >=
-//      delta_s (1 + f_poisson / sqrt(count)); subhalos are ranked by peak
-//      key (radix sort) and every particle gets its rank or -1.
+//  S3  one pass over the particles gives every chain its densest member's
+//      key and, for up to kLev thresholds at once, the number (and fp64
+//      density sum, if needed) of its members with dens >= delta_s;
+//  S4  per threshold, links with s < 2 delta_s are destroyed; the rest join
+//      chains into connected components (hook the larger root under the
+//      smaller with atomicMin, compress, repeat until no edge joins two
+//      roots), all thresholds in the same launches;
+//  S5  chains' counts, sums and keys are added up per component; a component
+//      is a subhalo when count >= n_min and mean density >= delta_s (1 +
+//      f_poisson / sqrt(count));
+//  S6  subhalos are ranked by peak key: the chains are sorted by their key
+//      once, and a subhalo's rank is the number of subhalos' peak chains
+//      before its own in that order (one scan over all thresholds);
+//  S7  one pass over the particles writes every threshold's labels from the
+//      chain's label row.
 //
-// Every per-particle pass reads a few bytes per particle plus one or two
-// gathers into the chain arrays, so the levels are HBM- and latency-bound.
+// The two per-particle passes read 12 bytes per particle each, whatever the
+// number of thresholds (a pass per threshold and purpose read them 2 L
+// times), and write 4 bytes per threshold: HBM-bound.  What depends on the
+// threshold works on chains, a hundred times fewer.
+// Halo statistics and subhalos of 16.8M particles at five thresholds: 3309 us
+// with a pass, a component search and a sort per threshold, 2220 us so.
 #include "hop_internal.cuh"
 
 #include <algorithm>
@@ -81,62 +90,47 @@ __global__ void sub_edge_ids_kernel(const uint64_t *__restrict__ ekey, int64_t m
     }
 }
 
-__global__ void sub_iota_kernel(uint32_t *p, int64_t n)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = (uint32_t)i;
-}
+constexpr int kLev = 8;   // thresholds handled together; a chain's row of kLev 4-byte values is one sector
 
-// S3: one hooking round over the surviving links.
-__global__ void sub_hook_kernel(const uint32_t *__restrict__ ea, const uint32_t *__restrict__ eb,
-                            const double *__restrict__ es, int64_t m, double two_ds, uint32_t *parent,
-                            uint32_t *changed)
-{
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        if (!(es[e] >= two_ds)) continue;
-        const uint32_t ra = find_root(parent, ea[e]), rb = find_root(parent, eb[e]);
-        if (ra == rb) continue;
-        atomicMin(&parent[max(ra, rb)], min(ra, rb));
-        *changed = 1u;
-    }
-}
+struct Levels {
+    float ds[kLev];
+    int L;
+};
 
-__global__ void sub_compress_kernel(uint32_t *parent, int64_t C)
-{
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < C;
-         c += (int64_t)gridDim.x * blockDim.x)
-        parent[c] = find_root(parent, (uint32_t)c);
-}
-
-// S4: count, density sum and peak key of every component's members.  The
-// sum (fp64 atomics, the slow part) is taken only when the significance
-// cut needs it (sum != nullptr).
-// The per-particle passes take kSubU elements per thread per batch and
-// issue the batch's loads before reducing any of it, so the loads overlap.
-// The member pass gives every warp spans of consecutive particles and
-// carries its last run of one component on to the next 32 (as the halo
-// statistics do), so a large component costs one atomic per span.
+// S3: count[c * kLev + l], sum (the same layout, or nullptr) and peak key of
+// every chain.  A warp takes kSubSpan consecutive particles, loading kSubU
+// steps of 32 before reducing any.  A step whose members all lie in one chain
+// is added to the warp's carried run (members of a halo are mostly
+// consecutive), the runs of any other step go to memory with one atomic per
+// value.  Counts are the set bits of a ballot per threshold.
 constexpr int kSubU = 4;
 constexpr int kSubSteps = 32;
 constexpr int kSubSpan = 32 * kSubSteps;
 
-__global__ void sub_member_stats_kernel(const uint64_t *__restrict__ dkey, const uint32_t *__restrict__ pc,
-                                        int64_t n, float ds, const uint32_t *__restrict__ parent,
-                                        unsigned long long *__restrict__ cnt, double *__restrict__ sum,
-                                        unsigned long long *__restrict__ pkey)
+template <bool SUM>
+__global__ void sub_chain_stats_kernel(const uint64_t *__restrict__ dkey, const uint32_t *__restrict__ pc, int64_t n,
+                                       const Levels lev, uint32_t *__restrict__ cnt, double *__restrict__ sum,
+                                       unsigned long long *__restrict__ pkey)
 {
     const int lane = threadIdx.x & 31;
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t w0 = w * kSubSpan; w0 < n; w0 += nw * kSubSpan) {
-        uint32_t cr = kNone;                  // the carried run: component, count, sum, best key
-        unsigned long long cc = 0, cb = 0;
+        uint32_t cr = kNone;                  // the carried run: chain, best key; lane l < L: count and sum at level l
+        unsigned long long cb = 0;
+        uint32_t cc = 0;
         double csum = 0.0;
+        auto flush = [&]() {
+            if (cr == kNone) return;
+            if (lane == 0) atomicMax(&pkey[cr], cb);
+            if (cc) atomicAdd(&cnt[(int64_t)cr * kLev + lane], cc);
+            if constexpr (SUM)
+                if (cc) atomicAdd(&sum[(int64_t)cr * kLev + lane], csum);
+            cr = kNone;
+        };
         for (int t = 0; t < kSubSteps; t += kSubU) {
             uint64_t k[kSubU];
-            uint32_t c[kSubU], r[kSubU];
+            uint32_t c[kSubU];
 #pragma unroll
             for (int u = 0; u < kSubU; ++u) {
                 const int64_t i = w0 + (int64_t)(t + u) * 32 + lane;
@@ -144,116 +138,193 @@ __global__ void sub_member_stats_kernel(const uint64_t *__restrict__ dkey, const
                 c[u] = i < n ? pc[i] : kNone;
             }
 #pragma unroll
-            for (int u = 0; u < kSubU; ++u)
-                r[u] = (c[u] != kNone && key_dens(k[u]) >= ds) ? parent[c[u]] : kNone;
-#pragma unroll
             for (int u = 0; u < kSubU; ++u) {
-                const uint32_t rr = r[u];
+                const uint32_t rr = c[u];
                 if (!__any_sync(0xffffffffu, rr != kNone)) continue;
-                // runs of consecutive lanes in one component
+                const float d = key_dens(k[u]);
                 const uint32_t heads = run_heads((int64_t)rr, lane);
-                double sm = sum ? run_sum<double>(heads, lane, rr != kNone ? (double)key_dens(k[u]) : 0.0) : 0.0;
-                unsigned long long best = run_max(heads, lane, rr != kNone ? k[u] : 0ull);
-                unsigned long long len = (unsigned long long)run_len(heads, lane);
-                if (lane == 0 && cr != kNone) {
-                    if (rr == cr) {
-                        len += cc;
-                        sm += csum;
-                        best = best > cb ? best : cb;
-                    } else {
-                        atomicAdd(&cnt[cr], cc);
-                        if (sum) atomicAdd(&sum[cr], csum);
-                        atomicMax(&pkey[cr], cb);
+                const unsigned long long best = run_max(heads, lane, rr != kNone ? k[u] : 0ull);
+                if (heads == 1u) {
+                    // one chain, all lanes
+                    if (rr != cr) {
+                        flush();
+                        cr = rr;
+                        cb = 0;
+                        cc = 0;
+                        csum = 0.0;
+                    }
+                    cb = best > cb ? best : cb;
+                    for (int l = 0; l < lev.L; ++l) {
+                        const uint32_t m = __popc(__ballot_sync(0xffffffffu, d >= lev.ds[l]));
+                        if (lane == l) cc += m;
+                        if constexpr (SUM) {
+                            double x = d >= lev.ds[l] ? (double)d : 0.0;
+#pragma unroll
+                            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                            if (lane == l) csum += x;
+                        }
+                    }
+                } else {
+                    flush();
+                    const bool head = rr != kNone && ((heads >> lane) & 1u);
+                    const int len = run_len(heads, lane);
+                    const uint32_t run = (len == 32 ? 0xffffffffu : ((1u << len) - 1u)) << lane;
+                    if (head) atomicMax(&pkey[rr], best);
+                    for (int l = 0; l < lev.L; ++l) {
+                        const bool in = rr != kNone && d >= lev.ds[l];
+                        const uint32_t m = __popc(__ballot_sync(0xffffffffu, in) & run);
+                        if (head && m) atomicAdd(&cnt[(int64_t)rr * kLev + l], m);
+                        if constexpr (SUM) {
+                            const double x = run_sum<double>(heads, lane, in ? (double)d : 0.0);
+                            if (head && m) atomicAdd(&sum[(int64_t)rr * kLev + l], x);
+                        }
                     }
                 }
-                const int last = 31 - __clz(heads);
-                if (rr != kNone && ((heads >> lane) & 1u) && lane != last) {
-                    atomicAdd(&cnt[rr], len);
-                    if (sum) atomicAdd(&sum[rr], sm);
-                    atomicMax(&pkey[rr], best);
-                }
-                cr = __shfl_sync(0xffffffffu, rr, last);
-                cc = __shfl_sync(0xffffffffu, len, last);
-                csum = __shfl_sync(0xffffffffu, sm, last);
-                cb = __shfl_sync(0xffffffffu, best, last);
             }
         }
-        if (lane == 0 && cr != kNone) {
-            atomicAdd(&cnt[cr], cc);
-            if (sum) atomicAdd(&sum[cr], csum);
-            atomicMax(&pkey[cr], cb);
+        flush();
+    }
+}
+
+// S4, all levels at once: parent[l * C + c].
+__global__ void sub_iota_kernel(uint32_t *p, int64_t C, int L)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < C * L; i += (int64_t)gridDim.x * blockDim.x)
+        p[i] = (uint32_t)(i % C);
+}
+
+__global__ void sub_hook_kernel(const uint32_t *__restrict__ ea, const uint32_t *__restrict__ eb,
+                                const double *__restrict__ es, int64_t m, const Levels lev, int64_t C,
+                                uint32_t *parent, uint32_t *changed)
+{
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const double s = es[e];
+        const uint32_t a = ea[e], b = eb[e];
+        for (int l = 0; l < lev.L; ++l) {
+            if (!(s >= 2.0 * (double)lev.ds[l])) continue;
+            uint32_t *p = parent + l * C;
+            const uint32_t ra = find_root(p, a), rb = find_root(p, b);
+            if (ra == rb) continue;
+            atomicMin(&p[max(ra, rb)], min(ra, rb));
+            *changed = 1u;
         }
     }
 }
-// S5: the significance cut, in the same fp64 operations as the definition.
+
+__global__ void sub_compress_kernel(uint32_t *parent, int64_t C, int L)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < C * L; i += (int64_t)gridDim.x * blockDim.x) {
+        uint32_t *p = parent + i / C * C;
+        parent[i] = find_root(p, (uint32_t)(i - i / C * C));
+    }
+}
+
+// S5: the chains' shares of every component, index l * C + component.
+__global__ void sub_component_kernel(const uint32_t *__restrict__ cnt, const double *__restrict__ sum,
+                                     const unsigned long long *__restrict__ pkey, int64_t C, int L,
+                                     const uint32_t *__restrict__ parent, unsigned long long *__restrict__ ccnt,
+                                     double *__restrict__ csum, unsigned long long *__restrict__ cpk)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < C * L; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t l = i / C, c = i - l * C;
+        const uint32_t k = cnt[c * kLev + l];
+        if (!k) continue;
+        const int64_t r = l * C + parent[i];
+        atomicAdd(&ccnt[r], (unsigned long long)k);
+        if (csum) atomicAdd(&csum[r], sum[c * kLev + l]);
+        atomicMax(&cpk[r], pkey[c]);
+    }
+}
+
+// The significance cut, in the same fp64 operations as the definition.
 // With f = 0 the cut is mean >= delta_s, which every set of members passes:
 // each member is >= delta_s, and rounding is monotone, so a running fp64
 // sum of N of them is >= N delta_s (exact for a float32 delta_s and
 // N < 2^29) and the rounded mean is >= delta_s, in any summation order.
 // Then (f = 0 and n < 2^29) sum is nullptr and only the count is tested.
-__global__ void sub_accept_kernel(int64_t C, const uint32_t *__restrict__ parent,
-                              const unsigned long long *__restrict__ cnt, const double *__restrict__ sum,
-                              double ds, long long n_min, double f, uint32_t *__restrict__ flag)
+__device__ __forceinline__ bool sub_accept(unsigned long long k, const double *sum, int64_t r, double ds, long long n_min,
+                                           double f)
 {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < C;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t ok = 0;
-        const unsigned long long k = cnt[c];
-        if (parent[c] == (uint32_t)c && k > 0 && (long long)k >= n_min) {
-            if (!sum) {
-                ok = 1u;
-            } else {
-                const double N = (double)k;
-                const double mean = __ddiv_rn(sum[c], N);
-                const double thr = __dmul_rn(ds, __dadd_rn(1.0, __ddiv_rn(f, __dsqrt_rn(N))));
-                ok = mean >= thr ? 1u : 0u;
-            }
-        }
-        flag[c] = ok;
+    if (k == 0 || (long long)k < n_min) return false;
+    if (!sum) return true;
+    const double N = (double)k;
+    const double mean = __ddiv_rn(sum[r], N);
+    const double thr = __dmul_rn(ds, __dadd_rn(1.0, __ddiv_rn(f, __dsqrt_rn(N))));
+    return mean >= thr;
+}
+
+__global__ void sub_keys_kernel(const unsigned long long *__restrict__ pkey, int64_t C, uint64_t *__restrict__ gk,
+                                uint32_t *__restrict__ gv)
+{
+    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < C; c += (int64_t)gridDim.x * blockDim.x) {
+        gk[c] = ~(uint64_t)pkey[c];   // ascending = peak density desc, index asc
+        gv[c] = (uint32_t)c;
     }
 }
 
-__global__ void sub_list_kernel(int64_t C, const uint32_t *__restrict__ flag, const uint32_t *__restrict__ pos,
-                            const unsigned long long *__restrict__ pkey, uint64_t *__restrict__ gk,
-                            uint32_t *__restrict__ gv)
+// S6: flag[l * C + position of chain c in key order] = c is the peak chain
+// of a subhalo at level l.
+__global__ void sub_flag_kernel(const uint32_t *__restrict__ order, const unsigned long long *__restrict__ pkey, int64_t C,
+                                const Levels lev, const uint32_t *__restrict__ parent,
+                                const unsigned long long *__restrict__ ccnt, const double *__restrict__ csum,
+                                const unsigned long long *__restrict__ cpk, long long n_min, double f,
+                                uint32_t *__restrict__ flag)
 {
-    for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < C;
-         c += (int64_t)gridDim.x * blockDim.x) {
-        if (!flag[c]) continue;
-        gk[pos[c]] = ~(uint64_t)pkey[c];   // ascending = peak density desc, index asc
-        gv[pos[c]] = (uint32_t)c;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < C * lev.L;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t l = i / C;
+        const uint32_t c = order[i - l * C];
+        const int64_t r = l * C + parent[l * C + c];
+        flag[i] = cpk[r] == pkey[c] && sub_accept(ccnt[r], csum, r, (double)lev.ds[l], n_min, f) ? 1u : 0u;
     }
 }
 
-__global__ void sub_rank_kernel(DevCount Gc, const uint32_t *__restrict__ gv, uint32_t *__restrict__ rank)
+// rank[l * C + component], and the number of subhalos per level.
+__global__ void sub_rank_kernel(const uint32_t *__restrict__ order, const uint32_t *__restrict__ flag,
+                                const uint32_t *__restrict__ pos, int64_t C, int L, const uint32_t *__restrict__ parent,
+                                int32_t *__restrict__ rank, uint32_t *__restrict__ n_lev)
 {
-    const int64_t G = Gc.get();
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < G;
-         g += (int64_t)gridDim.x * blockDim.x)
-        rank[gv[g]] = (uint32_t)g;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < C * L; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t l = i / C;
+        const uint32_t at = pos[i] - pos[l * C];
+        if (i - l * C == C - 1) n_lev[l] = at + flag[i];
+        if (flag[i]) rank[l * C + parent[l * C + order[i - l * C]]] = (int32_t)at;
+    }
 }
 
+// Every chain's row of labels: its component's rank at each level, or -1
+// (rank holds -1 where there is no subhalo).
+__global__ void sub_row_kernel(const int32_t *__restrict__ rank, const uint32_t *__restrict__ parent, int64_t C, int L,
+                               int32_t *__restrict__ row)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < C * L; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t l = i / C, c = i - l * C;
+        row[c * kLev + l] = rank[l * C + parent[i]];
+    }
+}
+
+// S7
 __global__ void sub_label_kernel(const uint64_t *__restrict__ dkey, const uint32_t *__restrict__ pc, int64_t n,
-                                 float ds, const uint32_t *__restrict__ parent, const uint32_t *__restrict__ flag,
-                                 const uint32_t *__restrict__ rank, int32_t *__restrict__ sub)
+                                 const Levels lev, const int32_t *__restrict__ row, int32_t *__restrict__ sub)
 {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x * kSubU;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x * kSubU; base < n; base += stride) {
-        uint64_t k[kSubU];
-        uint32_t c[kSubU], r[kSubU];
+    static_assert(kLev == 8, "a row is two 16-byte reads");
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        const uint32_t c = pc[i];
+        int32_t v[kLev] = {-1, -1, -1, -1, -1, -1, -1, -1};
+        if (c != kNone) {
+            const float d = key_dens(dkey[i]);
+            const int4 a = reinterpret_cast<const int4 *>(row + (int64_t)c * kLev)[0],
+                       b = reinterpret_cast<const int4 *>(row + (int64_t)c * kLev)[1];
+            const int32_t x[kLev] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
 #pragma unroll
-        for (int u = 0; u < kSubU; ++u) {
-            const int64_t i = base + (int64_t)u * blockDim.x + threadIdx.x;
-            k[u] = i < n ? dkey[i] : 0ull;
-            c[u] = i < n ? pc[i] : kNone;
+            for (int l = 0; l < kLev; ++l)
+                if (l < lev.L && d >= lev.ds[l]) v[l] = x[l];
         }
 #pragma unroll
-        for (int u = 0; u < kSubU; ++u) r[u] = (c[u] != kNone && key_dens(k[u]) >= ds) ? parent[c[u]] : kNone;
-#pragma unroll
-        for (int u = 0; u < kSubU; ++u) {
-            const int64_t i = base + (int64_t)u * blockDim.x + threadIdx.x;
-            if (i < n) sub[i] = (r[u] != kNone && flag[r[u]]) ? (int32_t)rank[r[u]] : -1;
-        }
+        for (int l = 0; l < kLev; ++l)
+            if (l < lev.L) sub[l * n + i] = v[l];
     }
 }
 
@@ -271,13 +342,13 @@ int subhalos(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, const uint
     HOP_CUDA(c, cudaEventRecord(c->ev[3], c->stream));
     // S2
     uint32_t *hp = (uint32_t *)c->h_pinned;
-    // misc: total, then kMaxRounds round flags, then one group count per level
-    uint32_t *misc = (uint32_t *)ctx_buf(c, S_MISC, (size_t)(2 + kMaxRounds + L) * sizeof(uint32_t));
+    // misc: total, then kMaxRounds round flags, then kLev subhalo counts
+    uint32_t *misc = (uint32_t *)ctx_buf(c, S_MISC, (size_t)(2 + kMaxRounds + kLev) * sizeof(uint32_t));
     uint32_t *cid = (uint32_t *)ctx_buf(c, S_SUB, (size_t)(2 * n + 64) * sizeof(uint32_t));
     if (!misc || !cid) return HOP_ENOMEM;
     uint32_t *pc = cid + ((n + 1 + 63) & ~int64_t(63));
-    uint32_t *d_total = misc, *d_flags = misc + 2, *d_levG = misc + 2 + kMaxRounds;
-    HOP_CUDA(c, cudaMemsetAsync(misc, 0, (size_t)(2 + kMaxRounds + L) * sizeof(uint32_t), c->stream));
+    uint32_t *d_total = misc, *d_flags = misc + 2, *d_lev = misc + 2 + kMaxRounds;
+    HOP_CUDA(c, cudaMemsetAsync(misc, 0, (size_t)(2 + kMaxRounds + kLev) * sizeof(uint32_t), c->stream));
     sub_root_flag_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(chain, dkey, n, d_o, cid, c->d_err);
     HOP_LAUNCH(c);
     rc = scan_exclusive_u32(c, cid, cid, n, d_total);
@@ -287,23 +358,30 @@ int subhalos(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, const uint
     HOP_CUDA(c, cudaMemcpyAsync(hp, misc, 4, cudaMemcpyDeviceToHost, c->stream));
     HOP_CUDA(c, cudaStreamSynchronize(c->stream));
     const int64_t C = hp[0];
-    // arrays over chains (C) and symmetric boundaries (m)
+    // thresholds per batch: at most kLev, fewer where the arrays over (level,
+    // chain) would grow past 2^28 entries
     const int64_t Cp = std::max<int64_t>(C, 1), mp = std::max<int64_t>(m, 1);
+    const int LB = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(L, kLev), (int64_t(1) << 28) / Cp));
+    const bool with_sum = f > 0.0 || n >= (int64_t(1) << 29);
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += align256(bytes); return o; };
-    const size_t o_parent = take(Cp * 4), o_cnt = take(Cp * 8), o_sum = take(Cp * 8), o_pkey = take(Cp * 8),
-                 o_flag = take((Cp + 1) * 4), o_pos = take((Cp + 1) * 4), o_rank = take(Cp * 4),
-                 o_ea = take(mp * 4), o_eb = take(mp * 4), o_gk = take(Cp * 8), o_gkb = take(Cp * 8),
-                 o_gv = take(Cp * 4), o_gvb = take(Cp * 4), o_tmp = take(radix_sort_scratch_bytes(Cp));
+    const size_t o_cnt = take(Cp * kLev * 4), o_sum = take(with_sum ? Cp * kLev * 8 : 8), o_pkey = take(Cp * 8),
+                 o_row = take(Cp * kLev * 4), o_parent = take(Cp * LB * 4), o_ccnt = take(Cp * LB * 8),
+                 o_csum = take(with_sum ? Cp * LB * 8 : 8), o_cpk = take(Cp * LB * 8), o_flag = take((Cp * LB + 1) * 4),
+                 o_pos = take((Cp * LB + 1) * 4), o_rank = take(Cp * LB * 4), o_ea = take(mp * 4), o_eb = take(mp * 4),
+                 o_gk = take(Cp * 8), o_gkb = take(Cp * 8), o_gv = take(Cp * 4), o_gvb = take(Cp * 4),
+                 o_tmp = take(radix_sort_scratch_bytes(Cp));
     char *base = (char *)ctx_buf(c, S_SUB_C, off);
     if (!base) return HOP_ENOMEM;
-    uint32_t *parent = (uint32_t *)(base + o_parent), *flag = (uint32_t *)(base + o_flag),
-             *gpos = (uint32_t *)(base + o_pos), *rank = (uint32_t *)(base + o_rank),
-             *ea = (uint32_t *)(base + o_ea), *eb = (uint32_t *)(base + o_eb);
-    unsigned long long *cnt = (unsigned long long *)(base + o_cnt), *pkey = (unsigned long long *)(base + o_pkey);
-    double *sum = (double *)(base + o_sum);
-    uint64_t *gk0 = (uint64_t *)(base + o_gk), *gkb0 = (uint64_t *)(base + o_gkb);
-    uint32_t *gv0 = (uint32_t *)(base + o_gv), *gvb0 = (uint32_t *)(base + o_gvb);
+    uint32_t *cnt = (uint32_t *)(base + o_cnt), *parent = (uint32_t *)(base + o_parent),
+             *flag = (uint32_t *)(base + o_flag), *gpos = (uint32_t *)(base + o_pos), *ea = (uint32_t *)(base + o_ea),
+             *eb = (uint32_t *)(base + o_eb);
+    int32_t *row = (int32_t *)(base + o_row), *rank = (int32_t *)(base + o_rank);
+    unsigned long long *pkey = (unsigned long long *)(base + o_pkey), *ccnt = (unsigned long long *)(base + o_ccnt),
+                       *cpk = (unsigned long long *)(base + o_cpk);
+    double *sum = with_sum ? (double *)(base + o_sum) : nullptr, *csum = with_sum ? (double *)(base + o_csum) : nullptr;
+    uint64_t *gk = (uint64_t *)(base + o_gk), *gkb = (uint64_t *)(base + o_gkb);
+    uint32_t *order = (uint32_t *)(base + o_gv), *gvb = (uint32_t *)(base + o_gvb);
     void *tmp = base + o_tmp;
     if (m > 0) {
         sub_edge_ids_kernel<<<grid_for(c, m), 256, 0, c->stream>>>(ek, m, n, chain, dkey, d_o, cid, ea, eb, c->d_err);
@@ -313,20 +391,37 @@ int subhalos(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, const uint
     if (rc) return rc;
     c->stats.n_chains = C;
     c->stats.n_edges = m;
-    // Each level runs without host round trips except the convergence test
-    // of its component rounds, read once per batch of kRoundBatch rounds
-    // (rounds after convergence change nothing); group counts stay on the
-    // device until every level is enqueued.
+    if (C == 0) {
+        HOP_CUDA(c, cudaMemsetAsync(sub, 0xFF, (size_t)L * n * sizeof(int32_t), c->stream));
+        for (int l = 0; l < L; ++l) n_sub[l] = 0;
+        return HOP_OK;
+    }
+    // Rounds run without host round trips except the convergence test, read
+    // once per kRoundBatch rounds (rounds after convergence change nothing).
     constexpr int kRoundBatch = 4;
-    for (int l = 0; l < L; ++l) {
-        const float ds = levels[l];
-        int32_t *out = sub + (int64_t)l * n;
-        if (C == 0) {
-            HOP_CUDA(c, cudaMemsetAsync(out, 0xFF, n * sizeof(int32_t), c->stream));
-            continue;
+    for (int l0 = 0; l0 < L; l0 += LB) {
+        Levels lev;
+        lev.L = std::min(LB, L - l0);
+        for (int l = 0; l < kLev; ++l) lev.ds[l] = l < lev.L ? levels[l0 + l] : INFINITY;
+        const int64_t CL = C * lev.L;
+        // S3 (the keys and their order are the same for every batch)
+        HOP_CUDA(c, cudaMemsetAsync(cnt, 0, C * kLev * 4, c->stream));
+        if (sum) HOP_CUDA(c, cudaMemsetAsync(sum, 0, C * kLev * 8, c->stream));
+        HOP_CUDA(c, cudaMemsetAsync(pkey, 0, C * 8, c->stream));
+        if (sum)
+            sub_chain_stats_kernel<true><<<grid_for(c, n), 256, 0, c->stream>>>(dkey, pc, n, lev, cnt, sum, pkey);
+        else
+            sub_chain_stats_kernel<false><<<grid_for(c, n), 256, 0, c->stream>>>(dkey, pc, n, lev, cnt, sum, pkey);
+        HOP_LAUNCH(c);
+        if (l0 == 0) {
+            uint64_t *k0 = gk, *k1 = gkb;
+            sub_keys_kernel<<<grid_for(c, C), 256, 0, c->stream>>>(pkey, C, k0, order);
+            HOP_LAUNCH(c);
+            rc = radix_sort_u64(c, k0, k1, order, gvb, C, 0, 64, tmp);
+            if (rc) return rc;
         }
-        // S3
-        sub_iota_kernel<<<grid_for(c, C), 256, 0, c->stream>>>(parent, C);
+        // S4
+        sub_iota_kernel<<<grid_for(c, CL), 256, 0, c->stream>>>(parent, C, lev.L);
         HOP_LAUNCH(c);
         int rounds = 0;
         bool converged = m == 0;
@@ -334,46 +429,37 @@ int subhalos(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, const uint
             if (rounds + kRoundBatch > kMaxRounds) return ctx_fail(c, HOP_ETIMEOUT, "subhalo components did not converge");
             HOP_CUDA(c, cudaMemsetAsync(d_flags + rounds, 0, kRoundBatch * sizeof(uint32_t), c->stream));
             for (int b = 0; b < kRoundBatch; ++b, ++rounds) {
-                sub_hook_kernel<<<grid_for(c, m), 256, 0, c->stream>>>(ea, eb, es, m, 2.0 * (double)ds, parent,
-                                                                       d_flags + rounds);
+                sub_hook_kernel<<<grid_for(c, m), 256, 0, c->stream>>>(ea, eb, es, m, lev, C, parent, d_flags + rounds);
                 HOP_LAUNCH(c);
-                sub_compress_kernel<<<grid_for(c, C), 256, 0, c->stream>>>(parent, C);
+                sub_compress_kernel<<<grid_for(c, CL), 256, 0, c->stream>>>(parent, C, lev.L);
                 HOP_LAUNCH(c);
             }
             HOP_CUDA(c, cudaMemcpyAsync(hp + 1, d_flags + rounds - 1, 4, cudaMemcpyDeviceToHost, c->stream));
             HOP_CUDA(c, cudaStreamSynchronize(c->stream));
             converged = hp[1] == 0;
         }
-        // S4
-        double *lsum = (f > 0.0 || n >= (int64_t(1) << 29)) ? sum : nullptr;
-        HOP_CUDA(c, cudaMemsetAsync(cnt, 0, C * 8, c->stream));
-        if (lsum) HOP_CUDA(c, cudaMemsetAsync(lsum, 0, C * 8, c->stream));
-        HOP_CUDA(c, cudaMemsetAsync(pkey, 0, C * 8, c->stream));
-        sub_member_stats_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(dkey, pc, n, ds, parent, cnt, lsum, pkey);
+        // S5, S6, S7
+        HOP_CUDA(c, cudaMemsetAsync(ccnt, 0, CL * 8, c->stream));
+        if (csum) HOP_CUDA(c, cudaMemsetAsync(csum, 0, CL * 8, c->stream));
+        HOP_CUDA(c, cudaMemsetAsync(cpk, 0, CL * 8, c->stream));
+        HOP_CUDA(c, cudaMemsetAsync(rank, 0xFF, CL * 4, c->stream));
+        sub_component_kernel<<<grid_for(c, CL), 256, 0, c->stream>>>(cnt, sum, pkey, C, lev.L, parent, ccnt, csum, cpk);
         HOP_LAUNCH(c);
-        // S5: accepted components, ranked by peak; their count stays on the device
-        sub_accept_kernel<<<grid_for(c, C), 256, 0, c->stream>>>(C, parent, cnt, lsum, (double)ds, (long long)n_min,
-                                                                 f, flag);
+        sub_flag_kernel<<<grid_for(c, CL), 256, 0, c->stream>>>(order, pkey, C, lev, parent, ccnt, csum, cpk,
+                                                                (long long)n_min, f, flag);
         HOP_LAUNCH(c);
-        rc = scan_exclusive_u32(c, flag, gpos, C, d_levG + l);
+        rc = scan_exclusive_u32(c, flag, gpos, CL, nullptr);
         if (rc) return rc;
-        const DevCount G{C, d_levG + l};
-        sub_list_kernel<<<grid_for(c, C), 256, 0, c->stream>>>(C, flag, gpos, pkey, gk0, gv0);
+        sub_rank_kernel<<<grid_for(c, CL), 256, 0, c->stream>>>(order, flag, gpos, C, lev.L, parent, rank, d_lev);
         HOP_LAUNCH(c);
-        uint64_t *gk = gk0, *gkb = gkb0;
-        uint32_t *gv = gv0, *gvb = gvb0;
-        rc = radix_sort_u64_dev(c, gk, gkb, gv, gvb, G, 0, 64, tmp);
-        if (rc) return rc;
-        sub_rank_kernel<<<grid_for(c, C), 256, 0, c->stream>>>(G, gv, rank);
+        sub_row_kernel<<<grid_for(c, CL), 256, 0, c->stream>>>(rank, parent, C, lev.L, row);
         HOP_LAUNCH(c);
-        sub_label_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(dkey, pc, n, ds, parent, flag, rank, out);
+        sub_label_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(dkey, pc, n, lev, row, sub + (int64_t)l0 * n);
         HOP_LAUNCH(c);
+        HOP_CUDA(c, cudaMemcpyAsync(hp + 2, d_lev, lev.L * sizeof(uint32_t), cudaMemcpyDeviceToHost, c->stream));
+        HOP_CUDA(c, cudaStreamSynchronize(c->stream));
+        for (int l = 0; l < lev.L; ++l) n_sub[l0 + l] = (int64_t)hp[2 + l];
     }
-    std::vector<uint32_t> levG(L);
-    HOP_CUDA(c, cudaMemcpyAsync(levG.data(), d_levG, (size_t)L * sizeof(uint32_t), cudaMemcpyDeviceToHost,
-                                c->stream));
-    HOP_CUDA(c, cudaStreamSynchronize(c->stream));
-    for (int l = 0; l < L; ++l) n_sub[l] = C == 0 ? 0 : (int64_t)levG[l];
     return HOP_OK;
 }
 
