@@ -28,7 +28,7 @@
 // times), and write 4 bytes per threshold: HBM-bound.  What depends on the
 // threshold works on chains, a hundred times fewer.
 // Halo statistics and subhalos of 16.8M particles at five thresholds: 3309 us
-// with a pass, a component search and a sort per threshold, 2220 us so.
+// with a pass, a component search and a sort per threshold, 1996 us so.
 #include "hop_internal.cuh"
 
 #include <algorithm>
@@ -71,6 +71,15 @@ __global__ void sub_particle_chain_kernel(const uint32_t *__restrict__ chain, co
     }
 }
 
+// Every chain's key starts as its root's.
+__global__ void sub_root_key_kernel(const uint32_t *__restrict__ chain, const uint64_t *__restrict__ dkey, int64_t n,
+                                    const uint32_t *__restrict__ pc, unsigned long long *__restrict__ pkey)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (int64_t)gridDim.x * blockDim.x)
+        if (chain[i] == (uint32_t)i && pc[i] != kNone) pkey[pc[i]] = dkey[i];
+}
+
 __global__ void sub_edge_ids_kernel(const uint64_t *__restrict__ ekey, int64_t m, int64_t n,
                                 const uint32_t *__restrict__ chain, const uint64_t *__restrict__ dkey, float d_o,
                                 const uint32_t *__restrict__ cid, uint32_t *__restrict__ ea,
@@ -97,92 +106,68 @@ struct Levels {
     int L;
 };
 
+// Sum of x over the lanes of `peers` (the lane's own set of a match), in its
+// first lane: every round adds the next lane that is still in to each lane of
+// even rank and drops the odd ones.
+__device__ __forceinline__ double peer_sum(uint32_t peers, int lane, double x)
+{
+    uint32_t rank = __popc(peers & ((1u << lane) - 1u));
+    uint32_t above = peers & (0xfffffffeu << lane);
+    while (__any_sync(0xffffffffu, above != 0)) {
+        const int next = __ffs(above);                     // 0: none
+        const double y = __shfl_sync(0xffffffffu, x, next ? next - 1 : lane);
+        if (next) x += y;
+        above &= __ballot_sync(0xffffffffu, (rank & 1u) == 0);
+        rank >>= 1;
+    }
+    return x;
+}
+
 // S3: count[c * kLev + l], sum (the same layout, or nullptr) and peak key of
-// every chain.  A warp takes kSubSpan consecutive particles, loading kSubU
-// steps of 32 before reducing any.  A step whose members all lie in one chain
-// is added to the warp's carried run (members of a halo are mostly
-// consecutive), the runs of any other step go to memory with one atomic per
-// value.  Counts are the set bits of a ballot per threshold.
+// every chain.  The lanes of a warp that hold the same chain are found by a
+// match, wherever they are (a halo's particles alternate between its chains),
+// their counts are the set bits of a ballot per threshold, and one lane adds
+// them.  pkey holds the root's key on entry, normally the chain's largest, so
+// it is only read.
 constexpr int kSubU = 4;
-constexpr int kSubSteps = 32;
-constexpr int kSubSpan = 32 * kSubSteps;
 
 template <bool SUM>
 __global__ void sub_chain_stats_kernel(const uint64_t *__restrict__ dkey, const uint32_t *__restrict__ pc, int64_t n,
                                        const Levels lev, uint32_t *__restrict__ cnt, double *__restrict__ sum,
-                                       unsigned long long *__restrict__ pkey)
+                                       unsigned long long *pkey)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t w0 = w * kSubSpan; w0 < n; w0 += nw * kSubSpan) {
-        uint32_t cr = kNone;                  // the carried run: chain, best key; lane l < L: count and sum at level l
-        unsigned long long cb = 0;
-        uint32_t cc = 0;
-        double csum = 0.0;
-        auto flush = [&]() {
-            if (cr == kNone) return;
-            if (lane == 0) atomicMax(&pkey[cr], cb);
-            if (cc) atomicAdd(&cnt[(int64_t)cr * kLev + lane], cc);
-            if constexpr (SUM)
-                if (cc) atomicAdd(&sum[(int64_t)cr * kLev + lane], csum);
-            cr = kNone;
-        };
-        for (int t = 0; t < kSubSteps; t += kSubU) {
-            uint64_t k[kSubU];
-            uint32_t c[kSubU];
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x * kSubU;
+    for (int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31)) * kSubU; w0 < n; w0 += stride) {
+        uint64_t k[kSubU];
+        uint32_t c[kSubU];
+        unsigned long long top[kSubU];
 #pragma unroll
-            for (int u = 0; u < kSubU; ++u) {
-                const int64_t i = w0 + (int64_t)(t + u) * 32 + lane;
-                k[u] = i < n ? dkey[i] : 0ull;
-                c[u] = i < n ? pc[i] : kNone;
-            }
+        for (int u = 0; u < kSubU; ++u) {
+            const int64_t i = w0 + u * 32 + lane;
+            k[u] = i < n ? dkey[i] : 0ull;
+            c[u] = i < n ? pc[i] : kNone;
+        }
 #pragma unroll
-            for (int u = 0; u < kSubU; ++u) {
-                const uint32_t rr = c[u];
-                if (!__any_sync(0xffffffffu, rr != kNone)) continue;
-                const float d = key_dens(k[u]);
-                const uint32_t heads = run_heads((int64_t)rr, lane);
-                const unsigned long long best = run_max(heads, lane, rr != kNone ? k[u] : 0ull);
-                if (heads == 1u) {
-                    // one chain, all lanes
-                    if (rr != cr) {
-                        flush();
-                        cr = rr;
-                        cb = 0;
-                        cc = 0;
-                        csum = 0.0;
-                    }
-                    cb = best > cb ? best : cb;
-                    for (int l = 0; l < lev.L; ++l) {
-                        const uint32_t m = __popc(__ballot_sync(0xffffffffu, d >= lev.ds[l]));
-                        if (lane == l) cc += m;
-                        if constexpr (SUM) {
-                            double x = d >= lev.ds[l] ? (double)d : 0.0;
+        for (int u = 0; u < kSubU; ++u) top[u] = c[u] != kNone ? pkey[c[u]] : ~0ull;
 #pragma unroll
-                            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-                            if (lane == l) csum += x;
-                        }
-                    }
-                } else {
-                    flush();
-                    const bool head = rr != kNone && ((heads >> lane) & 1u);
-                    const int len = run_len(heads, lane);
-                    const uint32_t run = (len == 32 ? 0xffffffffu : ((1u << len) - 1u)) << lane;
-                    if (head) atomicMax(&pkey[rr], best);
-                    for (int l = 0; l < lev.L; ++l) {
-                        const bool in = rr != kNone && d >= lev.ds[l];
-                        const uint32_t m = __popc(__ballot_sync(0xffffffffu, in) & run);
-                        if (head && m) atomicAdd(&cnt[(int64_t)rr * kLev + l], m);
-                        if constexpr (SUM) {
-                            const double x = run_sum<double>(heads, lane, in ? (double)d : 0.0);
-                            if (head && m) atomicAdd(&sum[(int64_t)rr * kLev + l], x);
-                        }
-                    }
+        for (int u = 0; u < kSubU; ++u) {
+            const uint32_t rr = c[u];
+            if (!__any_sync(0xffffffffu, rr != kNone)) continue;
+            if (k[u] > top[u]) atomicMax(&pkey[rr], (unsigned long long)k[u]);
+            const float d = key_dens(k[u]);
+            const uint32_t peers = __match_any_sync(0xffffffffu, rr);
+            const bool head = rr != kNone && lane == __ffs(peers) - 1;
+            for (int l = 0; l < lev.L; ++l) {
+                const bool in = rr != kNone && d >= lev.ds[l];
+                const uint32_t m = __popc(__ballot_sync(0xffffffffu, in) & peers);
+                if (head && m) atomicAdd(&cnt[(int64_t)rr * kLev + l], m);
+                if constexpr (SUM) {
+                    const double x = peer_sum(peers, lane, in ? (double)d : 0.0);
+                    if (head && m) atomicAdd(&sum[(int64_t)rr * kLev + l], x);
                 }
             }
         }
-        flush();
     }
 }
 
@@ -407,7 +392,10 @@ int subhalos(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, const uint
         // S3 (the keys and their order are the same for every batch)
         HOP_CUDA(c, cudaMemsetAsync(cnt, 0, C * kLev * 4, c->stream));
         if (sum) HOP_CUDA(c, cudaMemsetAsync(sum, 0, C * kLev * 8, c->stream));
-        HOP_CUDA(c, cudaMemsetAsync(pkey, 0, C * 8, c->stream));
+        if (l0 == 0) {
+            sub_root_key_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(chain, dkey, n, pc, pkey);
+            HOP_LAUNCH(c);
+        }
         if (sum)
             sub_chain_stats_kernel<true><<<grid_for(c, n), 256, 0, c->stream>>>(dkey, pc, n, lev, cnt, sum, pkey);
         else
