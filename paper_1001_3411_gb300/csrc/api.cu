@@ -374,14 +374,10 @@ int hop_boundaries(hop_ctx *c, const uint32_t *chain, const float *dens, const u
     if (!chain || !dens || !nbr || !n_edges || n <= 0) return ctx_fail(c, HOP_EINVAL, "missing argument");
     if (n_merge < 1 || n_merge > ld_nbr) return ctx_fail(c, HOP_EINVAL, "n_merge must be in [1, ld_nbr]");
     HOP_CUDA(c, cudaSetDevice(c->device));
-    uint64_t *dkey = (uint64_t *)ctx_buf(c, S_DKEY, n * sizeof(uint64_t));
-    if (!dkey) return HOP_ENOMEM;
-    int rc = make_dkey(c, dens, nullptr, n, dkey);
-    if (rc) return rc;
     uint64_t *ek;
     double *es;
     int64_t m;
-    rc = boundaries_table(c, chain, dkey, nbr, ld_nbr, n, n_merge, delta_outer, &ek, &es, &m);
+    int rc = boundaries_table(c, chain, dens, nbr, ld_nbr, n, n_merge, delta_outer, &ek, &es, &m);
     if (rc) return rc;
     *n_edges = m;
     if (m > cap || !edge_pair || !edge_sum) {
@@ -483,7 +479,7 @@ int hop_run(hop_ctx *c, const void *pos, int64_t n, const hop_params *p, float *
     uint64_t *ek;
     double *es;
     int64_t m;
-    rc = boundaries_table(c, chain_s, dkey, st.nbr_s, st.ld_s, n, p->n_merge, p->delta_outer, &ek, &es, &m);
+    rc = boundaries_table(c, chain_s, st.dens_s, st.nbr_s, st.ld_s, n, p->n_merge, p->delta_outer, &ek, &es, &m);
     if (rc) return rc;
     ev_record(c, 6);
     int32_t *group_s = (int32_t *)ctx_buf(c, S_GROUP_OUT, n * sizeof(int32_t));

@@ -283,7 +283,7 @@ int enqueue_pass(hop_ctx *c, const BatchPlan &pl, const SegDesc *seg, const Pass
     if ((rc = record(c, 5))) return rc;
     uint64_t *ek;
     double *es;
-    rc = boundaries_table_async(c, chain_s, dkey, nbr_s, n_out, n, p->n_merge, p->delta_outer, table_cap,
+    rc = boundaries_table_async(c, chain_s, dens_s, nbr_s, n_out, n, p->n_merge, p->delta_outer, table_cap,
                                 w.m_dev, w.nins, &ek, &es);
     if (rc) return rc;
     if ((rc = record(c, 6))) return rc;

@@ -49,8 +49,8 @@ enum Slot {
     S_RK_S,        // r_k in sorted order
     S_DKEY,        // (density bits << 32) | ~original index
     S_HOP, S_CHAIN,
-    S_HKEY, S_HVAL, // boundary hash table
-    S_EDGE_KEY, S_EDGE_SUM, S_EDGE_TMP,
+    S_HTAB,        // boundary hash table
+    S_EDGE_KEY, S_EDGE_SUM,
     S_MERGE,       // merge arrays (chains, components, ranks ...)
     S_GROUP_S,
     S_MISC,
@@ -452,7 +452,7 @@ int hop_links(hop_ctx *c, const uint64_t *dkey, const uint32_t *nbr, int ld, int
               uint32_t *hop, uint32_t *chain);
 // symmetric: only pairs whose chains link each other in both directions
 // (ADAPTAHOP), each with the larger of the two directions' sums.
-int boundaries_table(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, const uint32_t *nbr,
+int boundaries_table(hop_ctx *c, const uint32_t *chain, const float *dens, const uint32_t *nbr,
                      int ld, int64_t n, int n_merge, float delta_outer,
                      uint64_t **edge_key, double **edge_sum, int64_t *n_edges, bool symmetric = false);
 int hop_links_async(hop_ctx *c, const uint64_t *dkey, const uint32_t *nbr, int ld, int64_t n,
@@ -461,7 +461,7 @@ int hop_links_async(hop_ctx *c, const uint64_t *dkey, const uint32_t *nbr, int l
 // repeated pairs (tables gathered from several subvolumes).
 int edges_max_table(hop_ctx *c, const uint64_t *pair, const double *sum, int64_t m, uint64_t **edge_key,
                     double **edge_sum, int64_t *n_edges);
-int boundaries_table_async(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey,
+int boundaries_table_async(hop_ctx *c, const uint32_t *chain, const float *dens,
                            const uint32_t *nbr, int ld, int64_t n, int n_merge, float delta_outer,
                            int64_t cap, uint32_t *m_dev, unsigned long long *nins,
                            uint64_t **edge_key, double **edge_sum);

@@ -147,35 +147,45 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z)
     return z;
 }
 
-__device__ __forceinline__ bool table_insert(uint64_t *hkey, unsigned long long *hval,
-                                             uint64_t mask, uint64_t key, unsigned long long v,
-                                             unsigned long long *n_ins)
+// The table: {key, value} slots of 16 bytes, so a probe is one sector.
+typedef ulonglong2 Entry;
+
+// A slot as it is in memory now (other threads fill it meanwhile; key and
+// value may be of different times, which costs a redundant atomic at most).
+__device__ __forceinline__ Entry load_entry(const Entry *p)
 {
-    uint64_t h = mix64(key) & mask;
+    Entry e;
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(e.x), "=l"(e.y) : "l"(p) : "memory");
+    return e;
+}
+
+// Inserts from slot h on, whose contents e were read before.
+__device__ __forceinline__ bool table_insert(Entry *tab, uint64_t mask, uint64_t key, unsigned long long v, uint64_t h,
+                                             Entry e, unsigned long long *n_ins)
+{
     for (int probe = 0; probe < kMaxProbe; ++probe) {
-        uint64_t k = *(volatile uint64_t *)&hkey[h];
-        if (k == kEmpty) {
-            const unsigned long long prev =
-                atomicCAS((unsigned long long *)&hkey[h], (unsigned long long)kEmpty,
-                          (unsigned long long)key);
+        if (e.x == kEmpty) {
+            const unsigned long long prev = atomicCAS(&tab[h].x, (unsigned long long)kEmpty, (unsigned long long)key);
             if (prev == kEmpty) atomicAdd(n_ins, 1ull);
-            k = prev == kEmpty ? key : prev;
+            e.x = prev == kEmpty ? key : prev;
+            e.y = 0;
         }
-        if (k == key) {
-            if (*(volatile unsigned long long *)&hval[h] < v) atomicMax(&hval[h], v);
+        if (e.x == key) {
+            if (e.y < v) atomicMax(&tab[h].y, v);
             return true;
         }
         h = (h + 1) & mask;
+        e = load_entry(tab + h);
     }
     return false;
 }
 
 // Slot of `key`, or -1.  Inserts never probe further than kMaxProbe.
-__device__ __forceinline__ int64_t table_find(const uint64_t *hkey, uint64_t mask, uint64_t key)
+__device__ __forceinline__ int64_t table_find(const Entry *tab, uint64_t mask, uint64_t key)
 {
     uint64_t h = mix64(key) & mask;
     for (int probe = 0; probe < kMaxProbe; ++probe) {
-        const uint64_t k = hkey[h];
+        const uint64_t k = tab[h].x;
         if (k == key) return (int64_t)h;
         if (k == kEmpty) return -1;
         h = (h + 1) & mask;
@@ -190,76 +200,87 @@ __device__ __forceinline__ int64_t table_find(const uint64_t *hkey, uint64_t mas
 // With `directed` the key is (chain_i, chain_j) in that order, so the table
 // holds each direction of a pair separately (ADAPTAHOP's symmetric test).
 // VEC: rows start on 16 bytes and n_merge is at most four, so a row's part is
-// one read.  A pair's chains are compared before its density is fetched: most
-// neighbours are in the particle's own chain.
+// one read.  A pair's chains are compared before its density is fetched (most
+// neighbours are in the particle's own chain), and the densities and first
+// table slots of a particle's pairs are read together: the pass is bound by
+// the latency of these gathers.  (Pairs one after the other, on the density
+// keys and on keys and values in two arrays: statistics and subhalos of 16.8M
+// particles took 1996 us, 1901 us so; a pass over 4,913 particles 531 us and
+// 482 us, of which most is the scan of the table that the compaction used.)
 template <bool VEC>
-__global__ void boundary_kernel(const uint32_t *__restrict__ chain,
-                                const uint64_t *__restrict__ dkey,
+__global__ void boundary_kernel(const uint32_t *__restrict__ chain, const float *__restrict__ dens,
                                 const uint32_t *__restrict__ nbr, int ld, int64_t n, int n_merge,
-                                float d_o, uint64_t *hkey, unsigned long long *hval, uint64_t mask,
-                                uint32_t *err, unsigned long long *n_ins, bool directed)
+                                float d_o, Entry *tab, uint64_t mask, uint32_t *err, unsigned long long *n_ins,
+                                bool directed)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const float di = key_dens(dkey[i]);
+        const float di = dens[i];
         if (!(di >= d_o)) continue;
         const uint32_t ci = chain[i];
         const uint32_t *row = nbr + i * (int64_t)ld;
-        auto link = [&](uint32_t j, uint32_t cj) {
-            const float dj = key_dens(dkey[j]);
-            if (!(dj >= d_o)) return;
-            const uint64_t key = (directed || ci < cj) ? (((uint64_t)ci << 32) | cj)
-                                                       : (((uint64_t)cj << 32) | ci);
-            const double s = (double)di + (double)dj;
-            if (!table_insert(hkey, hval, mask, key, (unsigned long long)__double_as_longlong(s), n_ins))
-                atomicOr(err, kErrTableFull);
-        };
-        if constexpr (VEC) {
-            const uint4 v = *reinterpret_cast<const uint4 *>(row);
-            const uint32_t j[4] = {v.x, v.y, v.z, v.w};
-            uint32_t cj[4];
+        for (int t0 = 0; t0 < n_merge; t0 += 4) {
+            uint32_t j[4], cj[4];
+            if constexpr (VEC) {
+                const uint4 v = *reinterpret_cast<const uint4 *>(row);
+                j[0] = v.x;
+                j[1] = v.y;
+                j[2] = v.z;
+                j[3] = v.w;
+            } else {
+#pragma unroll
+                for (int t = 0; t < 4; ++t) j[t] = t0 + t < n_merge ? row[t0 + t] : (uint32_t)i;
+            }
+            bool any = false;
 #pragma unroll
             for (int t = 0; t < 4; ++t) {
                 cj[t] = ci;
-                if (t >= n_merge || j[t] == (uint32_t)i) continue;
+                if (t0 + t >= n_merge || j[t] == (uint32_t)i) continue;
                 if (j[t] >= (uint64_t)n) atomicOr(err, kErrBadIndex);
                 else cj[t] = chain[j[t]];
             }
-#pragma unroll 1
+#pragma unroll
+            for (int t = 0; t < 4; ++t) any |= cj[t] != ci;
+            if (!any) continue;
+            float dj[4];
+            uint64_t key[4];
+            Entry e[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) dj[t] = cj[t] != ci ? dens[j[t]] : 0.f;
+#pragma unroll
             for (int t = 0; t < 4; ++t) {
-                const uint32_t jt = t == 0 ? j[0] : t == 1 ? j[1] : t == 2 ? j[2] : j[3];
-                const uint32_t ct = t == 0 ? cj[0] : t == 1 ? cj[1] : t == 2 ? cj[2] : cj[3];
-                if (ct != ci) link(jt, ct);
+                if (!(cj[t] != ci && dj[t] >= d_o)) cj[t] = ci;
+                key[t] = (directed || ci < cj[t]) ? (((uint64_t)ci << 32) | cj[t]) : (((uint64_t)cj[t] << 32) | ci);
+                if (cj[t] != ci) e[t] = load_entry(tab + (mix64(key[t]) & mask));
             }
-        } else {
-            for (int t = 0; t < n_merge; ++t) {
-                const uint32_t j = row[t];
-                if (j == (uint32_t)i) continue;
-                if (j >= (uint64_t)n) { atomicOr(err, kErrBadIndex); continue; }
-                const uint32_t cj = chain[j];
-                if (cj != ci) link(j, cj);
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                if (cj[t] == ci) continue;
+                const double s = (double)di + (double)dj[t];
+                if (!table_insert(tab, mask, key[t], (unsigned long long)__double_as_longlong(s), mix64(key[t]) & mask,
+                                  e[t], n_ins))
+                    atomicOr(err, kErrTableFull);
             }
         }
     }
 }
 
-void boundary_launch(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, const uint32_t *nbr, int ld, int64_t n,
-                     int n_merge, float d_o, uint64_t *hkey, unsigned long long *hval, uint64_t mask, uint32_t *err,
-                     unsigned long long *n_ins, bool directed)
+void boundary_launch(hop_ctx *c, const uint32_t *chain, const float *dens, const uint32_t *nbr, int ld, int64_t n,
+                     int n_merge, float d_o, Entry *tab, uint64_t mask, uint32_t *err, unsigned long long *n_ins,
+                     bool directed)
 {
     if (n_merge <= 4 && ld >= 4 && ld % 4 == 0 && (uintptr_t)nbr % 16 == 0)
-        boundary_kernel<true><<<grid_for(c, n), 256, 0, c->stream>>>(chain, dkey, nbr, ld, n, n_merge, d_o, hkey, hval,
-                                                                    mask, err, n_ins, directed);
+        boundary_kernel<true><<<grid_for(c, n), 256, 0, c->stream>>>(chain, dens, nbr, ld, n, n_merge, d_o, tab, mask, err,
+                                                                    n_ins, directed);
     else
-        boundary_kernel<false><<<grid_for(c, n), 256, 0, c->stream>>>(chain, dkey, nbr, ld, n, n_merge, d_o, hkey, hval,
-                                                                     mask, err, n_ins, directed);
+        boundary_kernel<false><<<grid_for(c, n), 256, 0, c->stream>>>(chain, dens, nbr, ld, n, n_merge, d_o, tab, mask,
+                                                                     err, n_ins, directed);
 }
 
 // Inserts a list of (pair, sum) boundaries into the table; each pair keeps
 // its largest sum (the sums are >= 0, so their bits order like the values).
 __global__ void edge_insert_kernel(const uint64_t *__restrict__ pair, const double *__restrict__ sum, int64_t m,
-                                   uint64_t *hkey, unsigned long long *hval, uint64_t mask, uint32_t *err,
-                                   unsigned long long *n_ins)
+                                   Entry *tab, uint64_t mask, uint32_t *err, unsigned long long *n_ins)
 {
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t key = pair[e];
@@ -268,77 +289,57 @@ __global__ void edge_insert_kernel(const uint64_t *__restrict__ pair, const doub
             atomicOr(err, kErrBadIndex);
             continue;
         }
-        if (!table_insert(hkey, hval, mask, key, (unsigned long long)__double_as_longlong(s), n_ins))
+        const uint64_t h = mix64(key) & mask;
+        if (!table_insert(tab, mask, key, (unsigned long long)__double_as_longlong(s), h, load_entry(tab + h), n_ins))
             atomicOr(err, kErrTableFull);
-    }
-}
-
-__global__ void occupied_kernel(const uint64_t *__restrict__ hkey, int64_t cap, uint32_t *__restrict__ occ)
-{
-    for (int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; h < cap;
-         h += (int64_t)gridDim.x * blockDim.x)
-        occ[h] = hkey[h] != kEmpty;
-}
-
-__global__ void compact_table_kernel(const uint64_t *__restrict__ hkey,
-                                     const unsigned long long *__restrict__ hval, int64_t cap,
-                                     const uint32_t *__restrict__ pos, uint64_t *__restrict__ ekey,
-                                     double *__restrict__ esum)
-{
-    for (int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; h < cap;
-         h += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t k = hkey[h];
-        if (k == kEmpty) continue;
-        const uint32_t p = pos[h];
-        ekey[p] = k;
-        esum[p] = __longlong_as_double((long long)hval[h]);
     }
 }
 
 // Symmetric boundaries (ADAPTAHOP, Parallel HOP Sec. 6) from the directed
 // table: slot (a, b) with a < b is kept when (b, a) is present too, and
-// takes the larger of the two directions' sums.  Only a < b slots are
-// written and only a > b slots are read as partners, so there is no race.
-__device__ __forceinline__ bool sym_partner(const uint64_t *hkey, uint64_t mask, uint64_t k, int64_t *r)
+// takes the larger of the two directions' sums.
+__device__ __forceinline__ bool sym_partner(const Entry *tab, uint64_t mask, uint64_t k, int64_t *r)
 {
-    if (k == kEmpty) return false;
     const uint32_t a = (uint32_t)(k >> 32), b = (uint32_t)k;
     if (a >= b) return false;
-    *r = table_find(hkey, mask, ((uint64_t)b << 32) | a);
+    *r = table_find(tab, mask, ((uint64_t)b << 32) | a);
     return *r >= 0;
 }
 
-__global__ void symmetric_flag_kernel(const uint64_t *__restrict__ hkey, unsigned long long *hval, int64_t cap,
-                                      uint32_t *__restrict__ flag)
+// The table's entries (symmetric: the kept ones), in any order: *count goes
+// up by one atomic per warp, so the table is read once and nothing is scanned.
+template <bool SYM>
+__global__ void compact_table_kernel(const Entry *__restrict__ tab, int64_t cap, uint64_t *__restrict__ ekey,
+                                     double *__restrict__ esum, uint32_t *__restrict__ count)
 {
-    for (int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; h < cap;
-         h += (int64_t)gridDim.x * blockDim.x) {
-        int64_t r;
-        const bool keep = sym_partner(hkey, (uint64_t)cap - 1, hkey[h], &r);
-        if (keep && hval[r] > hval[h]) hval[h] = hval[r];
-        flag[h] = keep ? 1u : 0u;
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t h0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); h0 < cap; h0 += stride) {
+        const int64_t h = h0 + lane;                       // cap is a multiple of 32
+        const Entry e = tab[h];
+        bool keep = e.x != kEmpty;
+        unsigned long long v = e.y;
+        if constexpr (SYM) {
+            int64_t r = -1;
+            keep = keep && sym_partner(tab, (uint64_t)cap - 1, e.x, &r);
+            if (keep) v = tab[r].y > v ? tab[r].y : v;
+        }
+        const uint32_t bal = __ballot_sync(0xffffffffu, keep);
+        if (!bal) continue;
+        uint32_t at = 0;
+        if (lane == __ffs(bal) - 1) at = atomicAdd(count, (uint32_t)__popc(bal));
+        at = __shfl_sync(0xffffffffu, at, __ffs(bal) - 1) + __popc(bal & ((1u << lane) - 1u));
+        if (keep) {
+            ekey[at] = e.x;
+            esum[at] = __longlong_as_double((long long)v);
+        }
     }
 }
 
-__global__ void symmetric_compact_kernel(const uint64_t *__restrict__ hkey,
-                                         const unsigned long long *__restrict__ hval, int64_t cap,
-                                         const uint32_t *__restrict__ pos, uint64_t *__restrict__ ekey,
-                                         double *__restrict__ esum)
+__global__ void table_clear_kernel(Entry *tab, int64_t cap)
 {
-    for (int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; h < cap;
-         h += (int64_t)gridDim.x * blockDim.x) {
-        int64_t r;
-        if (!sym_partner(hkey, (uint64_t)cap - 1, hkey[h], &r)) continue;
-        ekey[pos[h]] = hkey[h];
-        esum[pos[h]] = __longlong_as_double((long long)hval[h]);
-    }
-}
-
-__global__ void fill_u64_kernel(uint64_t *p, int64_t n, uint64_t v)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x)
-        p[i] = v;
+    for (int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; h < cap; h += (int64_t)gridDim.x * blockDim.x)
+        tab[h] = make_ulonglong2(kEmpty, 0ull);
 }
 
 // Results in the caller's order: one value per particle each.
@@ -426,7 +427,7 @@ int hop_links(hop_ctx *c, const uint64_t *dkey, const uint32_t *nbr, int ld, int
     return HOP_OK;
 }
 
-int boundaries_table(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, const uint32_t *nbr,
+int boundaries_table(hop_ctx *c, const uint32_t *chain, const float *dens, const uint32_t *nbr,
                      int ld, int64_t n, int n_merge, float delta_outer, uint64_t **edge_key,
                      double **edge_sum, int64_t *n_edges, bool symmetric)
 {
@@ -436,16 +437,13 @@ int boundaries_table(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, co
     if (!nins) return HOP_ENOMEM;
     unsigned long long *hn = (unsigned long long *)c->h_pinned;
     for (int attempt = 0; attempt < 6; ++attempt) {
-        uint64_t *hkey = (uint64_t *)ctx_buf(c, S_HKEY, cap * sizeof(uint64_t));
-        unsigned long long *hval = (unsigned long long *)ctx_buf(c, S_HVAL, cap * sizeof(uint64_t));
-        if (!hkey || !hval) return HOP_ENOMEM;
-        fill_u64_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(hkey, cap, kEmpty);
+        Entry *tab = (Entry *)ctx_buf(c, S_HTAB, cap * sizeof(Entry));
+        if (!tab) return HOP_ENOMEM;
+        table_clear_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(tab, cap);
         HOP_LAUNCH(c);
-        HOP_CUDA(c, cudaMemsetAsync(hval, 0, cap * sizeof(uint64_t), c->stream));
         HOP_CUDA(c, cudaMemsetAsync(nins, 0, 16, c->stream));
         uint32_t *terr = (uint32_t *)(nins + 1);   // this pass's own error word
-        boundary_launch(c, chain, dkey, nbr, ld, n, n_merge, delta_outer, hkey, hval, (uint64_t)cap - 1, terr, nins,
-                        symmetric);
+        boundary_launch(c, chain, dens, nbr, ld, n, n_merge, delta_outer, tab, (uint64_t)cap - 1, terr, nins, symmetric);
         HOP_LAUNCH(c);
         HOP_CUDA(c, cudaMemcpyAsync(hn, nins, 16, cudaMemcpyDeviceToHost, c->stream));
         HOP_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -456,34 +454,23 @@ int boundaries_table(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, co
             cap <<= 2;
             continue;
         }
-        uint32_t *occ = (uint32_t *)ctx_buf(c, S_EDGE_TMP, (cap + 1) * sizeof(uint32_t));
         uint64_t *ek = (uint64_t *)ctx_buf(c, S_EDGE_KEY, std::max<int64_t>(m, 1) * sizeof(uint64_t));
         double *es = (double *)ctx_buf(c, S_EDGE_SUM, std::max<int64_t>(m, 1) * sizeof(double));
-        if (!occ || !ek || !es) return HOP_ENOMEM;
-        if (symmetric) {
-            uint32_t *total = terr + 1;
-            symmetric_flag_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(hkey, hval, cap, occ);
-            HOP_LAUNCH(c);
-            int rc = scan_exclusive_u32(c, occ, occ, cap, total);
-            if (rc) return rc;
-            symmetric_compact_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(hkey, hval, cap, occ, ek, es);
-            HOP_LAUNCH(c);
-            HOP_CUDA(c, cudaMemcpyAsync(hn, nins, 16, cudaMemcpyDeviceToHost, c->stream));
-            HOP_CUDA(c, cudaStreamSynchronize(c->stream));
-            *edge_key = ek;
-            *edge_sum = es;
-            *n_edges = *(uint32_t *)((char *)hn + 12);
-            return HOP_OK;
-        }
-        occupied_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(hkey, cap, occ);
-        HOP_LAUNCH(c);
-        int rc = scan_exclusive_u32(c, occ, occ, cap, nullptr);
-        if (rc) return rc;
-        compact_table_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(hkey, hval, cap, occ, ek, es);
+        if (!ek || !es) return HOP_ENOMEM;
+        uint32_t *count = terr + 1;
+        if (symmetric)
+            compact_table_kernel<true><<<grid_for(c, cap), 256, 0, c->stream>>>(tab, cap, ek, es, count);
+        else
+            compact_table_kernel<false><<<grid_for(c, cap), 256, 0, c->stream>>>(tab, cap, ek, es, count);
         HOP_LAUNCH(c);
         *edge_key = ek;
         *edge_sum = es;
         *n_edges = m;
+        if (symmetric) {
+            HOP_CUDA(c, cudaMemcpyAsync(hn, nins, 16, cudaMemcpyDeviceToHost, c->stream));
+            HOP_CUDA(c, cudaStreamSynchronize(c->stream));
+            *n_edges = *(uint32_t *)((char *)hn + 12);
+        }
         return HOP_OK;
     }
     return ctx_fail(c, HOP_ENOMEM, "boundary table could not be sized");
@@ -498,17 +485,14 @@ int edges_max_table(hop_ctx *c, const uint64_t *pair, const double *sum, int64_t
     if (!nins) return HOP_ENOMEM;
     unsigned long long *hn = (unsigned long long *)c->h_pinned;
     for (int attempt = 0; attempt < 4; ++attempt) {
-        uint64_t *hkey = (uint64_t *)ctx_buf(c, S_HKEY, cap * sizeof(uint64_t));
-        unsigned long long *hval = (unsigned long long *)ctx_buf(c, S_HVAL, cap * sizeof(uint64_t));
-        if (!hkey || !hval) return HOP_ENOMEM;
-        fill_u64_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(hkey, cap, kEmpty);
+        Entry *tab = (Entry *)ctx_buf(c, S_HTAB, cap * sizeof(Entry));
+        if (!tab) return HOP_ENOMEM;
+        table_clear_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(tab, cap);
         HOP_LAUNCH(c);
-        HOP_CUDA(c, cudaMemsetAsync(hval, 0, cap * sizeof(uint64_t), c->stream));
         HOP_CUDA(c, cudaMemsetAsync(nins, 0, 16, c->stream));
         uint32_t *terr = (uint32_t *)(nins + 1);
         if (m > 0) {
-            edge_insert_kernel<<<grid_for(c, m), 256, 0, c->stream>>>(pair, sum, m, hkey, hval, (uint64_t)cap - 1,
-                                                                     terr, nins);
+            edge_insert_kernel<<<grid_for(c, m), 256, 0, c->stream>>>(pair, sum, m, tab, (uint64_t)cap - 1, terr, nins);
             HOP_LAUNCH(c);
         }
         HOP_CUDA(c, cudaMemcpyAsync(hn, nins, 16, cudaMemcpyDeviceToHost, c->stream));
@@ -520,15 +504,10 @@ int edges_max_table(hop_ctx *c, const uint64_t *pair, const double *sum, int64_t
             cap <<= 2;
             continue;
         }
-        uint32_t *occ = (uint32_t *)ctx_buf(c, S_EDGE_TMP, (cap + 1) * sizeof(uint32_t));
         uint64_t *ek = (uint64_t *)ctx_buf(c, S_EDGE_KEY, std::max<int64_t>(u, 1) * sizeof(uint64_t));
         double *es = (double *)ctx_buf(c, S_EDGE_SUM, std::max<int64_t>(u, 1) * sizeof(double));
-        if (!occ || !ek || !es) return HOP_ENOMEM;
-        occupied_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(hkey, cap, occ);
-        HOP_LAUNCH(c);
-        int rc = scan_exclusive_u32(c, occ, occ, cap, nullptr);
-        if (rc) return rc;
-        compact_table_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(hkey, hval, cap, occ, ek, es);
+        if (!ek || !es) return HOP_ENOMEM;
+        compact_table_kernel<false><<<grid_for(c, cap), 256, 0, c->stream>>>(tab, cap, ek, es, terr + 1);
         HOP_LAUNCH(c);
         *edge_key = ek;
         *edge_sum = es;
@@ -557,28 +536,21 @@ int hop_links_async(hop_ctx *c, const uint64_t *dkey, const uint32_t *nbr, int l
 // Boundary table of fixed capacity `cap` (a power of two).  The edge count
 // lands in *m_dev; edge_key / edge_sum hold cap entries, the first *m_dev
 // valid.  An overfull table sets kErrTableFull in the error word.
-int boundaries_table_async(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey,
+int boundaries_table_async(hop_ctx *c, const uint32_t *chain, const float *dens,
                            const uint32_t *nbr, int ld, int64_t n, int n_merge, float delta_outer,
                            int64_t cap, uint32_t *m_dev, unsigned long long *nins,
                            uint64_t **edge_key, double **edge_sum)
 {
-    uint64_t *hkey = (uint64_t *)ctx_buf(c, S_HKEY, cap * sizeof(uint64_t));
-    unsigned long long *hval = (unsigned long long *)ctx_buf(c, S_HVAL, cap * sizeof(uint64_t));
-    uint32_t *occ = (uint32_t *)ctx_buf(c, S_EDGE_TMP, (cap + 1) * sizeof(uint32_t));
+    Entry *tab = (Entry *)ctx_buf(c, S_HTAB, cap * sizeof(Entry));
     uint64_t *ek = (uint64_t *)ctx_buf(c, S_EDGE_KEY, cap * sizeof(uint64_t));
     double *es = (double *)ctx_buf(c, S_EDGE_SUM, cap * sizeof(double));
-    if (!hkey || !hval || !occ || !ek || !es) return HOP_ENOMEM;
-    fill_u64_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(hkey, cap, kEmpty);
+    if (!tab || !ek || !es) return HOP_ENOMEM;
+    table_clear_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(tab, cap);
     HOP_LAUNCH(c);
-    HOP_CUDA(c, cudaMemsetAsync(hval, 0, cap * sizeof(uint64_t), c->stream));
-    boundary_launch(c, chain, dkey, nbr, ld, n, n_merge, delta_outer, hkey, hval, (uint64_t)cap - 1, c->d_err, nins,
-                    false);
+    HOP_CUDA(c, cudaMemsetAsync(m_dev, 0, sizeof(uint32_t), c->stream));
+    boundary_launch(c, chain, dens, nbr, ld, n, n_merge, delta_outer, tab, (uint64_t)cap - 1, c->d_err, nins, false);
     HOP_LAUNCH(c);
-    occupied_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(hkey, cap, occ);
-    HOP_LAUNCH(c);
-    int rc = scan_exclusive_u32(c, occ, occ, cap, m_dev);
-    if (rc) return rc;
-    compact_table_kernel<<<grid_for(c, cap), 256, 0, c->stream>>>(hkey, hval, cap, occ, ek, es);
+    compact_table_kernel<false><<<grid_for(c, cap), 256, 0, c->stream>>>(tab, cap, ek, es, m_dev);
     HOP_LAUNCH(c);
     *edge_key = ek;
     *edge_sum = es;

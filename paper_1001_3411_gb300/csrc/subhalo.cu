@@ -313,7 +313,7 @@ __global__ void sub_label_kernel(const uint64_t *__restrict__ dkey, const uint32
     }
 }
 
-int subhalos(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, const uint32_t *nbr, int ld, int64_t n,
+int subhalos(hop_ctx *c, const uint32_t *chain, const float *dens, const uint64_t *dkey, const uint32_t *nbr, int ld, int64_t n,
              int n_merge, float d_o, const float *levels, int L, int64_t n_min, double f, int32_t *sub,
              int64_t *n_sub)
 {
@@ -322,7 +322,7 @@ int subhalos(hop_ctx *c, const uint32_t *chain, const uint64_t *dkey, const uint
     uint64_t *ek;
     double *es;
     int64_t m;
-    int rc = boundaries_table(c, chain, dkey, nbr, ld, n, n_merge, d_o, &ek, &es, &m, true);
+    int rc = boundaries_table(c, chain, dens, nbr, ld, n, n_merge, d_o, &ek, &es, &m, true);
     if (rc) return rc;
     HOP_CUDA(c, cudaEventRecord(c->ev[3], c->stream));
     // S2
@@ -475,7 +475,7 @@ extern "C" int hop_subhalos(hop_ctx *c, const uint32_t *chain, const float *dens
     if (!dkey) return HOP_ENOMEM;
     int rc = make_dkey(c, dens, nullptr, n, dkey);
     if (rc) return rc;
-    rc = subhalos(c, chain, dkey, nbr, ld_nbr, n, n_merge, delta_outer, levels, n_levels, n_min, f_poisson, sub,
+    rc = subhalos(c, chain, dens, dkey, nbr, ld_nbr, n, n_merge, delta_outer, levels, n_levels, n_min, f_poisson, sub,
                   n_sub);
     if (rc) return rc;
     HOP_CUDA(c, cudaEventRecord(c->ev[1], c->stream));
