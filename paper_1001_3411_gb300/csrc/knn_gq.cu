@@ -21,7 +21,10 @@
 //      sorted index of those within R go to the lane's own list, one column
 //      of a [slot][lane] array: no two lanes meet in a bank and no ballot is
 //      needed.  When a list is nearly full, the query's limit drops to the
-//      upper edge of the bin holding its Ndens-th entry.
+//      upper edge of the bin holding its Ndens-th entry, divided again until
+//      few others remain, and the reach of the box with it; where a region
+//      meets many nodes the query's own comes first, so that this happens
+//      early.
 //   4. Selection.  A histogram of the query's lists (32 bins linear in d^2,
 //      16-bit counts) places the entries up to the Ndens-th
 //      bin, bin by bin, in one array (a counting sort).  The exact Ndens-th
@@ -31,12 +34,17 @@
 // A query is certified when at least Ndens particles lie within R; the
 // others search again with a larger R.  A group whose region crosses both a
 // face and L/2 is served one query at a time.  What this kernel does not take
-// -- a ball that wraps around the box, more nodes than it lists, a crowd at
-// the Ndens-th distance, float64 distances too close for float32 to bin -- it
-// hands over to a warp-per-query kernel (knn_cg.cu; float64: knn.cu), which
-// runs after it over the list of such queries.  Such a query takes 0.3 ms
-// however few there are, so radii reach the largest that does not wrap before
-// one is handed over (4,913 particles: 0.37 -> 0.08 ms).
+// -- a ball that wraps around the box, more nodes than it lists at every
+// radius that holds Ndens, more than 32 particles too many at the Ndens-th
+// distance, float64 distances too close for float32 to bin -- it hands over
+// to a warp-per-query kernel (knn_cg.cu; float64: knn.cu), which runs after
+// it over the list of such queries.  Such queries take 0.3 ms however few
+// there are, and 2 to 8 ms where their radii are far too large, so radii reach
+// the largest that does not wrap before one is handed over (4,913 particles:
+// 0.37 -> 0.08 ms), and shrink where a region meets too many nodes.  (Limits
+// cut once instead, and no smaller radius: 4,200 of 16.8M queries handed over
+// and 33.6 ms instead of 31.7, 14,700 of 2.1M with the plain radius and 19.1
+// ms instead of 7.2.)
 //
 // What bounds it: instruction issue and shared-memory wavefronts (58 % of
 // issue slots and 66 % of wavefronts at 16 warps per SM, 1.35k warp
@@ -50,11 +58,10 @@
 // 33.6: a 16-byte read costs four wavefronts whether or not the four queries
 // read the same words.
 // Kernel time, with learned first radius unless stated (in brackets a warp
-// per query): 16.8M particles 33.6 ms (82.1), 64 subvolumes of 22M together
-// 46.5 ms (111.8), 3M with Ndens = Nhop = 65 (closed form) 9.2 ms (22.2), 2.1M
-// with the plain radius, whose start is cut to what the boxes show to be
-// enough, 19.1 ms (59.2), 4,913 particles 0.08 ms (0.99), 32,768 float64
-// particles 0.72 ms (5.2, the single-scan kernel).
+// per query): 16.8M particles 31.7 ms (82.1), 64 subvolumes of 22M together
+// 43.3 ms (111.8), 3M with Ndens = Nhop = 65 (closed form) 7.1 ms (22.2), 2.1M
+// with the plain radius 5.0 ms (59.2), 4,913 particles 0.08 ms (0.99), 32,768
+// float64 particles 0.54 ms (5.2, the single-scan kernel).
 //
 // Results equal those of the other kNN kernels bit for bit: the same
 // per-component minimum-image differences, the same fused d^2, the same
@@ -102,7 +109,6 @@ struct GqDev {
     uint32_t *hand;                    // queries handed over ...
     unsigned long long *hand_n;        // ... and their number
     unsigned long long *task_counter, *counters;
-    uint32_t *err;
 };
 
 // Shared memory of one warp, byte offsets.  The node lists (search) share
@@ -221,9 +227,11 @@ struct Region {
         hy += eps;
         lz -= eps;
         hz += eps;
-        r2c = r * r * 1.00001f + box * box * 1e-12f;
+        r2c = reach(r * r);
         return true;
     }
+    __device__ __forceinline__ float reach(float d2) const { return d2 * 1.00001f + box * box * 1e-12f; }
+    __device__ __forceinline__ void set_reach(float d2) { r2c = fminf(r2c, reach(fmaxf(d2, 0.f))); }
 };
 
 // Sum over the eight lanes of a query.
@@ -270,13 +278,15 @@ __device__ __forceinline__ float gq_edge(int bin, float scale) { return __fdivid
 // finds, for each query, the bin of its k-th and of its n_out-th entry:
 // packed as bin << 20 | below << 10 | upto (0 when the lists hold fewer).
 // With PLACE the histogram becomes the positions at which each lane's
-// entries of a bin go, and bst the bins' starts.
+// entries of a bin go, and bst the bins' starts.  Without it, entries outside
+// [lo, hi] are not counted and the bins start at lo.
 struct GqFound {
     uint32_t k, o;
 };
 template <int BINS, bool PLACE>
 __device__ __forceinline__ GqFound gq_count(const float2 *list, int cnt, int cmax, uint16_t *hist,
-                                            uint16_t *bst, float scale, int k, int n_out, int lane)
+                                            uint16_t *bst, float scale, int k, int n_out, int lane, float lo = 0.f,
+                                            float hi = 0.f)
 {
     const int q = lane >> 3, p = lane & 7;
 #pragma unroll
@@ -287,8 +297,13 @@ __device__ __forceinline__ GqFound gq_count(const float2 *list, int cnt, int cma
     for (int i = 0; i < cmax; i += 2) {
         // (a column has an even number of slots)
         const float v0 = list[i * 32].x, v1 = list[(i + 1) * 32].x;
-        gq_next(col + gq_bin_bits(v0, scale) * 64, i < cnt);
-        gq_next(col + gq_bin_bits(v1, scale) * 64, i + 1 < cnt);
+        if constexpr (PLACE) {
+            gq_next(col + gq_bin_bits(v0, scale) * 64, i < cnt);
+            gq_next(col + gq_bin_bits(v1, scale) * 64, i + 1 < cnt);
+        } else {
+            gq_next(col + gq_bin_bits(v0 - lo, scale) * 64, i < cnt && v0 >= lo && v0 <= hi);
+            gq_next(col + gq_bin_bits(v1 - lo, scale) * 64, i + 1 < cnt && v1 >= lo && v1 <= hi);
+        }
     }
     __syncwarp();
     // lane p holds bins p, p + 8 .. of its query, each one read of 16 bytes
@@ -357,21 +372,44 @@ __device__ __forceinline__ GqFound gq_count(const float2 *list, int cnt, int cma
 
 // Drops the limit of every query that holds at least k entries (and is in
 // `which`) to the upper edge of the bin of its k-th (plus slack), and its
-// lists to the entries up to it.  Out of line: only lists that are nearly full, or a
-// crowded k-th bin, need it.
+// lists to the entries up to it.  While more than `most` entries remain, the
+// k-th's bin is divided again: a query in a void beside a halo has most of
+// its entries in the outermost bin, one at a halo's cusp in the innermost.
+// Out of line: only lists that are nearly full, or a crowded k-th bin, need it.
 struct Tight {
     int cnt;
     float tau;
 };
-__device__ __noinline__ Tight gq_tighten(uint32_t wo, int cnt, bool which, float tau, float slack, int k, int lane)
+__device__ __noinline__ Tight gq_tighten(uint32_t wo, int cnt, bool which, float tau, float slack, int k, int most,
+                                         int lane)
 {
     float2 *list = (float2 *)(gq_smem + wo + GqSmem::list) + lane;
     uint16_t *hist = (uint16_t *)(gq_smem + wo + GqSmem::thist);
     const int cmax = (int)__reduce_max_sync(kAll, which ? (unsigned)cnt : 0u);
-    const float scale = gq_scale<kGqCutBins>(tau);
-    const GqFound f = gq_count<kGqCutBins, false>(list, which ? cnt : 0, cmax, hist, nullptr, scale, k, 0, lane);
-    if (which && f.k) {
-        tau = fminf(tau, gq_edge((int)(f.k >> 20), scale) + slack);
+    float lo = 0.f, hi = tau;
+    bool on = which;
+    int below = 0;   // entries under lo
+#pragma unroll 1
+    for (int it = 0; it < 4; ++it) {
+        const float scale = gq_scale<kGqCutBins>(hi - lo);
+        const GqFound f =
+            gq_count<kGqCutBins, false>(list, on ? cnt : 0, cmax, hist, nullptr, scale, k - below, 0, lane, lo, hi);
+        on = on && f.k;
+        if (on) {
+            const int b = (int)(f.k >> 20);
+            hi = fminf(hi, (lo + gq_edge(b, scale)) * 1.000001f);
+            lo += __fdividef((float)b, scale);
+            on = below + (int)(f.k & 1023u) > most && hi > lo;
+        }
+        if (!__any_sync(kAll, on)) break;
+        int u = 0;
+#pragma unroll 1
+        for (int i = 0; on && i < cnt; ++i) u += list[i * 32].x < lo;
+        below = oct_sum(u);
+        on = on && below < k;
+    }
+    if (which && hi < tau) {
+        tau = fminf(tau, hi + slack);
         int m = 0;
 #pragma unroll 1
         for (int i = 0; i < cnt; ++i) {
@@ -462,24 +500,32 @@ __device__ __forceinline__ int gq_open(const BoxTree &t, int lv, const Region &r
     return m;
 }
 
-// The first radius of the plain policy at particle s: the mean-density
-// distance, or where that is larger the distance to the farthest corner of
-// the boxes that hold the particle's own 64 (more than 64 wanted: 128)
-// neighbours in sort order, which is enough for k of them.
+// The first radius of the plain policy at particle s, from the boxes that
+// hold the particle's own 64 (more than 64 wanted: 128) neighbours in sort
+// order: the radius that holds k at their mean density, 1.1 times, no more
+// than the distance to the boxes' farthest corner, which is enough, and no
+// more than 1.5 times the mean-density distance, so that boxes stretched over
+// a jump of the Morton curve do not count.  2.1M particles, kNN: 4.97 ms
+// (7.19 with the smaller of mean-density and corner distance); factors of 0.9
+// to 1.35 without the last bound 5.70 to 6.67, bounds of 1, 1.25 and 2 6.18,
+// 6.05 and 5.30.
 __device__ __noinline__ float gq_plain_radius(const BoxTree &t, float4 v, uint32_t s, uint32_t base, uint32_t end, int k,
                                               float plain_r)
 {
     const int nodes = k <= 64 ? 1 : 2;
     const uint32_t node = (s >> 6) & ~(uint32_t)(nodes - 1);
     if (node * 64 < base || (uint64_t)(node + nodes) * 64 > end) return plain_r;
-    float dx = 0.f, dy = 0.f, dz = 0.f;
+    float dx = 0.f, dy = 0.f, dz = 0.f, vol = 0.f;
     for (int i = 0; i < nodes; ++i) {
         const float4 lo = t.lo[t.off[1] + node + i], hi = t.hi[t.off[1] + node + i];
         dx = fmaxf(dx, fmaxf(v.x - lo.x, hi.x - v.x));
         dy = fmaxf(dy, fmaxf(v.y - lo.y, hi.y - v.y));
         dz = fmaxf(dz, fmaxf(v.z - lo.z, hi.z - v.z));
+        const float ex = hi.x - lo.x, ey = hi.y - lo.y, ez = hi.z - lo.z, least = 0.125f * fmaxf(ex, fmaxf(ey, ez));
+        vol += fmaxf(ex, least) * fmaxf(ey, least) * fmaxf(ez, least);
     }
-    return fminf(plain_r, sqrtf(dx * dx + dy * dy + dz * dz) * 1.0001f);
+    const float est = 1.1f * cbrtf((float)k * vol / (float)(64 * nodes) * 0.238732f);   // 3 / (4 pi)
+    return fminf(1.5f * plain_r, fminf(est, sqrtf(dx * dx + dy * dy + dz * dz) * 1.0001f));
 }
 
 // The factor by which a radius grows that held tot < k particles.
@@ -581,21 +627,21 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
             if (rg.build(true, x, y, z, ru, box)) n2u = gq_descend(a.tree, rg, base, end, wo + L::u2, wo + L::t2, lane);
         }
         for (int g = 0; g < nu; g += kGqQ) {
-        const int nq = min(kGqQ, nu - g);
-        ++warp_acc;
-        const uint32_t sq = s_unit + g + min(q, nq - 1);
-        const float R0 = __shfl_sync(kAll, r4, g);
-        const float qx = __shfl_sync(kAll, ux, g + min(q, nq - 1)), qy = __shfl_sync(kAll, uy, g + min(q, nq - 1)),
-                    qz = __shfl_sync(kAll, uz, g + min(q, nq - 1));
-        // a query farther than R0 from the one before it starts a new search
-        const float ex = qx - __shfl_up_sync(kAll, qx, 8), ey = qy - __shfl_up_sync(kAll, qy, 8),
-                    ez = qz - __shfl_up_sync(kAll, qz, 8);
-        const uint32_t cuts = __ballot_sync(kAll, p == 0 && q > 0 && q < nq && ex * ex + ey * ey + ez * ez > R0 * R0);
-        uint32_t todo = (1u << (8 * nq - 1)) * 2u - 1u;   // the lanes of the queries still to be served
-        float rq = R0;                                     // the query's radius
-        bool alone = false;
-        int tries = 0;
-        {
+            const int nq = min(kGqQ, nu - g);
+            ++warp_acc;
+            const uint32_t sq = s_unit + g + min(q, nq - 1);
+            const float R0 = __shfl_sync(kAll, r4, g);
+            const float qx = __shfl_sync(kAll, ux, g + min(q, nq - 1)), qy = __shfl_sync(kAll, uy, g + min(q, nq - 1)),
+                        qz = __shfl_sync(kAll, uz, g + min(q, nq - 1));
+            // a query farther than R0 from the one before it starts a new search
+            const float ex = qx - __shfl_up_sync(kAll, qx, 8), ey = qy - __shfl_up_sync(kAll, qy, 8),
+                        ez = qz - __shfl_up_sync(kAll, qz, 8);
+            const uint32_t cuts = __ballot_sync(kAll, p == 0 && q > 0 && q < nq && ex * ex + ey * ey + ez * ez > R0 * R0);
+            uint32_t todo = (1u << (8 * nq - 1)) * 2u - 1u;   // the lanes of the queries still to be served
+            // the query's radius; the largest that held too few, the smallest that met too many nodes
+            float rq = R0, rfew = 0.f, rmany = INFINITY;
+            bool alone = false;
+            int tries = 0;
             while (todo) {
                 // from the first one up to the next cut, or the first alone
                 const int g0 = __ffs(todo) - 1;
@@ -608,7 +654,8 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                 Region rg;
                 float fx = qx, fy = qy, fz = qz;
                 int n2 = -1;
-                if (rg.build(member, fx, fy, fz, R, box) && tries < kGqTries) {
+                const bool built = rg.build(member, fx, fy, fz, R, box) && tries < kGqTries;
+                if (built) {
                     if (n2u >= 0 && R <= ru) {
                         n2 = 0;
                         for (int i = 0; i < n2u; i += 32) {
@@ -629,9 +676,20 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                 }
                 if (n2 < 0) {
                     // several queries' region that crosses both a face and L/2,
-                    // or meets too many nodes: the first one alone
+                    // or meets too many nodes: the first one alone, then
+                    // with a smaller radius as long as that may hold enough
                     alone = !alone && set != (0xffu << g0);
                     if (!alone) {
+                        const float few = warp_max(member ? rfew : 0.f);
+                        if (built && R > 1.05f * few) {
+                            ++tries;
+                            alone = true;
+                            if (member) {
+                                rmany = R;
+                                rq = few > 0.f ? sqrtf(R * few) : 0.5f * R;
+                            }
+                            continue;
+                        }
                         if (member && p == 0) a.hand[atomicAdd(a.hand_n, 1ull)] = sq;
                         todo &= ~set;
                     }
@@ -639,6 +697,17 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                 }
                 alone = false;
                 ++search_acc;
+                if (n2 > 8) {
+                    // a large region: the query's own node first, so that the
+                    // limits drop before the others are opened
+                    const uint32_t own = __shfl_sync(kAll, sq, g0) >> 9;
+                    for (int i = lane; i < n2; i += 32)
+                        if (i > 0 && T2[i] == own) {
+                            T2[i] = T2[0];
+                            T2[0] = own;
+                        }
+                    __syncwarp();
+                }
                 // ------------- open them and evaluate the runs
                 uint32_t lp = list0;   // the end of the lane's list
                 float tau = member ? R * R : -1.f;
@@ -741,7 +810,8 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                             }
                             if (over) {
                                 __syncwarp();
-                                const Tight t = gq_tighten(wo, (int)(lp - list0) >> 8, member && !crowd, tau, slack, k, lane);
+                                const Tight t = gq_tighten(wo, (int)(lp - list0) >> 8, member && !crowd, tau, slack, k,
+                                                           a.capq, lane);
                                 lp = list0 + t.cnt * 256;
                                 tau = t.tau;
                                 // a list that stays full: a crowd at the limit
@@ -750,6 +820,8 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                                     lp = list0;
                                     tau = -1.f;
                                 }
+                                // no more than the largest limit needs be read
+                                rg.set_reach(warp_max(tau));
                             }
                         }
                         // what is left (fewer than 16) moves to the front
@@ -799,7 +871,7 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                             }
                             break;
                         }
-                        const Tight c = gq_tighten(wo, cnt, over, tau, slack, k, lane);
+                        const Tight c = gq_tighten(wo, cnt, over, tau, slack, k, a.capq, lane);
                         cnt = c.cnt;
                         tau = c.tau;
                     }
@@ -885,7 +957,6 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                     // the entry's bin and its rank in it
                     if (n_out > 0) {
                         uint32_t *row = a.nbr_s + (size_t)sq * a.ld_out;
-#pragma unroll 1
                         // the entries that may come before or after entry e
                         auto around = [&](int e, D2 v, int &h0, int &h1) {
                             if constexpr (F64) {
@@ -901,6 +972,7 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                             }
                         };
                         int sum = 0;
+#pragma unroll 1
                         for (int e = p; e < upto_o; e += 8) {
                             const D2 v = Dd[e];
                             int h0, h1;
@@ -946,11 +1018,12 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                         const float most = 0.2499f * box;
                         rq = R * fminf(gq_grow(k, tot), 8.f);
                         if (R < 0.99f * most) rq = fminf(rq, most);
+                        rfew = R;
+                        rq = fminf(rq, sqrtf(R * rmany));
                     }
                 }
                 __syncwarp();
             }
-        }
         }
     }
     if (lane == 0) {
@@ -1014,7 +1087,6 @@ template <bool SEG, bool F64> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int 
     d.counters = c->d_counters;
     d.task_counter = c->d_counters + kCntNum;
     d.hand_n = c->d_counters + kCntNum + 1;
-    d.err = c->d_err;
     d.hand = (uint32_t *)ctx_buf(c, S_KNN_HAND, (size_t)ka.n * sizeof(uint32_t));
     if (!d.hand) return HOP_ENOMEM;
     HOP_CUDA(c, cudaMemsetAsync(d.task_counter, 0, 3 * sizeof(unsigned long long), c->stream));
