@@ -55,50 +55,86 @@ __device__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *smem_warp, uint32
     return r;
 }
 
+// Four consecutive items from i on, zeros past n; vec: 16-byte aligned.
+__device__ __forceinline__ uint4 scan_load(const uint32_t *in, int64_t i, int64_t n, bool vec)
+{
+    if (vec && i + 4 <= n) return *reinterpret_cast<const uint4 *>(in + i);
+    return make_uint4(i < n ? in[i] : 0u, i + 1 < n ? in[i + 1] : 0u, i + 2 < n ? in[i + 2] : 0u,
+                      i + 3 < n ? in[i + 3] : 0u);
+}
+
 __global__ void scan_reduce_kernel(const uint32_t *__restrict__ in, DevCount nc,
                                    uint32_t *__restrict__ partial)
 {
     __shared__ uint32_t sw[33];
     const int64_t n = nc.get();
     const int64_t base = (int64_t)blockIdx.x * kScanTile;
+    const bool vec = (uintptr_t)in % 16 == 0;
     uint32_t s = 0;
 #pragma unroll
-    for (int r = 0; r < kScanItems; ++r) {
-        int64_t i = base + (int64_t)r * kScanThreads + threadIdx.x;
-        if (i < n) s += in[i];
+    for (int r = 0; r < kScanItems / 4; ++r) {
+        const uint4 v = scan_load(in, base + ((int64_t)r * kScanThreads + threadIdx.x) * 4, n, vec);
+        s += v.x + v.y + v.z + v.w;
     }
     uint32_t tot;
     block_exclusive_scan(s, sw, &tot);
     if (threadIdx.x == 0) partial[blockIdx.x] = tot;
 }
 
-// Each thread owns kScanItems consecutive items.
-__global__ void scan_apply_kernel(const uint32_t *__restrict__ in, uint32_t *__restrict__ out,
+// A warp owns 512 consecutive items in four rows of 128, a lane four
+// consecutive ones of each: 16-byte accesses side by side, bound by HBM.
+// (`in` may be `out`.  16.8M items: 17 us; sixteen consecutive items per lane,
+// one load each, 83 us.)
+__global__ void scan_apply_kernel(const uint32_t *in, uint32_t *out,
                                   DevCount nc, const uint32_t *__restrict__ partial_scanned,
                                   uint32_t *__restrict__ total_dev, int write_total)
 {
-    __shared__ uint32_t sw[33];
+    constexpr int kRows = kScanItems / 4;
+    __shared__ uint32_t sw[kScanThreads / 32];
     const int64_t n = nc.get();
-    const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-    uint32_t v[kScanItems];
-    uint32_t s = 0;
+    const int lane = (int)lane_id(), warp = threadIdx.x >> 5;
+    const int64_t base = (int64_t)blockIdx.x * kScanTile + warp * 32 * kScanItems + lane * 4;
+    const bool vec = ((uintptr_t)in | (uintptr_t)out) % 16 == 0;
+    uint4 v[kRows];
+    uint32_t pre[kRows];   // exclusive prefix of the lane's four items in the warp
+    uint32_t tot = 0;
 #pragma unroll
-    for (int r = 0; r < kScanItems; ++r) {
-        int64_t i = base + r;
-        v[r] = i < n ? in[i] : 0u;
-        s += v[r];
+    for (int r = 0; r < kRows; ++r) v[r] = scan_load(in, base + r * 128, n, vec);
+#pragma unroll
+    for (int r = 0; r < kRows; ++r) {
+        const uint32_t s = v[r].x + v[r].y + v[r].z + v[r].w;
+        uint32_t x = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        pre[r] = tot + x - s;
+        tot += __shfl_sync(0xffffffffu, x, 31);
     }
-    uint32_t tot;
-    uint32_t pre = block_exclusive_scan(s, sw, &tot);
-    pre += partial_scanned ? partial_scanned[blockIdx.x] : 0u;
+    if (lane == 0) sw[warp] = tot;
+    __syncthreads();
+    uint32_t before = partial_scanned ? partial_scanned[blockIdx.x] : 0u;
+    for (int w = 0; w < warp; ++w) before += sw[w];
 #pragma unroll
-    for (int r = 0; r < kScanItems; ++r) {
-        int64_t i = base + r;
-        if (i < n) out[i] = pre;
-        pre += v[r];
+    for (int r = 0; r < kRows; ++r) {
+        const int64_t i = base + r * 128;
+        uint4 o;
+        o.x = before + pre[r];
+        o.y = o.x + v[r].x;
+        o.z = o.y + v[r].y;
+        o.w = o.z + v[r].z;
+        if (vec && i + 4 <= n) {
+            *reinterpret_cast<uint4 *>(out + i) = o;
+        } else {
+            if (i < n) out[i] = o.x;
+            if (i + 1 < n) out[i + 1] = o.y;
+            if (i + 2 < n) out[i + 2] = o.z;
+            if (i + 3 < n) out[i + 3] = o.w;
+        }
     }
     if (write_total && total_dev && threadIdx.x == blockDim.x - 1 && blockIdx.x == gridDim.x - 1)
-        *total_dev = pre;
+        *total_dev = before + tot;
 }
 
 // ------------------------------------------------------------ radix sort --
