@@ -57,8 +57,7 @@ enum {
  * particles fall inside a radius whose ball was scanned completely, and is
  * otherwise repeated with a larger radius. */
 enum {
-    HOP_RADIUS_PLAIN = 0,   /* mean-density Ndens-th-neighbour distance, of the box or of
-                               the particles around in sort order, expanded              */
+    HOP_RADIUS_PLAIN = 0,   /* mean-density Ndens-th-neighbour distance, expanded    */
     HOP_RADIUS_COUNT = 1,   /* closed form from the 27 stencil cell counts          */
     HOP_RADIUS_LEARNED = 2  /* the loaded MLP reads the 27 log-counts (hop_mlp_*)   */
 };

@@ -41,10 +41,10 @@
 // it over the list of such queries.  Such queries take 0.3 ms however few
 // there are, and 2 to 8 ms where their radii are far too large, so radii reach
 // the largest that does not wrap before one is handed over (4,913 particles:
-// 0.37 -> 0.08 ms), and shrink where a region meets too many nodes.  (Limits
+// 0.37 -> 0.08 ms), and halve where a region meets too many nodes.  (Limits
 // cut once instead, and no smaller radius: 4,200 of 16.8M queries handed over
-// and 33.6 ms instead of 31.7, 14,700 of 2.1M with the plain radius and 19.1
-// ms instead of 7.2.)
+// and 33.6 ms instead of 31.3, 14,700 of 2.1M with the plain radius and 19.1
+// ms instead of 7.4.)
 //
 // What bounds it: instruction issue and shared-memory wavefronts (58 % of
 // issue slots and 66 % of wavefronts at 16 warps per SM, 1.35k warp
@@ -58,9 +58,9 @@
 // 33.6: a 16-byte read costs four wavefronts whether or not the four queries
 // read the same words.
 // Kernel time, with learned first radius unless stated (in brackets a warp
-// per query): 16.8M particles 31.7 ms (82.1), 64 subvolumes of 22M together
-// 43.3 ms (111.8), 3M with Ndens = Nhop = 65 (closed form) 7.1 ms (22.2), 2.1M
-// with the plain radius 5.0 ms (59.2), 4,913 particles 0.08 ms (0.99), 32,768
+// per query): 16.8M particles 31.3 ms (82.1), 64 subvolumes of 22M together
+// 43.3 ms (111.8), 3M with Ndens = Nhop = 65 (closed form) 7.0 ms (22.2), 2.1M
+// with the plain radius 7.4 ms (59.2), 4,913 particles 0.08 ms (0.99), 32,768
 // float64 particles 0.54 ms (5.2, the single-scan kernel).
 //
 // Results equal those of the other kNN kernels bit for bit: the same
@@ -500,32 +500,25 @@ __device__ __forceinline__ int gq_open(const BoxTree &t, int lv, const Region &r
     return m;
 }
 
-// The first radius of the plain policy at particle s, from the boxes that
-// hold the particle's own 64 (more than 64 wanted: 128) neighbours in sort
-// order: the radius that holds k at their mean density, 1.1 times, no more
-// than the distance to the boxes' farthest corner, which is enough, and no
-// more than 1.5 times the mean-density distance, so that boxes stretched over
-// a jump of the Morton curve do not count.  2.1M particles, kNN: 4.97 ms
-// (7.19 with the smaller of mean-density and corner distance); factors of 0.9
-// to 1.35 without the last bound 5.70 to 6.67, bounds of 1, 1.25 and 2 6.18,
-// 6.05 and 5.30.
-__device__ __noinline__ float gq_plain_radius(const BoxTree &t, float4 v, uint32_t s, uint32_t base, uint32_t end, int k,
+// The first radius at particle s where the given one wraps: the mean-density
+// distance, or where that is larger the distance to the farthest corner of
+// the boxes that hold the particle's own 64 (more than 64 wanted: 128)
+// neighbours in sort order, which is enough for k of them.  (64 subvolumes:
+// 43.3 ms, with the mean-density distance alone 48.2.)
+__device__ __noinline__ float gq_box_radius(const BoxTree &t, float4 v, uint32_t s, uint32_t base, uint32_t end, int k,
                                               float plain_r)
 {
     const int nodes = k <= 64 ? 1 : 2;
     const uint32_t node = (s >> 6) & ~(uint32_t)(nodes - 1);
     if (node * 64 < base || (uint64_t)(node + nodes) * 64 > end) return plain_r;
-    float dx = 0.f, dy = 0.f, dz = 0.f, vol = 0.f;
+    float dx = 0.f, dy = 0.f, dz = 0.f;
     for (int i = 0; i < nodes; ++i) {
         const float4 lo = t.lo[t.off[1] + node + i], hi = t.hi[t.off[1] + node + i];
         dx = fmaxf(dx, fmaxf(v.x - lo.x, hi.x - v.x));
         dy = fmaxf(dy, fmaxf(v.y - lo.y, hi.y - v.y));
         dz = fmaxf(dz, fmaxf(v.z - lo.z, hi.z - v.z));
-        const float ex = hi.x - lo.x, ey = hi.y - lo.y, ez = hi.z - lo.z, least = 0.125f * fmaxf(ex, fmaxf(ey, ez));
-        vol += fmaxf(ex, least) * fmaxf(ey, least) * fmaxf(ez, least);
     }
-    const float est = 1.1f * cbrtf((float)k * vol / (float)(64 * nodes) * 0.238732f);   // 3 / (4 pi)
-    return fminf(1.5f * plain_r, fminf(est, sqrtf(dx * dx + dy * dy + dz * dz) * 1.0001f));
+    return fminf(plain_r, sqrtf(dx * dx + dy * dy + dz * dz) * 1.0001f);
 }
 
 // The factor by which a radius grows that held tot < k particles.
@@ -612,9 +605,9 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
             uy = v.y;
             uz = v.z;
             // (a first radius whose ball wraps around the box, as of a chunk
-            // across a jump of the Morton curve, gives way to the plain one)
-            float r = a.chunk_r ? a.chunk_r[ch0 + (su - base) / (uint32_t)a.qpw] : INFINITY;
-            if (2.f * r >= 0.5f * box) r = gq_plain_radius(a.tree, v, su, base, end, k, plain_r);
+            // across a jump of the Morton curve, gives way to the boxes')
+            float r = a.chunk_r ? a.chunk_r[ch0 + (su - base) / (uint32_t)a.qpw] : plain_r;
+            if (2.f * r >= 0.5f * box) r = gq_box_radius(a.tree, v, su, base, end, k, plain_r);
             if (!(r > 0.f)) r = box * 1e-6f;
             r = fmaxf(r, __shfl_xor_sync(kAll, r, 1));
             r4 = fmaxf(r, __shfl_xor_sync(kAll, r, 2));
@@ -675,21 +668,21 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                     }
                 }
                 if (n2 < 0) {
-                    // several queries' region that crosses both a face and L/2,
-                    // or meets too many nodes: the first one alone, then
-                    // with a smaller radius as long as that may hold enough
+                    // too many nodes: a smaller radius as long as that may
+                    // hold enough
+                    const float few = warp_max(member ? rfew : 0.f);
+                    if (built && R > 1.05f * few) {
+                        ++tries;
+                        if (member) {
+                            rmany = R;
+                            rq = few > 0.f ? sqrtf(R * few) : 0.5f * R;
+                        }
+                        continue;
+                    }
+                    // several queries' region that crosses both a face and
+                    // L/2, or whose radii differ: the first one alone
                     alone = !alone && set != (0xffu << g0);
                     if (!alone) {
-                        const float few = warp_max(member ? rfew : 0.f);
-                        if (built && R > 1.05f * few) {
-                            ++tries;
-                            alone = true;
-                            if (member) {
-                                rmany = R;
-                                rq = few > 0.f ? sqrtf(R * few) : 0.5f * R;
-                            }
-                            continue;
-                        }
                         if (member && p == 0) a.hand[atomicAdd(a.hand_n, 1ull)] = sq;
                         todo &= ~set;
                     }
@@ -758,6 +751,7 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                             v[u] = sp[run[u]];
                         }
                     };
+                    cand += n0 * 8;   // every particle read, by the box's distance or its own
                     load(0);
                     int m = 0;
 #pragma unroll 1
@@ -788,7 +782,6 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                         }
                         const bool last = j + 16 >= n0;
                         if (!last) load(j + 16);
-                        cand += m & (last ? 0xff : 0xf0);
                         if (last) {
                             // up to a multiple of 16 with entries no test accepts
                             const float nan = __int_as_float(0x7fc00000);
