@@ -299,10 +299,10 @@ def stage(st):
     return {k[3:]: round(statistics.median(s[k] for s in st), 3) for k in keys}
 
 
-# (queries per warp, cells per radius, buffer factor): 4 queries per warp runs
-# the one-warp-per-query kernel, 8 and 16 the grouped count-then-gather
-# kernel, 32 one query per lane; a buffer factor selects the single-scan
-# kernel with that candidate buffer
+# (queries per radius chunk, cells per radius, buffer factor): 4, 8 and 16 run
+# the grouped kernel (cells per radius matter only to the queries it hands
+# over), 32 one query per lane; a buffer factor selects the single-scan kernel
+# with that candidate buffer
 CANDS = {"learned": [(4, 2, 0), (4, 1, 0), (4, 3, 0), (8, 1, 0), (8, 2, 0), (16, 1, 0), (4, 1, 3), (32, 1, 3)],
          "count": [(4, 2, 0), (4, 1, 0), (8, 1, 0), (16, 1, 0), (4, 1, 3), (32, 1, 3)],
          "plain": [(4, 2, 0), (8, 2, 0), (32, 1, 0), (32, 1, 3)]}
