@@ -43,7 +43,7 @@
 // the largest that does not wrap before one is handed over (4,913 particles:
 // 0.37 -> 0.08 ms), and halve where a region meets too many nodes.  (Limits
 // cut once instead, and no smaller radius: 4,200 of 16.8M queries handed over
-// and 33.6 ms instead of 31.3, 14,700 of 2.1M with the plain radius and 19.1
+// and 33.6 ms instead of 31.7, 14,700 of 2.1M with the plain radius and 19.1
 // ms instead of 7.4.)
 //
 // What bounds it: instruction issue and shared-memory wavefronts (58 % of
@@ -58,9 +58,9 @@
 // 33.6: a 16-byte read costs four wavefronts whether or not the four queries
 // read the same words.
 // Kernel time, with learned first radius unless stated (in brackets a warp
-// per query): 16.8M particles 31.3 ms (82.1), 64 subvolumes of 22M together
-// 43.3 ms (111.8), 3M with Ndens = Nhop = 65 (closed form) 7.0 ms (22.2), 2.1M
-// with the plain radius 7.4 ms (59.2), 4,913 particles 0.08 ms (0.99), 32,768
+// per query): 16.8M particles 31.7 ms (82.1), 64 subvolumes of 22M together
+// 43.6 ms (111.8), 3M with Ndens = Nhop = 65 (closed form) 7.0 ms (22.2), 2.1M
+// with the plain radius 7.5 ms (59.2), 4,913 particles 0.08 ms (0.99), 32,768
 // float64 particles 0.54 ms (5.2, the single-scan kernel).
 //
 // Results equal those of the other kNN kernels bit for bit: the same
@@ -503,8 +503,7 @@ __device__ __forceinline__ int gq_open(const BoxTree &t, int lv, const Region &r
 // The first radius at particle s where the given one wraps: the mean-density
 // distance, or where that is larger the distance to the farthest corner of
 // the boxes that hold the particle's own 64 (more than 64 wanted: 128)
-// neighbours in sort order, which is enough for k of them.  (64 subvolumes:
-// 43.3 ms, with the mean-density distance alone 48.2.)
+// neighbours in sort order, which is enough for k of them.
 __device__ __noinline__ float gq_box_radius(const BoxTree &t, float4 v, uint32_t s, uint32_t base, uint32_t end, int k,
                                               float plain_r)
 {
@@ -669,10 +668,14 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                 }
                 if (n2 < 0) {
                     // too many nodes: a smaller radius as long as that may
-                    // hold enough
+                    // hold enough: of the whole group with the plain radius
+                    // (2.1M particles: 7.4 ms, 9.6 one by one), otherwise of
+                    // one query at a time (64 subvolumes, learned radius:
+                    // 43.6 ms, 48.2 together)
                     const float few = warp_max(member ? rfew : 0.f);
-                    if (built && R > 1.05f * few) {
+                    if (built && R > 1.05f * few && (!a.chunk_r || alone || set == (0xffu << g0))) {
                         ++tries;
+                        alone = a.chunk_r != nullptr;
                         if (member) {
                             rmany = R;
                             rq = few > 0.f ? sqrtf(R * few) : 0.5f * R;
@@ -680,7 +683,7 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                         continue;
                     }
                     // several queries' region that crosses both a face and
-                    // L/2, or whose radii differ: the first one alone
+                    // L/2, or meets too many nodes: the first one alone
                     alone = !alone && set != (0xffu << g0);
                     if (!alone) {
                         if (member && p == 0) a.hand[atomicAdd(a.hand_n, 1ull)] = sq;
