@@ -1136,8 +1136,9 @@ int knn_launch(hop_ctx *c, const KnnArgs &a, bool f64, int qpw, int cpr)
     // candidate-buffer factor was set (the single-scan kernel below)
     if (!f64 && c->capf == 0 && (qpw == 4 || qpw == 8 || qpw == 16)) return knn_gq_launch(c, a, false, qpw, cpr);
     // float64, whatever the queries per warp: the same kernel (the radius is
-    // per chunk of that many)
-    if (f64 && c->capf == 0 && !a.seg) return knn_gq_launch(c, a, true, qpw, cpr);
+    // per chunk of that many), up to box sides whose squares stay well inside
+    // double's range
+    if (f64 && c->capf == 0 && !a.seg && std::abs(std::ilogb(a.box)) <= 400) return knn_gq_launch(c, a, true, qpw, cpr);
     if (a.seg) {
         // batched passes: float32 positions, 4, 8, 16 or 32 queries per warp
         if (f64) return ctx_fail(c, HOP_EINVAL, "batched passes take float32 positions");

@@ -34,17 +34,17 @@
 // A query is certified when at least Ndens particles lie within R; the
 // others search again with a larger R.  A group whose region crosses both a
 // face and L/2 is served one query at a time.  What this kernel does not take
-// -- a ball that wraps around the box, more nodes than it lists at every
-// radius that holds Ndens, more than 32 particles too many at the Ndens-th
-// distance, float64 distances too close for float32 to bin -- it hands over
-// to a warp-per-query kernel (knn_cg.cu; float64: knn.cu), which runs after
-// it over the list of such queries.  Such queries take 0.3 ms however few
-// there are, and 2 to 8 ms where their radii are far too large, so radii reach
-// the largest that does not wrap before one is handed over (4,913 particles:
-// 0.37 -> 0.08 ms), and halve where a region meets too many nodes.  (Limits
-// cut once instead, and no smaller radius: 4,200 of 16.8M queries handed over
-// and 33.6 ms instead of 31.7, 14,700 of 2.1M with the plain radius and 19.1
-// ms instead of 7.4.)
+// -- a ball that wraps around the box, a float32 box whose squares leave
+// float32's range, more nodes than it lists at every radius that holds Ndens,
+// more than 32 particles too many at the Ndens-th distance, float64 distances
+// too close for float32 to bin -- it hands over to a warp-per-query kernel
+// (knn_cg.cu; float64: knn.cu), which runs after it over the list of such
+// queries.  Such queries take 0.3 ms however few there are, and 2 to 8 ms
+// where their radii are far too large, so radii reach the largest that does
+// not wrap before one is handed over (4,913 particles: 0.37 -> 0.08 ms), and
+// halve where a region meets too many nodes.  (Limits cut once instead, and
+// no smaller radius: 4,200 of 16.8M queries handed over and 33.6 ms instead
+// of 31.7, 14,700 of 2.1M with the plain radius and 19.1 ms instead of 7.4.)
 //
 // What bounds it: instruction issue and shared-memory wavefronts (58 % of
 // issue slots and 66 % of wavefronts at 16 warps per SM, 1.35k warp
@@ -70,6 +70,7 @@
 #include "knn_common.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <math.h>
 #include <type_traits>
 
@@ -87,6 +88,13 @@ constexpr int kGqBins = 32;            // histogram bins, linear in d^2
 constexpr int kGqCutBins = 16;         // the same for a cut during the search
 constexpr int kGqTile = 144;           // particles staged: 16 runs, and up to 15 left over
 constexpr int kGqTries = 96;
+// Box sides whose float32 squares stay in range: the largest square is 3 L^2
+// (2^121.6), and the smallest margin of a box test, 1e-12 L^2, is still
+// hundreds of denormal steps, far above the test's rounding.  Beyond them a
+// limit could become infinite (and an infinite d^2 has no bin) or a neighbour
+// be missed: float32 particles in such boxes go to the warp-per-query kernel,
+// float64 ones are searched in units of the box.
+constexpr float kGqBoxMin = 0x1p-50f, kGqBoxMax = 0x1p60f;
 
 struct GqDev {
     const float4 *spos;
@@ -96,8 +104,9 @@ struct GqDev {
     int64_t n_tasks;                   // units of 16 queries, in `split` parts each
     int split;
     int qpw;                           // queries per radius chunk
-    float box, norm;
+    float box, norm;                   // F64: the box in the search's units, in [1, 2)
     double box64, norm64;
+    float unit;                        // F64: the search's units per unit of the caller's
     int k, n_out, ld_out, capq;
     const float *chunk_r;
     float plain_r;
@@ -595,6 +604,12 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
         }
         const int nu = (int)min((int64_t)per_task, (int64_t)end - (int64_t)s_unit);
         if (nu <= 0) continue;   // the last unit of a subvolume may hold fewer parts
+        if constexpr (!F64) {
+            if (!(box >= kGqBoxMin && box <= kGqBoxMax)) {
+                if (lane < nu) a.hand[atomicAdd(a.hand_n, 1ull)] = s_unit + (uint32_t)lane;
+                continue;
+            }
+        }
         // lane i (and i + 16) holds query i of the unit; r4: its group's radius
         float ux, uy, uz, r4, ru;
         {
@@ -606,6 +621,8 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
             // (a first radius whose ball wraps around the box, as of a chunk
             // across a jump of the Morton curve, gives way to the boxes')
             float r = a.chunk_r ? a.chunk_r[ch0 + (su - base) / (uint32_t)a.qpw] : plain_r;
+            if constexpr (F64)
+                if (a.chunk_r) r *= a.unit;
             if (2.f * r >= 0.5f * box) r = gq_box_radius(a.tree, v, su, base, end, k, plain_r);
             if (!(r > 0.f)) r = box * 1e-6f;
             r = fmaxf(r, __shfl_xor_sync(kAll, r, 1));
@@ -1030,12 +1047,15 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
     }
 }
 
-// Rounded copies of double-precision particles, the padding included.
-__global__ void to_float4_kernel(const double4 *__restrict__ in, int64_t n, float4 *__restrict__ out)
+// Rounded copies of double-precision particles, the padding included, times
+// 2^e (exact): a box side of any size becomes one in [1, 2), so that neither
+// the search's squares nor its error bounds leave float32's range.
+__global__ void to_float4_kernel(const double4 *__restrict__ in, int64_t n, int e, float4 *__restrict__ out)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const double4 v = in[i];
-        out[i] = make_float4((float)v.x, (float)v.y, (float)v.z, __uint_as_float((uint32_t)__double_as_longlong(v.w)));
+        out[i] = make_float4((float)scalbn(v.x, e), (float)scalbn(v.y, e), (float)scalbn(v.z, e),
+                             __uint_as_float((uint32_t)__double_as_longlong(v.w)));
     }
 }
 
@@ -1044,11 +1064,19 @@ template <bool SEG, bool F64> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int 
     GqDev d;
     d.spos64 = nullptr;
     d.spos = (const float4 *)ka.spos;
+    d.box = (float)ka.box;
+    d.plain_r = ka.plain_r;
+    d.unit = 1.f;
     if constexpr (F64) {
+        const int e = -std::ilogb(ka.box);
+        const double side = std::scalbn(ka.box, e);
+        d.box = (float)side;
+        d.plain_r = plain_radius_for(ka.n, side, ka.k);
+        d.unit = (float)std::scalbn(1.0, e);   // (0 or inf where the caller's radii are inf or 0: the boxes' radius then)
         const int64_t m = ka.n + kSposPad;
         float4 *f = (float4 *)ctx_buf(c, S_SPOS_F, (size_t)m * sizeof(float4));
         if (!f) return HOP_ENOMEM;
-        to_float4_kernel<<<grid_for(c, m), 256, 0, c->stream>>>((const double4 *)ka.spos, m, f);
+        to_float4_kernel<<<grid_for(c, m), 256, 0, c->stream>>>((const double4 *)ka.spos, m, e, f);
         HOP_LAUNCH(c);
         d.spos = f;
         d.spos64 = (const double4 *)ka.spos;
@@ -1065,7 +1093,6 @@ template <bool SEG, bool F64> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int 
     d.split = units >= 2 * warps ? 1 : units >= warps ? 2 : 4;
     d.n_tasks = units * d.split;
     d.qpw = qpw;
-    d.box = (float)ka.box;
     d.norm = (float)(ka.box * ka.box * ka.box / ((double)(ka.n_norm > 0 ? ka.n_norm : ka.n) * 3.14159265358979323846));
     d.box64 = ka.box;
     d.norm64 = ka.box * ka.box * ka.box / ((double)(ka.n_norm > 0 ? ka.n_norm : ka.n) * 3.14159265358979323846);
@@ -1074,7 +1101,6 @@ template <bool SEG, bool F64> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int 
     d.ld_out = ka.ld_out;
     d.capq = ((ka.k + 32 + 7) / 8) * 8;
     d.chunk_r = ka.chunk_r;
-    d.plain_r = ka.plain_r;
     d.seg = ka.seg;
     d.B = ka.B;
     d.nbr_s = ka.nbr_s;
