@@ -604,12 +604,6 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
         }
         const int nu = (int)min((int64_t)per_task, (int64_t)end - (int64_t)s_unit);
         if (nu <= 0) continue;   // the last unit of a subvolume may hold fewer parts
-        if constexpr (!F64) {
-            if (!(box >= kGqBoxMin && box <= kGqBoxMax)) {
-                if (lane < nu) a.hand[atomicAdd(a.hand_n, 1ull)] = s_unit + (uint32_t)lane;
-                continue;
-            }
-        }
         // lane i (and i + 16) holds query i of the unit; r4: its group's radius
         float ux, uy, uz, r4, ru;
         {
@@ -625,6 +619,9 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                 if (a.chunk_r) r *= a.unit;
             if (2.f * r >= 0.5f * box) r = gq_box_radius(a.tree, v, su, base, end, k, plain_r);
             if (!(r > 0.f)) r = box * 1e-6f;
+            // (a ball that wraps is handed over)
+            if constexpr (!F64)
+                if (!(box >= kGqBoxMin && box <= kGqBoxMax)) r = INFINITY;
             r = fmaxf(r, __shfl_xor_sync(kAll, r, 1));
             r4 = fmaxf(r, __shfl_xor_sync(kAll, r, 2));
             ru = warp_max(r4);
