@@ -87,7 +87,10 @@ constexpr int kGqN0 = 256;             // runs of eight particles held at once
 constexpr int kGqBins = 32;            // histogram bins, linear in d^2
 constexpr int kGqCutBins = 16;         // the same for a cut during the search
 constexpr int kGqTile = 144;           // particles staged: 16 runs, and up to 15 left over
-constexpr int kGqTries = 96;
+constexpr int kGqTries = 96;           // searches and halvings until some query of a group is done
+// A region is grown by this much of the box whatever its radius: below it a
+// smaller radius meets the same nodes.
+constexpr float kGqFinest = 0x1p-20f;
 // Box sides whose float32 squares stay in range: the largest square is 3 L^2
 // (2^121.6), and the smallest margin of a box test, 1e-12 L^2, is still
 // hundreds of denormal steps, far above the test's rounding.  Beyond them a
@@ -204,7 +207,7 @@ struct Region {
     __device__ __forceinline__ bool build(bool in, float &x, float &y, float &z, float r, float box_)
     {
         box = box_;
-        const float half = 0.5f * box, eps = box * 9.5367431640625e-7f;   // 2^-20 of the box: far above rounding
+        const float half = 0.5f * box, eps = box * kGqFinest;   // far above rounding
         lx = warp_min(in ? x : INFINITY);
         hx = warp_max(in ? x : -INFINITY);
         ly = warp_min(in ? y : INFINITY);
@@ -644,9 +647,9 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                         ez = qz - __shfl_up_sync(kAll, qz, 8);
             const uint32_t cuts = __ballot_sync(kAll, p == 0 && q > 0 && q < nq && ex * ex + ey * ey + ez * ez > R0 * R0);
             uint32_t todo = (1u << (8 * nq - 1)) * 2u - 1u;   // the lanes of the queries still to be served
-            // the query's radius; the largest that held too few, the smallest that met too many nodes
-            float rq = R0, rfew = 0.f, rmany = INFINITY;
-            bool alone = false;
+            // the query's radius; the largest that held too few
+            float rq = R0, rfew = 0.f;
+            bool alone = false;   // the first query left is searched by itself until it is done
             int tries = 0;
             while (todo) {
                 // from the first one up to the next cut, or the first alone
@@ -685,15 +688,19 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                     // hold enough: of the whole group with the plain radius
                     // (2.1M particles: 7.4 ms, 9.6 one by one), otherwise of
                     // one query at a time (64 subvolumes, learned radius:
-                    // 43.6 ms, 48.2 together)
+                    // 43.6 ms, 48.2 together).  The radius is remembered only
+                    // through the one that held too few, which grows with
+                    // every search: a limit kept from a region that met too
+                    // many nodes binds queries it was not measured on, and
+                    // they crept up to it until the tries ran out (200
+                    // particles in a void around a ball of 100,000, plain
+                    // radius: 25.2 ms and 3,059 searches that held too few,
+                    // now 3.6 ms and 257)
                     const float few = warp_max(member ? rfew : 0.f);
-                    if (built && R > 1.05f * few && (!a.chunk_r || alone || set == (0xffu << g0))) {
+                    if (built && R > fmaxf(1.05f * few, kGqFinest * box) &&
+                        (!a.chunk_r || alone || set == (0xffu << g0))) {
                         ++tries;
-                        alone = a.chunk_r != nullptr;
-                        if (member) {
-                            rmany = R;
-                            rq = few > 0.f ? sqrtf(R * few) : 0.5f * R;
-                        }
+                        if (member) rq = few > 0.f ? sqrtf(R * few) : 0.5f * R;
                         continue;
                     }
                     // several queries' region that crosses both a face and
@@ -702,10 +709,10 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                     if (!alone) {
                         if (member && p == 0) a.hand[atomicAdd(a.hand_n, 1ull)] = sq;
                         todo &= ~set;
+                        tries = 0;
                     }
                     continue;
                 }
-                alone = false;
                 ++search_acc;
                 if (n2 > 8) {
                     // a large region: the query's own node first, so that the
@@ -1019,6 +1026,10 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                 }
                 if (member && crowd && p == 0) a.hand[atomicAdd(a.hand_n, 1ull)] = (uint32_t)sq;
                 todo &= ~__ballot_sync(kAll, ok || (member && crowd));
+                if (!(todo & set)) {
+                    alone = false;
+                    tries = 0;
+                }
                 // the others of the set hold too few within R: a larger one, at
                 // first not beyond the largest this kernel takes
                 if (todo & set) {
@@ -1029,7 +1040,6 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                         rq = R * fminf(gq_grow(k, tot), 8.f);
                         if (R < 0.99f * most) rq = fminf(rq, most);
                         rfew = R;
-                        rq = fminf(rq, sqrtf(R * rmany));
                     }
                 }
                 __syncwarp();
