@@ -441,6 +441,9 @@ int knn32_launch(hop_ctx *c, const KnnArgs &a, int cpr);   // knn32.cu: one quer
 int knn_gq_launch(hop_ctx *c, const KnnArgs &a, bool f64, int qpw, int cpr);
 int knn_hand_f64_launch(hop_ctx *c, const KnnArgs &a, int qpw, int cpr, const uint32_t *hand,
                         const unsigned long long *hand_n, unsigned long long *counter);
+// the same for runs of four consecutive queries, given by their first
+int knn_runs_f64_launch(hop_ctx *c, const KnnArgs &a, int qpw, int cpr, const uint32_t *runs,
+                        const unsigned long long *runs_n, unsigned long long *counter);
 // knn_cg.cu: one warp per query, over a list of *hand_n sorted indices;
 // `counter` is a device word that is zero on entry
 int knn_wq_launch(hop_ctx *c, const KnnArgs &a, int qpw, int cpr, const uint32_t *hand,

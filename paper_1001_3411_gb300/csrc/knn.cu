@@ -464,7 +464,7 @@ template <typename T> struct KnnDev {
     unsigned long long *chunk_counter;
     unsigned long long *counters;
     uint32_t *err;
-    const uint32_t *hand;               // when set: the queries (sorted index), one per warp ...
+    const uint32_t *hand;               // when set: the first query (sorted index) of each warp's ...
     const unsigned long long *hand_n;   // ... their number ...
     int qpw;                            // ... and the queries per radius chunk
 };
@@ -533,6 +533,8 @@ __global__ void __launch_bounds__(kKnnThreads, 4) knn_kernel(KnnDev<T> a)
 
     const int k = a.k;
     unsigned long long cand_acc = 0, search_acc = 0, retry_acc = 0, warp_acc = 0;
+    // an empty list, the ordinary case, costs no atomics
+    if (a.hand && *a.hand_n == 0) return;
 
     for (;;) {
         unsigned long long ch = 0;
@@ -1125,6 +1127,12 @@ int knn_hand_f64_launch(hop_ctx *c, const KnnArgs &a, int qpw, int cpr, const ui
                         const unsigned long long *hand_n, unsigned long long *counter)
 {
     return knn_run<double, 32, false>(c, a, cpr, hand, hand_n, counter, qpw);
+}
+
+int knn_runs_f64_launch(hop_ctx *c, const KnnArgs &a, int qpw, int cpr, const uint32_t *runs,
+                        const unsigned long long *runs_n, unsigned long long *counter)
+{
+    return knn_run<double, 8, false>(c, a, cpr, runs, runs_n, counter, qpw);
 }
 
 int knn_launch(hop_ctx *c, const KnnArgs &a, bool f64, int qpw, int cpr)

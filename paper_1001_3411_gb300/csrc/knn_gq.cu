@@ -38,13 +38,14 @@
 // float32's range, more nodes than it lists at every radius that holds Ndens,
 // more than 32 particles too many at the Ndens-th distance, float64 distances
 // too close for float32 to bin -- it hands over to a warp-per-query kernel
-// (knn_cg.cu; float64: knn.cu), which runs after it over the list of such
-// queries.  Such queries take 0.3 ms however few there are, and 2 to 8 ms
-// where their radii are far too large, so radii reach the largest that does
-// not wrap before one is handed over (4,913 particles: 0.37 -> 0.08 ms), and
-// halve where a region meets too many nodes.  (Limits cut once instead, and
-// no smaller radius: 4,200 of 16.8M queries handed over and 33.6 ms instead
-// of 31.7, 14,700 of 2.1M with the plain radius and 19.1 ms instead of 7.4.)
+// (knn_cg.cu; float64: knn.cu, and whole nodes of such particles four queries
+// per warp), which runs after it over the list of such queries.  Such queries
+// take 0.3 ms however few there are, and 2 to 8 ms where their radii are far
+// too large, so radii reach the largest that does not wrap before one is
+// handed over (4,913 particles: 0.37 -> 0.08 ms), and halve where a region
+// meets too many nodes.  (Limits cut once instead, and no smaller radius:
+// 4,200 of 16.8M queries handed over and 33.6 ms instead of 31.7, 14,700 of
+// 2.1M with the plain radius and 19.1 ms instead of 7.4.)
 //
 // What bounds it: instruction issue and shared-memory wavefronts (58 % of
 // issue slots and 66 % of wavefronts at 16 warps per SM, 1.35k warp
@@ -91,6 +92,9 @@ constexpr int kGqTries = 96;           // searches and halvings until some query
 // A region is grown by this much of the box whatever its radius: below it a
 // smaller radius meets the same nodes.
 constexpr float kGqFinest = 0x1p-20f;
+// Float64 particles: within a ball of this radius the rounding's slack is more
+// than a bin, whatever the limit.
+constexpr float kGqFinest64 = 0x1p-15f;
 // Box sides whose float32 squares stay in range: the largest square is 3 L^2
 // (2^121.6), and the smallest margin of a box test, 1e-12 L^2, is still
 // hundreds of denormal steps, far above the test's rounding.  Beyond them a
@@ -120,6 +124,8 @@ struct GqDev {
     float *rk_s;
     uint32_t *hand;                    // queries handed over ...
     unsigned long long *hand_n;        // ... and their number
+    uint32_t *runs;                    // F64: runs of four queries handed over ...
+    unsigned long long *runs_n;        // ... and their number
     unsigned long long *task_counter, *counters;
 };
 
@@ -532,6 +538,19 @@ __device__ __noinline__ float gq_box_radius(const BoxTree &t, float4 v, uint32_t
     return fminf(plain_r, sqrtf(dx * dx + dy * dy + dz * dz) * 1.0001f);
 }
 
+// Whether a full 512-particle node of double-precision particles is too tight
+// for the float search.  That search is certain of an order only while the
+// rounding's slack stays below a bin, which is so for limits above 2^-14.1 of
+// the box; a node with a diagonal below 2^-17 lies within one bin of any such
+// limit, with more particles than a query's list holds.
+__device__ __noinline__ bool gq_tight_node(const BoxTree &t, uint32_t node, uint32_t end, float box)
+{
+    if (((uint64_t)node + 1) * 512 > end) return false;
+    const float4 lo = t.lo[t.off[2] + node], hi = t.hi[t.off[2] + node];
+    const float dx = hi.x - lo.x, dy = hi.y - lo.y, dz = hi.z - lo.z;
+    return dx * dx + dy * dy + dz * dz < box * box * 0x1p-34f;
+}
+
 // The factor by which a radius grows that held tot < k particles.
 __device__ __noinline__ float gq_grow(int k, int tot)
 {
@@ -607,6 +626,16 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
         }
         const int nu = (int)min((int64_t)per_task, (int64_t)end - (int64_t)s_unit);
         if (nu <= 0) continue;   // the last unit of a subvolume may hold fewer parts
+        if constexpr (F64) {
+            // (63,000 particles, 60,000 of them within 1e-6 of the box: 172 ms
+            // where every query was searched and handed over by itself, 120 ms
+            // so, 123 ms through the single-scan kernel alone)
+            if (__any_sync(kAll, gq_tight_node(a.tree, s_unit >> 9, end, box))) {
+                if (lane < nu && lane % 4 == 0) a.runs[atomicAdd(a.runs_n, 1ull)] = s_unit + (uint32_t)lane;
+                warp_acc += (nu + 3) / 4;
+                continue;
+            }
+        }
         // lane i (and i + 16) holds query i of the unit; r4: its group's radius
         float ux, uy, uz, r4, ru;
         {
@@ -697,7 +726,7 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
                     // radius: 25.2 ms and 3,059 searches that held too few,
                     // now 3.6 ms and 257)
                     const float few = warp_max(member ? rfew : 0.f);
-                    if (built && R > fmaxf(1.05f * few, kGqFinest * box) &&
+                    if (built && R > fmaxf(1.05f * few, (F64 ? kGqFinest64 : kGqFinest) * box) &&
                         (!a.chunk_r || alone || set == (0xffu << g0))) {
                         ++tries;
                         if (member) rq = few > 0.f ? sqrtf(R * few) : 0.5f * R;
@@ -1055,13 +1084,14 @@ __global__ void __launch_bounds__(kGqWarps * 32, F64 ? 3 : 4) knn_gq_kernel(cons
 }
 
 // Rounded copies of double-precision particles, the padding included, times
-// 2^e (exact): a box side of any size becomes one in [1, 2), so that neither
-// the search's squares nor its error bounds leave float32's range.
-__global__ void to_float4_kernel(const double4 *__restrict__ in, int64_t n, int e, float4 *__restrict__ out)
+// `unit`, a power of two (exact): a box side of any size becomes one in
+// [1, 2), so that neither the search's squares nor its error bounds leave
+// float32's range.
+__global__ void to_float4_kernel(const double4 *__restrict__ in, int64_t n, double unit, float4 *__restrict__ out)
 {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const double4 v = in[i];
-        out[i] = make_float4((float)scalbn(v.x, e), (float)scalbn(v.y, e), (float)scalbn(v.z, e),
+        out[i] = make_float4((float)(v.x * unit), (float)(v.y * unit), (float)(v.z * unit),
                              __uint_as_float((uint32_t)__double_as_longlong(v.w)));
     }
 }
@@ -1075,15 +1105,14 @@ template <bool SEG, bool F64> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int 
     d.plain_r = ka.plain_r;
     d.unit = 1.f;
     if constexpr (F64) {
-        const int e = -std::ilogb(ka.box);
-        const double side = std::scalbn(ka.box, e);
+        const double unit = std::scalbn(1.0, -std::ilogb(ka.box)), side = ka.box * unit;
         d.box = (float)side;
         d.plain_r = plain_radius_for(ka.n, side, ka.k);
-        d.unit = (float)std::scalbn(1.0, e);   // (0 or inf where the caller's radii are inf or 0: the boxes' radius then)
+        d.unit = (float)unit;   // (0 or inf where the caller's radii are inf or 0: the boxes' radius then)
         const int64_t m = ka.n + kSposPad;
         float4 *f = (float4 *)ctx_buf(c, S_SPOS_F, (size_t)m * sizeof(float4));
         if (!f) return HOP_ENOMEM;
-        to_float4_kernel<<<grid_for(c, m), 256, 0, c->stream>>>((const double4 *)ka.spos, m, e, f);
+        to_float4_kernel<<<grid_for(c, m), 256, 0, c->stream>>>((const double4 *)ka.spos, m, unit, f);
         HOP_LAUNCH(c);
         d.spos = f;
         d.spos64 = (const double4 *)ka.spos;
@@ -1114,11 +1143,13 @@ template <bool SEG, bool F64> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int 
     d.dens_s = ka.dens_s;
     d.rk_s = ka.rk_s;
     d.counters = c->d_counters;
+    // (the words after the counters are zero: a pass clears them at its start)
     d.task_counter = c->d_counters + kCntNum;
     d.hand_n = c->d_counters + kCntNum + 1;
-    d.hand = (uint32_t *)ctx_buf(c, S_KNN_HAND, (size_t)ka.n * sizeof(uint32_t));
+    d.runs_n = d.hand_n + 2;
+    d.hand = (uint32_t *)ctx_buf(c, S_KNN_HAND, (size_t)(ka.n + (F64 ? ka.n / 4 + 4 : 0)) * sizeof(uint32_t));
     if (!d.hand) return HOP_ENOMEM;
-    HOP_CUDA(c, cudaMemsetAsync(d.task_counter, 0, 3 * sizeof(unsigned long long), c->stream));
+    d.runs = d.hand + ka.n;
     const size_t smem = (size_t)GqSmem::total(d.capq, F64) * kGqWarps;
     auto kern = knn_gq_kernel<SEG, F64>;
     HOP_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1129,7 +1160,10 @@ template <bool SEG, bool F64> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int 
     const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((int64_t)per_sm * c->num_sms, need));
     kern<<<(unsigned)blocks, kGqWarps * 32, smem, c->stream>>>(d);
     HOP_LAUNCH(c);
-    if constexpr (F64) return knn_hand_f64_launch(c, ka, qpw, cpr, d.hand, d.hand_n, d.hand_n + 1);
+    if constexpr (F64) {
+        const int rr = knn_runs_f64_launch(c, ka, qpw, cpr, d.runs, d.runs_n, d.runs_n + 1);
+        return rr ? rr : knn_hand_f64_launch(c, ka, qpw, cpr, d.hand, d.hand_n, d.hand_n + 1);
+    }
     return knn_wq_launch(c, ka, qpw, cpr, d.hand, d.hand_n, d.hand_n + 1);
 }
 
