@@ -19,24 +19,30 @@ int ctx_cuda(hop_ctx *c, cudaError_t e, const char *what)
     return e == cudaErrorMemoryAllocation ? HOP_ENOMEM : HOP_ECUDA;
 }
 
+void ctx_release(hop_ctx *c, Slot s)
+{
+    DevBuf &b = c->buf[s];
+    if (!b.p) return;
+    if (c->capturing) {
+        // nodes captured earlier use the old buffer: keep it with the graph
+        c->graveyard.push_back(b.p);
+    } else {
+        // work already enqueued may still use the old buffer
+        cudaStreamSynchronize(c->stream);
+        cudaFree(b.p);
+    }
+    b.p = nullptr;
+    b.cap = 0;
+    ++c->buf_epoch;   // a cached graph that used this slot is stale
+}
+
 void *ctx_buf(hop_ctx *c, Slot s, size_t bytes)
 {
     DevBuf &b = c->buf[s];
     if (bytes == 0) bytes = 16;
     if (b.cap >= bytes) return b.p;
-    if (b.p) {
-        if (c->capturing) {
-            // nodes captured earlier use the old buffer: keep it with the graph
-            c->graveyard.push_back(b.p);
-        } else {
-            // work already enqueued may still use the old buffer
-            cudaStreamSynchronize(c->stream);
-            cudaFree(b.p);
-        }
-        b.p = nullptr;
-        b.cap = 0;
-    }
-    ++c->buf_epoch;   // a cached graph that used this slot is stale
+    ctx_release(c, s);
+    ++c->buf_epoch;
     size_t want = bytes + bytes / 8;
     want = (want + (size_t(2) << 20) - 1) & ~((size_t(2) << 20) - 1);
     cudaError_t e = cudaMalloc(&b.p, want);

@@ -136,6 +136,7 @@ enum { kCntCand = 0, kCntSearch, kCntRetry, kCntWarps, kCntQual, kCntEdges, kCnt
 int ctx_fail(hop_ctx *c, int code, const std::string &msg);
 int ctx_cuda(hop_ctx *c, cudaError_t e, const char *what);
 void *ctx_buf(hop_ctx *c, Slot s, size_t bytes);   // nullptr on failure (err set)
+void ctx_release(hop_ctx *c, Slot s);              // gives a slot's buffer back
 int ctx_check_device_error(hop_ctx *c);            // syncs; maps the error word
 
 #define HOP_CUDA(ctx, call)                                   \

@@ -1141,12 +1141,18 @@ int knn_launch(hop_ctx *c, const KnnArgs &a, bool f64, int qpw, int cpr)
     if (cpr < 1 || cpr > 4) cpr = 1;
     if (qpw == 32 && !f64) return knn32_launch(c, a, cpr);   // one query per lane
     // float32 with 4, 8 or 16 queries per warp: the grouped kernel, unless a
-    // candidate-buffer factor was set (the single-scan kernel below)
-    if (!f64 && c->capf == 0 && (qpw == 4 || qpw == 8 || qpw == 16)) return knn_gq_launch(c, a, false, qpw, cpr);
-    // float64, whatever the queries per warp: the same kernel (the radius is
-    // per chunk of that many), up to box sides whose squares stay well inside
-    // double's range
-    if (f64 && c->capf == 0 && !a.seg && std::abs(std::ilogb(a.box)) <= 400) return knn_gq_launch(c, a, true, qpw, cpr);
+    // candidate-buffer factor was set (the single-scan kernel below); float64,
+    // whatever the queries per warp: the same kernel (the radius is per chunk
+    // of that many), up to box sides whose squares stay well inside double's
+    // range
+    if (c->capf == 0 && (f64 ? !a.seg && std::abs(std::ilogb(a.box)) <= 400 : qpw == 4 || qpw == 8 || qpw == 16)) {
+        const int rc = knn_gq_launch(c, a, f64, qpw, cpr);
+        if (rc != HOP_ENOMEM) return rc;
+        // no memory for its boxes and lists (9 bytes per particle, float64 26):
+        // the single-scan kernel needs none
+        for (Slot s : {S_KNN_HAND, S_SPOS_F, S_BOX}) ctx_release(c, s);
+        c->err.clear();
+    }
     if (a.seg) {
         // batched passes: float32 positions, 4, 8, 16 or 32 queries per warp
         if (f64) return ctx_fail(c, HOP_EINVAL, "batched passes take float32 positions");
