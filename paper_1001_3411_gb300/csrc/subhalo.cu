@@ -344,20 +344,33 @@ int subhalos(hop_ctx *c, const uint32_t *chain, const float *dens, const uint64_
     HOP_CUDA(c, cudaStreamSynchronize(c->stream));
     const int64_t C = hp[0];
     // thresholds per batch: at most kLev, fewer where the arrays over (level,
-    // chain) would grow past 2^28 entries
+    // chain) would grow past 2^28 entries, or past the memory that is left
     const int64_t Cp = std::max<int64_t>(C, 1), mp = std::max<int64_t>(m, 1);
-    const int LB = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(L, kLev), (int64_t(1) << 28) / Cp));
+    int LB = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(L, kLev), (int64_t(1) << 28) / Cp));
     const bool with_sum = f > 0.0 || n >= (int64_t(1) << 29);
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += align256(bytes); return o; };
+    // what does not depend on LB first
     const size_t o_cnt = take(Cp * kLev * 4), o_sum = take(with_sum ? Cp * kLev * 8 : 8), o_pkey = take(Cp * 8),
-                 o_row = take(Cp * kLev * 4), o_parent = take(Cp * LB * 4), o_ccnt = take(Cp * LB * 8),
-                 o_csum = take(with_sum ? Cp * LB * 8 : 8), o_cpk = take(Cp * LB * 8), o_flag = take((Cp * LB + 1) * 4),
-                 o_pos = take((Cp * LB + 1) * 4), o_rank = take(Cp * LB * 4), o_ea = take(mp * 4), o_eb = take(mp * 4),
-                 o_gk = take(Cp * 8), o_gkb = take(Cp * 8), o_gv = take(Cp * 4), o_gvb = take(Cp * 4),
-                 o_tmp = take(radix_sort_scratch_bytes(Cp));
-    char *base = (char *)ctx_buf(c, S_SUB_C, off);
+                 o_row = take(Cp * kLev * 4), o_ea = take(mp * 4), o_eb = take(mp * 4), o_gk = take(Cp * 8),
+                 o_gkb = take(Cp * 8), o_gv = take(Cp * 4), o_gvb = take(Cp * 4),
+                 o_tmp = take(radix_sort_scratch_bytes(Cp)), fixed = off;
+    size_t o_parent, o_ccnt, o_csum, o_cpk, o_flag, o_pos, o_rank;
+    char *base = nullptr;
+    for (;; LB = (LB + 1) / 2) {
+        off = fixed;
+        o_parent = take(Cp * LB * 4);
+        o_ccnt = take(Cp * LB * 8);
+        o_csum = take(with_sum ? Cp * LB * 8 : 8);
+        o_cpk = take(Cp * LB * 8);
+        o_flag = take((Cp * LB + 1) * 4);
+        o_pos = take((Cp * LB + 1) * 4);
+        o_rank = take(Cp * LB * 4);
+        base = (char *)ctx_buf(c, S_SUB_C, off);
+        if (base || LB == 1) break;
+    }
     if (!base) return HOP_ENOMEM;
+    c->err.clear();
     uint32_t *cnt = (uint32_t *)(base + o_cnt), *parent = (uint32_t *)(base + o_parent),
              *flag = (uint32_t *)(base + o_flag), *gpos = (uint32_t *)(base + o_pos), *ea = (uint32_t *)(base + o_ea),
              *eb = (uint32_t *)(base + o_eb);

@@ -76,3 +76,35 @@ def test_batched_pass_without_room_for_the_boxes(eager):
         torch.cuda.empty_cache()
     for key in ("dens", "group", "nbr"):
         assert torch.equal(out[key], ref[key]), key
+
+
+def test_subhalos_without_room_for_eight_thresholds():
+    """Arrays for eight thresholds at once (about 0.35 kB per chain) do not
+    fit, those for fewer do."""
+    hopgpu.build_library()
+    rng = np.random.default_rng(4)
+    n, n_chains = 2000000, 400000
+    chain = rng.integers(0, n_chains, n).astype(np.int32)
+    chain[:n_chains] = np.arange(n_chains)
+    dens = (100.0 + rng.random(n) * 1000.0).astype(np.float32)
+    dens[:n_chains] = (1200.0 + rng.permutation(n_chains) * 1e-3).astype(np.float32)
+    nbr = rng.integers(0, n, (n, 4)).astype(np.int32)
+    levels = [100.0 + 100.0 * i for i in range(8)]
+    dev = [torch.from_numpy(x).cuda() for x in (chain, dens, nbr)]
+    hop = hopgpu.Hop(0)
+    try:
+        sub, n_sub = hop.hop_subhalos(*dev, 4, 100.0, levels)
+    finally:
+        hop.close()
+    hop = hopgpu.Hop(0)
+    hop.hop_subhalos(*dev, 4, 100.0, levels[:1])   # every other buffer of the call
+    again = torch.empty_like(sub)
+    del again                                      # kept by torch for the labels below
+    rest = _fill(48 * MB)
+    try:
+        out, n_out = hop.hop_subhalos(*dev, 4, 100.0, levels)
+    finally:
+        del rest
+        hop.close()
+        torch.cuda.empty_cache()
+    assert torch.equal(out, sub) and np.array_equal(n_out, n_sub)
