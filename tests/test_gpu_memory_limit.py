@@ -9,7 +9,6 @@ if not torch.cuda.is_available():
     pytest.skip("needs a CUDA GPU", allow_module_level=True)
 
 import paper_1001_3411_gb300 as hopgpu
-import synth
 
 pytestmark = pytest.mark.gpu
 MB = 1 << 20
