@@ -105,7 +105,6 @@ int box_tree_build(hop_ctx *c, const float4 *spos, int64_t n, BoxTree *t)
         if (triples == 4) return ctx_fail(c, HOP_EINVAL, "too many particles for the box levels");
         m = b;
     }
-    t->levels = 3 * triples;
     float4 *buf = (float4 *)ctx_buf(c, S_BOX, (size_t)total * 2 * sizeof(float4));
     if (!buf) return HOP_ENOMEM;
     float4 *lo = buf, *hi = buf + total;

@@ -1,6 +1,7 @@
-// The 3x3x3 stencil of a query chunk, shared by the feature kernel
-// (grid.cu: features, closed-form radii, training targets) and the fused
-// feature + network radius kernel (mlp.cu).
+// The 3x3x3 stencil of a query chunk, a warp per chunk: features, closed-form
+// radii of float64 particles and training targets (grid.cu).  The radius
+// kernel of float32 particles (mlp.cu) looks the same cells up 32 chunks at a
+// time.
 #pragma once
 
 #include "hop_internal.cuh"

@@ -271,31 +271,6 @@ __device__ __forceinline__ uint32_t find_root(const uint32_t *parent, uint32_t x
     return x;
 }
 
-// Warp aggregation for per-group atomics: `peers` is the set of lanes that
-// hold the same group (__match_any_sync); every lane of the set gets the
-// sum or maximum of the set's values, combined in ascending lane order.
-__device__ __forceinline__ long long peer_sum_ll(uint32_t peers, long long v)
-{
-    long long s = 0;
-    for (uint32_t m = peers; m; m &= m - 1) s += __shfl_sync(peers, v, __ffs(m) - 1);
-    return s;
-}
-__device__ __forceinline__ double peer_sum_f64(uint32_t peers, double v)
-{
-    double s = 0.0;
-    for (uint32_t m = peers; m; m &= m - 1) s += __shfl_sync(peers, v, __ffs(m) - 1);
-    return s;
-}
-__device__ __forceinline__ unsigned long long peer_max(uint32_t peers, unsigned long long v)
-{
-    unsigned long long b = 0;
-    for (uint32_t m = peers; m; m &= m - 1) {
-        const unsigned long long u = __shfl_sync(peers, v, __ffs(m) - 1);
-        b = u > b ? u : b;
-    }
-    return b;
-}
-
 // Runs of consecutive lanes with the same group key g (each run reduced by
 // one atomic): heads has a bit for every lane that starts a run.
 __device__ __forceinline__ uint32_t run_heads(int64_t g, int lane)
@@ -409,7 +384,6 @@ constexpr int kBoxLevels = 12;
 struct BoxTree {
     const float4 *lo, *hi;
     uint32_t off[kBoxLevels];
-    int levels;
 };
 int box_tree_build(hop_ctx *c, const float4 *spos, int64_t n, BoxTree *t);
 

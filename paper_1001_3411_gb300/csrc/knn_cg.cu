@@ -2,8 +2,8 @@
 // step 1, Parallel HOP Sec. 2) for float32 positions: count-then-gather with
 // a whole warp on one query.  It serves the queries that the grouped kernel
 // (knn_gq.cu) hands over: a ball that wraps around the box (tiny boxes, a
-// very large radius), more cells than that kernel lists, a crowd of
-// particles at the Ndens-th distance.
+// very large radius), a box side whose squares leave float32's range, more
+// boxes than that kernel lists, a crowd of particles at the Ndens-th distance.
 //
 // For each query the warp lists the cells (side >= R / cpr, cpr <= 3) that
 // meet its ball, and the lanes read the cells' particles straight from the

@@ -1121,9 +1121,13 @@ template <bool SEG, bool F64> int knn_gq_run(hop_ctx *c, const KnnArgs &ka, int 
     if (rc) return rc;
     d.n = (uint32_t)ka.n;
     d.pad_run = (uint32_t)((ka.n + 7) / 8);
-    // a warp takes a whole unit, except where that would leave warps idle:
-    // then a half or a quarter of one (4,913 particles: 461 us whole, 371 us in
-    // quarters)
+    // a warp takes a whole unit, except where that leaves warps idle or a long
+    // last wave: then a half or a quarter of one.  kNN of NFW boxes in us,
+    // learned radius, whole / half / quarter: 4,913 particles 164 / 104 / 82;
+    // 32,768 238 / 176 / 154; 65,537 301 / 260 / 250; 131,071 391 / 373 / 354;
+    // 262,147 637 / 586 / 604; 524,287 1110 / 1137 / 1196; 2.1M 4048 / 4269 /
+    // 4677 (each part walks the unit's boxes again).  The lines, at 39,000 and
+    // 78,000 particles, lie lower than these times would put them.
     const int64_t units = SEG ? ka.n_units : (ka.n + kGqUnit - 1) / kGqUnit;
     const int64_t warps = (int64_t)c->num_sms * 16;
     d.split = units >= 2 * warps ? 1 : units >= warps ? 2 : 4;
