@@ -138,10 +138,12 @@ def source_hashes(files):
     return out
 
 
-def knn_traffic_per_particle():
+def knn_traffic_per_particle(tuning=None):
     """DRAM bytes per particle of the kNN kernel from the committed ncu
-    capture record, or None when any source file the kernel is compiled from
-    changed since that capture."""
+    capture record, or None when a source file of the kernel or of the boxes
+    it reads changed since that capture, or when `tuning` (queries per warp,
+    cells per radius, buffer factor) runs another kernel or other radii than
+    the capture did."""
     try:
         rec = json.load(open(TRAFFIC_RECORD))
         now = source_hashes(rec["sources"].keys())
@@ -149,6 +151,8 @@ def knn_traffic_per_particle():
         return None, "no capture"
     if now != rec["sources"]:
         return None, "kernel sources changed since the ncu capture"
+    if tuning is not None and knn_case(tuning) != knn_case(rec["tuning"]):
+        return None, "the ncu capture is of another tuning"
     return float(rec["traffic_bytes_per_particle"]), rec["basis"]
 
 
@@ -294,18 +298,26 @@ def knn_kernel_name(t):
     return "knn_gq_kernel (four queries per warp)"
 
 
+def knn_case(t):
+    """What of a tuning the kNN depends on: the cells per radius matter only to
+    the queries that the grouped kernel hands over."""
+    qpw, cpr, buf = t
+    return (qpw, 0, 0) if qpw in (4, 8, 16) and not buf else (qpw, cpr, buf)
+
+
 def stage(st):
     keys = ("ms_sort", "ms_radius", "ms_knn", "ms_link", "ms_boundaries", "ms_merge", "ms_total")
     return {k[3:]: round(statistics.median(s[k] for s in st), 3) for k in keys}
 
 
 # (queries per radius chunk, cells per radius, buffer factor): 4, 8 and 16 run
-# the grouped kernel (cells per radius matter only to the queries it hands
-# over), 32 one query per lane; a buffer factor selects the single-scan kernel
-# with that candidate buffer
-CANDS = {"learned": [(4, 2, 0), (4, 1, 0), (4, 3, 0), (8, 1, 0), (8, 2, 0), (16, 1, 0), (4, 1, 3), (32, 1, 3)],
-         "count": [(4, 2, 0), (4, 1, 0), (8, 1, 0), (16, 1, 0), (4, 1, 3), (32, 1, 3)],
-         "plain": [(4, 2, 0), (8, 2, 0), (32, 1, 0), (32, 1, 3)]}
+# the grouped kernel (once each: cells per radius matter only to the queries
+# it hands over, and the plain radius is the same for every chunk), 32 one
+# query per lane; a buffer factor selects the single-scan kernel with that
+# candidate buffer
+CANDS = {"learned": [(4, 2, 0), (8, 2, 0), (16, 1, 0), (4, 1, 3), (32, 1, 3)],
+         "count": [(4, 2, 0), (8, 2, 0), (16, 1, 0), (4, 1, 3), (32, 1, 3)],
+         "plain": [(4, 2, 0), (32, 1, 0), (32, 1, 3)]}
 
 
 def batch_section(hop, args, dist):
@@ -536,7 +548,7 @@ def run_gb300(args):
     fp32_peak = sms * 128 * 2 * sm_mhz * 1e6 / 1e12           # TFLOP/s at the sampled clock
     alg_flop = n * IDEAL_CANDIDATES * FLOP_PER_CANDIDATE
     achieved = alg_flop / (knn_ms * 1e-3) / 1e12
-    tpp, tsrc = knn_traffic_per_particle()
+    tpp, tsrc = knn_traffic_per_particle(tuned["learned"])
 
     line = {
         "metric": METRIC,
